@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libmpslcc.so")
 BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["mpo.cpp", "engine.cpp", "sweep.cpp", "capi.cpp", "kernels.cu", "tc_gemm.cu"]
+SOURCES = ["mpo.cpp", "engine.cpp", "sweep.cpp", "capi.cpp", "kernels.cu", "gemm_f64.cu", "tc_gemm.cu"]
 
 
 def _nvcc():

@@ -14,6 +14,16 @@ struct mpslcc_ctx {
 
 namespace {
 
+void reset_families(Ctx& c) {
+  for (Family* F : {&c.f00, &c.f11, &c.f10, &c.s10, &c.u11, &c.h11}) {
+    F->L.clear();
+    F->R.clear();
+    F->bra = F->ket = nullptr;
+  }
+  c.ofam.clear();
+  c.series_valid = false;
+}
+
 template <class F>
 mpslcc_status guard(mpslcc_ctx* ctx, F&& f) {
   if (!ctx) return MPSLCC_E_ARG;
@@ -24,6 +34,8 @@ mpslcc_status guard(mpslcc_ctx* ctx, F&& f) {
   } catch (const Error& e) {
     ctx->c.err = e.what();
     if (!ctx->c.host_only) cudaGetLastError();
+    // an expired wait may be found after the environments it spoiled were kept
+    if (e.status == ST_TIMEOUT) reset_families(ctx->c);
     return (mpslcc_status)e.status;
   } catch (const std::bad_alloc&) {
     ctx->c.err = "host allocation failed";
@@ -48,16 +60,6 @@ mpslcc_status noconv_status(mpslcc_ctx* ctx, mpslcc_status st) {
   ctx->c.err = std::to_string(ctx->c.cf.noconv) +
                " local solve(s) stopped at max_iter above their tolerance; the states and energies were kept";
   return MPSLCC_E_NOCONV;
-}
-
-void reset_families(Ctx& c) {
-  for (Family* F : {&c.f00, &c.f11, &c.f10, &c.s10, &c.u11, &c.h11}) {
-    F->L.clear();
-    F->R.clear();
-    F->bra = F->ket = nullptr;
-  }
-  c.ofam.clear();
-  c.series_valid = false;
 }
 
 void build_partition_mpos(Ctx& c) {
@@ -138,6 +140,11 @@ mpslcc_status mpslcc_create(mpslcc_ctx** out, const mpslcc_opts* opts) {
     }
     MPSLCC_REQUIRE(cusolverDnCreate(&c.solver) == CUSOLVER_STATUS_SUCCESS, ST_CUDA, "cusolverDnCreate failed");
     cusolverDnSetStream(c.solver, c.stream);
+    int* flag = nullptr;
+    cuda_check(cudaHostAlloc((void**)&flag, sizeof(int), cudaHostAllocMapped), "flag");
+    *flag = 0;
+    c.f64_flag = flag;
+    cuda_check(cudaHostGetDevicePointer((void**)&c.f64_flag_dev, flag, 0), "flag address");
     for (cudaEvent_t* e : {&c.ev0, &c.ev1, &c.ev_p0, &c.ev_p1, &c.ev_p2}) cuda_check(cudaEventCreate(e), "event");
   });
   if (st != MPSLCC_OK) {
@@ -172,6 +179,7 @@ mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
       if (c.eig_ev[s]) cudaEventDestroy(c.eig_ev[s]);
     }
     if (c.eig_fork) cudaEventDestroy(c.eig_fork);
+    if (c.f64_flag) cudaFreeHost((void*)c.f64_flag);
     if (c.solver) cusolverDnDestroy(c.solver);
     for (cudaEvent_t e : {c.ev0, c.ev1, c.ev_p0, c.ev_p1, c.ev_p2})
       if (e) cudaEventDestroy(e);

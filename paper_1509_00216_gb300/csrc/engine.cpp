@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstring>
 #include <ctime>
+#include <functional>
 
 namespace mpslcc {
 
@@ -157,15 +158,27 @@ void validate_copy(const Ctx& c, const CopyTask& t) {
 void run_gemms(Ctx& c, std::vector<GemmTask>& t) {
   if (t.empty()) return;
   for (const auto& x : t) validate_gemm(c, x);
-  long long tiles = plan_gemm_tiles(t.data(), (int)t.size());
-  if (tiles == 0) return;
-  size_t bytes = t.size() * sizeof(GemmTask);
-  c.gtask.ensure(&c, bytes);
-  cuda_check(cudaMemcpyAsync(c.gtask.p, t.data(), bytes, cudaMemcpyHostToDevice, c.s()), "upload gemm tasks");
-  launch_gemm_f64((const GemmTask*)c.gtask.p, (int)t.size(), tiles, c.s());
+  F64Plan p;
+  plan_f64(t.data(), (int)t.size(), p);
+  if (p.tiles_tc + p.tiles_small == 0) return;
+  c.gtask.ensure(&c, f64_plan_bytes(p));
+  upload_f64(p, c.gtask.p, c.s());
+  run_f64(c, p, c.gtask.p);
+}
+
+void run_f64(Ctx& c, const F64Launch& l, const void* d) {
+  const int sms = std::max(1, sm_count_dev(c.device) - std::max(0, c.tc_sm_reserve));
+  const int n = launch_f64(l, d, c.device, sms, c.f64_flag_dev, c.s());
   cuda_check(cudaGetLastError(), "gemm_f64 launch");
-  c.st.gemm_launches++;
-  c.st.kernel_launches++;
+  c.st.gemm_launches += n;
+  c.st.kernel_launches += n;
+}
+
+void check_f64(Ctx& c) {
+  const int h = c.f64_flag ? *c.f64_flag : 0;
+  if (!h) return;
+  *c.f64_flag = 0;
+  throw Error(ST_TIMEOUT, "FP64 product gave up waiting on an mbarrier (code " + std::to_string(h) + ")");
 }
 
 void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t) {
@@ -204,6 +217,7 @@ double dev_dot(Ctx& c, const double* x, const double* y, long n) {
   double r = 0;
   cuda_check(cudaMemcpyAsync(&r, c.red_out.p, sizeof(double), cudaMemcpyDeviceToHost, c.s()), "dot d2h");
   cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
+  check_f64(c);
   return r;
 }
 
@@ -217,6 +231,7 @@ void dev_dot2(Ctx& c, const double* x1, const double* y1, const double* x2, cons
   double r[2] = {0, 0};
   cuda_check(cudaMemcpyAsync(r, c.red_out.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "dot d2h");
   cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
+  check_f64(c);
   *r1 = r[0];
   *r2 = r[1];
 }
@@ -1050,7 +1065,7 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
   // atomics: results are reproducible bit for bit)
   struct U2 { int bi, so, d, boff, kv; std::vector<int> tab; };
   std::vector<U2> u2;
-  long long base_tiles = 0;
+  long long base_tiles = 0, work = 0;   // 64 x 64 tiles; K values times 128 x 64 tiles
   for (size_t bi = 0; bi < P.mid_b.size(); ++bi) {
     const int fb = lf.kb[bi], dFRb = rf.FRb.d[rf.kb[bi]];
     for (int so = 0; so < 4; ++so) {
@@ -1069,51 +1084,64 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
       U2 u{(int)bi, so, d, piece_off(lf.FLb, fb, so), 0, {}};
       u.kv = add_runs(rg, (int)lf.K[bi], u.tab);
       base_tiles += (long long)((d + 63) / 64) * ((dFRb + 63) / 64);
+      work += (long long)((d + 127) / 128) * ((dFRb + 63) / 64) * u.kv;
       u2.push_back(std::move(u));
     }
   }
-  const long long target = 152LL * 6;
   std::vector<SplitSeg> segs;
-  std::vector<int> ksv(u2.size(), 0);
+  std::vector<int> ksv;
   long poff = 0;
-  for (size_t i = 0; i < u2.size(); ++i) {
-    const U2& u = u2[i];
-    const int dFRb = rf.FRb.d[rf.kb[u.bi]];
-    SplitSeg sg;
-    std::memset(&sg, 0, sizeof(sg));
-    sg.out_off = P.off_b[u.bi] + (long long)u.boff * dFRb;
-    sg.m = u.d;
-    sg.n = dFRb;
-    sg.ldp = dFRb;
-    sg.sstride = (long long)u.d * dFRb;
-    if (u.kv > 0) {  // no run: no operator channel reaches these rows, they stay zero
-      int ks = 1;
-      if (base_tiles < target) {
-        long long f = (target + base_tiles - 1) / std::max(1LL, base_tiles);
-        ks = (int)std::max(1LL, std::min(f, (long long)(u.kv / 256)));
+  // phase-2 tasks with ks(kv) splits of a unit's kv summed indices
+  auto split = [&](const std::function<int(int)>& ks) {
+    segs.clear();
+    ksv.assign(u2.size(), 0);
+    t2.clear();
+    poff = 0;
+    for (size_t i = 0; i < u2.size(); ++i) {
+      const U2& u = u2[i];
+      const long K = lf.K[u.bi];
+      const int dFRb = rf.FRb.d[rf.kb[u.bi]];
+      SplitSeg sg;
+      std::memset(&sg, 0, sizeof(sg));
+      sg.out_off = P.off_b[u.bi] + (long long)u.boff * dFRb;
+      sg.m = u.d;
+      sg.n = dFRb;
+      sg.ldp = dFRb;
+      sg.sstride = (long long)u.d * dFRb;
+      if (u.kv > 0) {  // no run: no operator channel reaches these rows, they stay zero
+        ksv[i] = ks(u.kv);
+        sg.nsplit = ksv[i];
+        sg.part_off = poff;
+        poff += (long)ksv[i] * sg.sstride;
+        GemmTask t = gemm(lf.data.d() + lf.off[u.bi] + (long)u.boff * K, P.tt.d() + P.tt_off[u.bi], nullptr, u.d, dFRb,
+                          (int)K, (int)K, (int)K, dFRb, GEMM_TB);
+        t.ksplit = ksv[i];
+        t.sK = sg.sstride;
+        t.kv = u.kv;
+        t.nkr = (int)u.tab.size() / 2 - 1;
+        t.kr = u.tab.data();   // marks a run task; the device table's address follows below
+        t2.push_back(t);
       }
-      ksv[i] = ks;
-      sg.nsplit = ks;
-      sg.part_off = poff;
-      poff += (long)ks * sg.sstride;
+      segs.push_back(sg);
     }
-    segs.push_back(sg);
+  };
+  // On the FP64 pipe the splits fill the chip with 64 x 64 blocks of at least
+  // 256 K values each.  On the tensor cores a split takes four tiles' share per
+  // SM where the sum allows it, at least 128 K values (a drain of the
+  // accumulators per 128 is paid anyway).
+  const long long target = 152LL * 6;
+  const long long f = base_tiles < target ? (target + base_tiles - 1) / std::max(1LL, base_tiles) : 1;
+  split([&](int kv) { return (int)std::max(1LL, std::min(f, (long long)(kv / 256))); });
+  if (!f64_on_pipe(t2.data(), (int)t2.size())) {
+    const long long kper = std::max(128LL, (work + 4 * 152 - 1) / (4 * 152));
+    split([&](int kv) { return (int)((kv + kper - 1) / kper); });
   }
   P.ypart.release();
   P.ypart.alloc(&c, std::max(poff, 1L) * sizeof(double));
-  for (size_t i = 0; i < u2.size(); ++i) {
+  for (size_t i = 0, j = 0; i < u2.size(); ++i) {
     if (ksv[i] == 0) continue;
-    U2& u = u2[i];
-    const long K = lf.K[u.bi];
-    const int dFRb = rf.FRb.d[rf.kb[u.bi]];
-    GemmTask t = gemm(lf.data.d() + lf.off[u.bi] + (long)u.boff * K, P.tt.d() + P.tt_off[u.bi],
-                      P.ypart.d() + segs[i].part_off, u.d, dFRb, (int)K, (int)K, (int)K, dFRb, GEMM_TB);
-    t.ksplit = ksv[i];
-    t.sK = segs[i].sstride;
-    t.kv = u.kv;
-    t.nkr = (int)u.tab.size() / 2 - 1;
-    rt2.push_back(std::move(u.tab));
-    t2.push_back(t);
+    t2[j++].C = P.ypart.d() + segs[i].part_off;
+    rt2.push_back(std::move(u2[i].tab));
   }
   // run tables of both phases in one device buffer
   std::vector<int> tab;
@@ -1139,20 +1167,17 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
   for (const auto& x : t1) validate_gemm(c, x);
   for (const auto& x : t2) validate_gemm(c, x);
   P.flops = fl;
-  P.n1 = (int)t1.size();
-  P.n2 = (int)t2.size();
-  P.tiles1 = t1.empty() ? 0 : plan_gemm_tiles(t1.data(), P.n1);
-  P.tiles2 = t2.empty() ? 0 : plan_gemm_tiles(t2.data(), P.n2);
+  F64Plan p1, p2;
+  plan_f64(t1.data(), (int)t1.size(), p1);
+  plan_f64(t2.data(), (int)t2.size(), p2);
+  P.l1 = p1;
+  P.l2 = p2;
   P.tasks1.release();
   P.tasks2.release();
-  P.tasks1.alloc(&c, std::max<size_t>(t1.size(), 1) * sizeof(GemmTask));
-  P.tasks2.alloc(&c, std::max<size_t>(t2.size(), 1) * sizeof(GemmTask));
-  if (!t1.empty())
-    cuda_check(cudaMemcpyAsync(P.tasks1.p, t1.data(), t1.size() * sizeof(GemmTask), cudaMemcpyHostToDevice, c.s()),
-               "upload sigma tasks");
-  if (!t2.empty())
-    cuda_check(cudaMemcpyAsync(P.tasks2.p, t2.data(), t2.size() * sizeof(GemmTask), cudaMemcpyHostToDevice, c.s()),
-               "upload sigma tasks");
+  P.tasks1.alloc(&c, std::max<size_t>(f64_plan_bytes(p1), 16));
+  P.tasks2.alloc(&c, std::max<size_t>(f64_plan_bytes(p2), 16));
+  upload_f64(p1, P.tasks1.p, c.s());
+  upload_f64(p2, P.tasks2.p, c.s());
   cuda_check(cudaStreamSynchronize(c.s()), "sigma plan sync");
 }
 
@@ -1164,17 +1189,17 @@ void sigma_apply(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
   if (P.nk > 0)
     cuda_check(cudaMemcpyAsync(P.xin.p, x, P.nk * sizeof(double), cudaMemcpyDeviceToDevice, c.s()), "sigma in");
   cudaEventRecord(c.ev_p0, c.s());
-  launch_gemm_f64((const GemmTask*)P.tasks1.p, P.n1, P.tiles1, c.s());
+  run_f64(c, P.l1, P.tasks1.p);
   cudaEventRecord(c.ev_p1, c.s());
-  launch_gemm_f64((const GemmTask*)P.tasks2.p, P.n2, P.tiles2, c.s());
+  run_f64(c, P.l2, P.tasks2.p);
   cudaEventRecord(c.ev_p2, c.s());
   launch_splitk_reduce_f64((const SplitSeg*)P.segs.p, P.nseg, P.seg_tiles, P.ypart.d(), y, c.s());
   cuda_check(cudaGetLastError(), "sigma launch");
-  c.st.kernel_launches += 3;
-  c.st.gemm_launches += 2;
+  c.st.kernel_launches++;
   c.st.sigma_calls++;
   c.st.sigma_flops += P.flops;
   cuda_check(cudaEventSynchronize(c.ev_p2), "sigma phase sync");
+  check_f64(c);
   float m1 = 0, m2 = 0;
   cudaEventElapsedTime(&m1, c.ev_p0, c.ev_p1);
   cudaEventElapsedTime(&m2, c.ev_p1, c.ev_p2);

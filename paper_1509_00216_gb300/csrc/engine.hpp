@@ -177,8 +177,7 @@ struct SigmaPlan {
   DBuf tt;
   DBuf xin;
   DBuf tasks1, tasks2;
-  int n1 = 0, n2 = 0;
-  long long tiles1 = 0, tiles2 = 0;
+  F64Launch l1, l2;
   // FP64 phase 2: per-split partial products and the segments of their
   // fixed-order sum into sigma
   DBuf ypart, segs;
@@ -247,6 +246,10 @@ struct Ctx {
   mpslcc_opts opts{};
   std::string err;
   cusolverDnHandle_t solver = nullptr;
+  // set (to a code) by an FP64 tensor-core product whose wait ran out; pinned
+  // host memory that the device writes, so that reading it costs no copy
+  volatile int* f64_flag = nullptr;
+  int* f64_flag_dev = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_p0 = nullptr, ev_p1 = nullptr, ev_p2 = nullptr;
 
   // problem
@@ -347,6 +350,10 @@ struct Ctx {
 void upload_boxes(Ctx& c, int which);
 void run_gemms(Ctx& c, std::vector<GemmTask>& t);
 void run_gemms_tc(Ctx& c, std::vector<GemmTask>& t);
+void run_f64(Ctx& c, const F64Launch& l, const void* d);
+// Throws ST_TIMEOUT if an FP64 product of the (synchronised) stream gave up.
+void check_f64(Ctx& c);
+int sm_count_dev(int device);
 // FP64 DFMA kernel or split-BF16 tensor cores, by c.gemm_prec
 void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t);
 void validate_gemm(const Ctx& c, const GemmTask& t);

@@ -1,7 +1,5 @@
-// FP64 device kernels: grouped batched GEMM over per-task descriptors (every
-// per-sector contraction of the sigma vector, environment fusion and
-// environment renormalisation is one task), strided window copies, and the
-// BLAS-1 / reduction kernels of the iterative solvers.
+// FP64 device kernels: strided window copies and the BLAS-1 / reduction
+// kernels of the iterative solvers.
 #include "kernels.hpp"
 
 #include <cuda_bf16.h>
@@ -10,7 +8,6 @@
 namespace mpslcc {
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16, GT = 256;
 constexpr int COPY_CHUNK = 2048;
 
 template <class T>
@@ -22,120 +19,6 @@ __device__ __forceinline__ int find_task(const T* t, int n, long long tile) {
     else hi = mid - 1;
   }
   return lo;
-}
-
-__global__ void __launch_bounds__(GT) gemm_f64_kernel(const GemmTask* __restrict__ tasks, int ntasks,
-                                                      long long total) {
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (long long tile = blockIdx.x; tile < total; tile += gridDim.x) {
-    const GemmTask T = tasks[find_task(tasks, ntasks, tile)];
-    long long local = tile - T.tile0;
-    const int tiles_mn = T.tm * T.tn;
-    const long long per_batch = (long long)T.ksplit * tiles_mn;
-    const int b = (int)(local / per_batch);
-    int r = (int)(local - (long long)b * per_batch);
-    const int ks = r / tiles_mn;
-    r -= ks * tiles_mn;
-    const int tm = r / T.tn, tn = r - (r / T.tn) * T.tn;
-    const double* A = T.A + (long long)b * T.sA;
-    const double* B = T.B + (long long)b * T.sB;
-    double* C = T.C + (long long)b * T.sC;
-    const bool ta = T.flags & GEMM_TA, tb = T.flags & GEMM_TB;
-    const int kv = T.kr ? T.kv : T.k;   // summed K length
-    int kchunk = (kv + T.ksplit - 1) / T.ksplit;
-    kchunk = ((kchunk + BK - 1) / BK) * BK;
-    const int k0 = ks * kchunk;
-    const int k1 = min(kv, k0 + kchunk);
-    const int row0 = tm * BM, col0 = tn * BN;
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    // the operand column spans [ps, pe) to sum over: [k0, k1) itself, or the
-    // parts of the K runs that overlap virtual [k0, k1) (the first found by
-    // binary search)
-    int run = 0;
-    if (T.kr) {
-      int lo = 0, hi = T.nkr - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (T.kr[2 * mid + 1] <= k0) lo = mid;
-        else hi = mid - 1;
-      }
-      run = lo;
-    }
-    for (bool first = true;; first = false) {
-      int ps, pe;
-      if (!T.kr) {
-        if (!first) break;
-        ps = k0;
-        pe = k1;
-      } else {
-        if (run >= T.nkr) break;
-        const int v0 = T.kr[2 * run + 1], v1 = T.kr[2 * run + 3];
-        if (v0 >= k1) break;
-        const int vb = max(v0, k0), ve = min(v1, k1);
-        ps = T.kr[2 * run] + (vb - v0);
-        pe = T.kr[2 * run] + (ve - v0);
-        ++run;
-      }
-      for (int kk = ps; kk < pe; kk += BK) {
-        for (int e = threadIdx.x; e < BM * BK; e += GT) {
-          int i, q;
-          if (!ta) { i = e / BK; q = e - i * BK; }
-          else { q = e / BM; i = e - q * BM; }
-          const int gi = row0 + i, gk = kk + q;
-          double v = 0.0;
-          if (gi < T.m && gk < pe) v = ta ? A[(long long)gk * T.lda + gi] : A[(long long)gi * T.lda + gk];
-          As[q][i] = v;
-        }
-        for (int e = threadIdx.x; e < BN * BK; e += GT) {
-          int j, q;
-          if (!tb) { q = e / BN; j = e - q * BN; }
-          else { j = e / BK; q = e - j * BK; }
-          const int gj = col0 + j, gk = kk + q;
-          double v = 0.0;
-          if (gj < T.n && gk < pe) v = tb ? B[(long long)gj * T.ldb + gk] : B[(long long)gk * T.ldb + gj];
-          Bs[q][j] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < BK; ++q) {
-          double a[4], bv[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[i] = As[q][ty + 16 * i];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) bv[j] = Bs[q][tx + 16 * j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int gi = row0 + ty + 16 * i;
-      if (gi >= T.m) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int gj = col0 + tx + 16 * j;
-        if (gj >= T.n) continue;
-        const double v = T.alpha * acc[i][j];
-        if (T.ksplit > 1 && T.sK > 0) {
-          C[(long long)ks * T.sK + (long long)gi * T.ldc + gj] = v;  // partial of split ks
-        } else {
-          double* c = C + (long long)gi * T.ldc + gj;
-          if (T.ksplit > 1) atomicAdd(c, v);
-          else *c = (T.beta != 0.0) ? v + T.beta * (*c) : v;
-        }
-      }
-    }
-  }
 }
 
 __global__ void copy_f64_kernel(const CopyTask* __restrict__ tasks, int ntasks, long long total) {
@@ -341,19 +224,6 @@ inline int elem_grid(long n) {
 }
 }  // namespace
 
-long long plan_gemm_tiles(GemmTask* t, int n) {
-  long long tot = 0;
-  for (int i = 0; i < n; ++i) {
-    t[i].tm = (t[i].m + BM - 1) / BM;
-    t[i].tn = (t[i].n + BN - 1) / BN;
-    if (t[i].ksplit < 1) t[i].ksplit = 1;
-    t[i].tile0 = tot;
-    if (t[i].m <= 0 || t[i].n <= 0) t[i].tm = t[i].tn = 0;
-    tot += (long long)t[i].batch * t[i].ksplit * t[i].tm * t[i].tn;
-  }
-  return tot;
-}
-
 long long plan_split_tiles(SplitSeg* s, int n) {
   long long tot = 0;
   for (int i = 0; i < n; ++i) {
@@ -385,12 +255,6 @@ long long plan_copy_tiles(CopyTask* t, int n) {
     tot += (long long)t[i].batch * ((nel + COPY_CHUNK - 1) / COPY_CHUNK);
   }
   return tot;
-}
-
-void launch_gemm_f64(const GemmTask* d_tasks, int ntasks, long long total, cudaStream_t s) {
-  if (total <= 0 || ntasks <= 0) return;
-  int grid = (int)std::min<long long>(total, 152LL * 8);
-  gemm_f64_kernel<<<grid, GT, 0, s>>>(d_tasks, ntasks, total);
 }
 
 void launch_copy_f64(const CopyTask* d_tasks, int ntasks, long long total, cudaStream_t s) {

@@ -2,17 +2,17 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <vector>
 
 namespace mpslcc {
 
 // One GEMM of a grouped launch: C = alpha * op(A) op(B) + beta * C for
 // `batch` problems at constant strides.  op(A) is m x k (A row-major m x k,
 // or k x m when transposed); op(B) is k x n (B row-major k x n, or n x k when
-// transposed).  With ksplit > 1 the K range is split across CTAs: with sK > 0
-// split j stores its partial product alpha * op(A) op(B)|_K-chunk j at C + j sK
-// (beta ignored; the partials are summed afterwards in a fixed order by
-// launch_splitk_reduce, so results do not depend on scheduling); with sK = 0
-// the partials are added to C atomically (C pre-scaled by the caller).
+// transposed).  With ksplit > 1 the K range is split across CTAs: split j
+// stores its partial product alpha * op(A) op(B)|_K-chunk j at C + j sK (beta
+// ignored; the partials are summed afterwards in a fixed order by
+// launch_splitk_reduce, so results do not depend on scheduling).
 struct GemmTask {
   const double* A;
   const double* B;
@@ -24,9 +24,7 @@ struct GemmTask {
   double alpha, beta;
   int flags;      // GEMM_TA | GEMM_TB
   int ksplit;
-  int tm, tn;     // tile counts (filled by plan_gemm_tiles)
-  long long tile0;
-  long long sK;   // element stride between split-K partials (0 = atomic adds)
+  long long sK;   // element stride between split-K partials
   // K runs (optional): the product sums over kv virtual K indices, run r
   // covering virtual [kr[2r+1], kr[2r+3]) at operand columns (rows, for a
   // transposed operand) from kr[2r]; nkr runs and a sentinel {0, kv}.  k is
@@ -48,11 +46,43 @@ struct CopyTask {
   long long tile0;
 };
 
+// A GEMM task as the FP64 kernels take it (gemm_f64.cu): C(i, j) = alpha
+// sum_k X(i, k) Y(j, k) (+ beta C(i, j)).  Row i of X is (entry i / nx, row
+// i % nx) of a folded batch, at x + entry xbs + row xrs, its K index at stride
+// xks; Y and both directions of C likewise.  Batches that fold into neither
+// operand advance by xub, yub, cub.
+struct F64Task {
+  const double *x, *y;
+  double* c;
+  long long xrs, xks, xbs, yrs, yks, ybs, cxs, cxb, cys, cyb, xub, yub, cub, sK;
+  double alpha, beta;
+  int nx, mx, ny, my, k, ksplit, kchunk, batch;
+  const int* kr;
+  int nkr, tx, ty;
+  long long tile0;
+};
+
+// Task lists of one launch pair: tensor-core tasks first, then the small
+// ones that run on the FP64 pipe.
+struct F64Launch {
+  int n_tc = 0, n_small = 0;
+  long long tiles_tc = 0, tiles_small = 0;
+};
+struct F64Plan : F64Launch {
+  std::vector<F64Task> tc, small;
+};
+// Whether a launch of these tasks is so short that it runs on the FP64 pipe whole.
+bool f64_on_pipe(const GemmTask* g, int n);
+void plan_f64(const GemmTask* g, int n, F64Plan& p);
+size_t f64_plan_bytes(const F64Plan& p);
+void upload_f64(const F64Plan& p, void* d, cudaStream_t s);
+// Runs the lists uploaded at d; returns the number of launches.  The
+// tensor-core kernel takes at most `sms` SMs and records an expired wait in *err.
+int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s);
+
 // Fill tile bookkeeping; returns total number of tiles.
-long long plan_gemm_tiles(GemmTask* t, int n);
 long long plan_copy_tiles(CopyTask* t, int n);
 
-void launch_gemm_f64(const GemmTask* d_tasks, int ntasks, long long total_tiles, cudaStream_t s);
 void launch_copy_f64(const CopyTask* d_tasks, int ntasks, long long total_tiles, cudaStream_t s);
 
 // BLAS-1 on FP64 device vectors.  Reductions write into a device scalar.
