@@ -86,11 +86,19 @@ __device__ __forceinline__ int k_col(const F64Task& T, int v) {
   return __ldg(T.kr + 2 * lo) + (v - __ldg(T.kr + 2 * lo + 1));
 }
 
-// Output element of tile row i and column j (offsets already resolved).
-__device__ __forceinline__ void put(const F64Task& T, double* c, double v, bool first) {
-  if (T.alpha != 1.0) v *= T.alpha;
-  if (!first) v += *c;
-  else if (T.beta != 0.0) v += T.beta * (*c);
+// How a tile is written: C = alpha v + beta C.  The cases that need the FP64
+// pipe are told apart once per tile (a comparison of doubles runs there too,
+// and two per element took 20 % of the tensor-core kernel's time).
+enum { PUT_SCALE = 1, PUT_BETA = 2, PUT_ADD = 4 };
+__device__ __forceinline__ int put_mode(const F64Task& T, bool first) {
+  return (T.alpha != 1.0 ? PUT_SCALE : 0) | (!first ? PUT_ADD : (T.beta != 0.0 ? PUT_BETA : 0));
+}
+__device__ __forceinline__ void put(const F64Task& T, int mode, double* c, double v) {
+  if (mode) {
+    if (mode & PUT_SCALE) v *= T.alpha;
+    if (mode & PUT_ADD) v += *c;
+    else if (mode & PUT_BETA) v += T.beta * (*c);
+  }
   *c = v;
 }
 
@@ -382,22 +390,22 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       __syncthreads();
       // write-out along the direction that is contiguous in memory
-      const bool first = kb == k0;
+      const int pm = put_mode(T, kb == k0);
       if (T.cys == 1) {
         const bool o0 = lane < ny, o1 = lane + 32 < ny;
         const long long c0 = o0 ? row_off(y0 + lane, T.ny, 1, T.cyb) : 0;
         const long long c1 = o1 ? row_off(y0 + lane + 32, T.ny, 1, T.cyb) : 0;
         for (int i = warp; i < nx; i += THREADS / 32) {
           double* r = C + row_off(x0 + i, T.nx, T.cxs, T.cxb);
-          if (o0) put(T, r + c0, stg[i * STG_LD + lane], first);
-          if (o1) put(T, r + c1, stg[i * STG_LD + lane + 32], first);
+          if (o0) put(T, pm, r + c0, stg[i * STG_LD + lane]);
+          if (o1) put(T, pm, r + c1, stg[i * STG_LD + lane + 32]);
         }
       } else {
         for (int i0 = 0; i0 < nx; i0 += 32) {
           const int i = i0 + lane;
           const long long ci = i < nx ? row_off(x0 + i, T.nx, T.cxs, T.cxb) : 0;
           for (int j = warp; j < ny; j += THREADS / 32)
-            if (i < nx) put(T, C + ci + row_off(y0 + j, T.ny, T.cys, T.cyb), stg[i * STG_LD + j], first);
+            if (i < nx) put(T, pm, C + ci + row_off(y0 + j, T.ny, T.cys, T.cyb), stg[i * STG_LD + j]);
         }
       }
       __syncthreads();
@@ -476,10 +484,11 @@ __global__ void __launch_bounds__(256) gemm_f64_small_kernel(const F64Task* __re
       }
       __syncthreads();
     }
+    const int pm = put_mode(T, true);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (oi[u] >= 0)
-        put(T, C + row_off(x0 + oi[u], T.nx, T.cxs, T.cxb) + row_off(y0 + oj[u], T.ny, T.cys, T.cyb), acc[u], true);
+        put(T, pm, C + row_off(x0 + oi[u], T.nx, T.cxs, T.cxb) + row_off(y0 + oj[u], T.ny, T.cys, T.cyb), acc[u]);
   }
 }
 
