@@ -730,51 +730,117 @@ struct ConvTask {
                         // two-piece split on both sides
   long long soff;
   int trans;            // read the source transposed: dst(r, c) = src[c * src_ld + r]
+  int pad;              // columns up to the next multiple of 8 belong to the row: write zeros there
+  int vec;              // (filled by plan_conv) rows in 16-byte groups of 8 columns
   long long tile0;
 };
-constexpr int CONV_CHUNK = 4096;
+// Items of one 256-thread tile: groups of 8 columns, one a thread, or single
+// elements, four a thread.
+constexpr int CONV_T = 256, CONV_E = 4;
 
-// One converted element at output offset o (in the task's pattern).
+// The BF16 pieces of v: h = v rounded to FP32 and then to BF16, m the same of
+// v - h, l of v - h - m (two roundings each, differences exact).
+struct Pieces { uint16_t h, m, l; };
+
+__device__ __forceinline__ Pieces pieces_f64(double v) {
+  const __nv_bfloat16 h = __float2bfloat16_rn((float)v);
+  const double r1 = v - (double)__bfloat162float(h);
+  const __nv_bfloat16 m = __float2bfloat16_rn((float)r1);
+  const __nv_bfloat16 l = __float2bfloat16_rn((float)(r1 - (double)__bfloat162float(m)));
+  return {__bfloat16_as_ushort(h), __bfloat16_as_ushort(m), __bfloat16_as_ushort(l)};
+}
+
+__device__ __forceinline__ uint32_t bf16_bits(uint32_t f) { return (f + 0x7fffu + ((f >> 16) & 1u)) >> 16; }
+
+// fl32(d + b + c) with one rounding, for b a multiple of some unit u, d one of
+// u or coarser and 0 <= c < u: TwoSum gives d + b = s + t exactly, and t + c
+// is exact too (at most 20 bits here).
+__device__ __forceinline__ float add3(float d, float b, float c) {
+  const float s = __fadd_rn(d, b);
+  const float bb = __fadd_rn(s, -d);
+  const float t = __fadd_rn(__fadd_rn(d, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb));
+  return __fadd_rn(s, __fadd_rn(t, c));
+}
+
+// The same pieces without the FP64 pipe (its conversions and subtractions, at
+// two a clock and SM, took longer than the kernel's memory traffic): |v| is cut
+// at bit level into a + b + c of 24, 23 and 6 bits, and every rounding is one
+// of exact FP32 sums.  Values below 2^-63 are scaled by 2^128 on the way.  The
+// FP64 form is left to what would round in the subnormal range, to |v| from
+// 2^118 on and to v - h between 0 and 2^-30 |v| (one value in 2^21).
+__device__ __forceinline__ Pieces split_pieces(double v, bool three) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  uint32_t e = (hi >> 20) & 0x7ffu;
+  const uint32_t sg = (hi >> 16) & 0x8000u;
+  if (e < 888u) return {(uint16_t)sg, 0, 0};   // below half the smallest subnormal
+  uint32_t down = 0;
+  if (e < 960u) {
+    down = 128u << 7;
+    e += 128u;
+  }
+  if (e - 960u > 180u) return pieces_f64(v);
+  const uint32_t ef = (e - 896u) << 23;   // FP32 exponent of |v|
+  const float a = __uint_as_float(ef | __funnelshift_l(lo, hi & 0xfffffu, 3));
+  const uint32_t ub = ef - (23u << 23), uc = ef - (46u << 23);
+  const float b = __fadd_rn(__uint_as_float(ub | ((lo >> 6) & 0x7fffffu)), -__uint_as_float(ub));
+  const float c = __fadd_rn(__uint_as_float(uc | ((lo & 63u) << 17)), -__uint_as_float(uc));
+  // only which side of half an ulp of a the rest lies on decides, so c's bits
+  // go into the lowest bit of b
+  const float bs = __fadd_rn(__uint_as_float(ub | ((lo >> 6) & 0x7fffffu) | ((lo & 63u) ? 1u : 0u)), -__uint_as_float(ub));
+  const float f = __fadd_rn(a, bs);
+  uint32_t h = bf16_bits(__float_as_uint(f));
+  const float d = __fadd_rn(a, -__uint_as_float(h << 16));
+  const float r1 = add3(d, b, c);
+  uint32_t m = 0, l = 0;
+  if (r1 != 0.0f) {
+    if (fabsf(r1) < __uint_as_float(ef - (30u << 23))) return pieces_f64(v);
+    m = bf16_bits(__float_as_uint(r1));
+    if (three) l = bf16_bits(__float_as_uint(add3(__fadd_rn(d, -__uint_as_float(m << 16)), b, c)));
+  }
+  if (down) {
+    const uint32_t low = down | 0x80u;   // the smallest normal after scaling back
+    if (h < low || ((m & 0x7fffu) && (m & 0x7fffu) < low) || ((l & 0x7fffu) && (l & 0x7fffu) < low)) return pieces_f64(v);
+    h -= down;
+    if (m & 0x7fffu) m -= down;
+    if (l & 0x7fffu) l -= down;
+  }
+  return {(uint16_t)(h ^ sg), (uint16_t)(m & 0x7fffu ? m ^ sg : 0u), (uint16_t)(l & 0x7fffu ? l ^ sg : 0u)};
+}
+
+// Block j of a row in the task's pattern: which piece it holds.
+__device__ __forceinline__ int piece_of(int pattern, int j) {
+  if (pattern == 1) return j;                       // [h m]
+  constexpr uint32_t A = 0x201100, B = 0x020110;    // [h h m m h l], [h m m h l h], one digit a block
+  return (int)(((pattern == 2 ? A : B) >> (4 * j)) & 3u);
+}
+__host__ __device__ __forceinline__ int blocks_of(int pattern) { return pattern == 0 ? 1 : (pattern == 1 ? 2 : 6); }
+
+// One converted element at output offset o.
 template <int PREC>
 __device__ __forceinline__ void conv_put(const ConvTask& T, long long o, double v) {
   if (PREC == MPSLCC_TF32) {
     ((float*)T.dst)[o] = (float)v;
     return;
   }
-  __nv_bfloat16* d = (__nv_bfloat16*)T.dst + o;
-  const __nv_bfloat16 h = __float2bfloat16_rn((float)v);
-  if (T.pattern == 0) {
-    d[0] = h;
-    return;
-  }
-  const double r1 = v - (double)__bfloat162float(h);
-  const __nv_bfloat16 m = __float2bfloat16_rn((float)r1);
-  const long long so = T.soff;
-  if (T.pattern == 1) {
-    d[0] = h;
-    d[so] = m;   // lo of the two-piece split: the rounded remainder
-    return;
-  }
-  const __nv_bfloat16 l = __float2bfloat16_rn((float)(r1 - (double)__bfloat162float(m)));
-  if (T.pattern == 2) {   // A side [h h m m h l]
-    d[0] = h;
-    d[so] = h;
-    d[2 * so] = m;
-    d[3 * so] = m;
-    d[4 * so] = h;
-    d[5 * so] = l;
-  } else {                // B side [h m m h l h]
-    d[0] = h;
-    d[so] = m;
-    d[2 * so] = m;
-    d[3 * so] = h;
-    d[4 * so] = l;
-    d[5 * so] = h;
+  uint16_t* d = (uint16_t*)T.dst + o;
+  const Pieces p = split_pieces(v, T.pattern >= 2);
+  const int nb = blocks_of(T.pattern);
+  for (int j = 0; j < nb; ++j) {
+    const int k = piece_of(T.pattern, j);
+    d[j * T.soff] = k == 0 ? p.h : (k == 1 ? p.m : p.l);
   }
 }
 
+// Window conversion.  Bound by its traffic (8 bytes read, 2 to 12 written per
+// element).  A thread takes 8 consecutive columns where the output allows
+// 16-byte stores (every copy but the R' stacks' inner pieces): a transposed
+// source is then read along its rows by consecutive threads and still written
+// in 16-byte groups.  Items run over (batch entry, row, group) without gaps,
+// so that small windows fill their blocks.  Before, one element a thread at a
+// time, 16 in sequence, with 2-byte stores and FP64-pipe arithmetic: 7.9 ms
+// for the operators of the M1 = 1500 position, now 3.0 ms.
 template <int PREC>
-__global__ void conv_kernel(const ConvTask* __restrict__ t, int ntasks, long long total) {
+__global__ void __launch_bounds__(CONV_T) conv_kernel(const ConvTask* __restrict__ t, int ntasks, long long total) {
   for (long long tile = blockIdx.x; tile < total; tile += gridDim.x) {
     int lo = 0, hi = ntasks - 1;
     while (lo < hi) {
@@ -784,47 +850,69 @@ __global__ void conv_kernel(const ConvTask* __restrict__ t, int ntasks, long lon
     }
     const ConvTask T = t[lo];
     const long long local = tile - T.tile0;
-    const long long nel = (long long)T.rows * T.cols;
-    const long long per = (nel + CONV_CHUNK - 1) / CONV_CHUNK;
-    const int b = (int)(local / per);
-    const long long ch = local - (long long)b * per;
-    const long long e1 = min(nel, (ch + 1) * CONV_CHUNK);
-    const double* src = T.src + (long long)b * T.s_src;
-    const long long dbase = (long long)b * T.s_dst;
-    if (nel < (1LL << 31)) {
-      // 32-bit index arithmetic (a 64-bit division per element dominated
-      // this instruction-bound loop)
-      const int rows = T.rows, cols = T.cols;
-      const int e1i = (int)e1;
-      for (int e = (int)(ch * CONV_CHUNK) + (int)threadIdx.x; e < e1i; e += (int)blockDim.x) {
-        int rr, cc;
-        double v;
-        if (T.trans) {  // consecutive threads walk the source row (coalesced reads)
-          cc = e / rows;
-          rr = e - cc * rows;
-          v = src[(long long)cc * T.src_ld + rr];
-        } else {
-          rr = e / cols;
-          cc = e - rr * cols;
-          v = src[(long long)rr * T.src_ld + cc];
-        }
-        conv_put<PREC>(T, dbase + (long long)rr * T.dst_ld + cc, v);
+    if (!T.vec) {
+      const long long per = (long long)T.rows * T.cols;
+#pragma unroll
+      for (int u = 0; u < CONV_E; ++u) {
+        const long long e = (local * CONV_E + u) * CONV_T + threadIdx.x;
+        const long long b = e / per;
+        if (b >= T.batch) break;
+        const unsigned q = (unsigned)(e - b * per);   // a window holds fewer than 2^31 elements
+        unsigned rr, cc;
+        if (T.trans) { cc = q / (unsigned)T.rows; rr = q - cc * T.rows; }
+        else { rr = q / (unsigned)T.cols; cc = q - rr * T.cols; }
+        const double* src = T.src + b * T.s_src;
+        const double v = T.trans ? src[(long long)cc * T.src_ld + rr] : src[(long long)rr * T.src_ld + cc];
+        conv_put<PREC>(T, b * T.s_dst + (long long)rr * T.dst_ld + cc, v);
       }
-    } else {
-      for (long long e = ch * CONV_CHUNK + threadIdx.x; e < e1; e += blockDim.x) {
-        int rr, cc;
-        double v;
-        if (T.trans) {
-          cc = (int)(e / T.rows);
-          rr = (int)(e - (long long)cc * T.rows);
-          v = src[(long long)cc * T.src_ld + rr];
-        } else {
-          rr = (int)(e / T.cols);
-          cc = (int)(e - (long long)rr * T.cols);
-          v = src[(long long)rr * T.src_ld + cc];
-        }
-        conv_put<PREC>(T, dbase + (long long)rr * T.dst_ld + cc, v);
-      }
+      continue;
+    }
+    const unsigned ng = (unsigned)(T.cols + 7) >> 3, per = ng * (unsigned)T.rows;
+    const long long item = local * CONV_T + threadIdx.x;
+    const long long b = item / per;
+    if (b >= T.batch) continue;
+    const unsigned q = (unsigned)(item - b * per);
+    unsigned rr, g;
+    if (T.trans) { g = q / (unsigned)T.rows; rr = q - g * T.rows; }
+    else { rr = q / ng; g = q - rr * ng; }
+    const int c0 = 8 * (int)g, nv = min(8, T.cols - c0);
+    const double* src = T.src + b * T.s_src +
+                        (T.trans ? (long long)c0 * T.src_ld + rr : (long long)rr * T.src_ld + c0);
+    const long long st = T.trans ? T.src_ld : 1;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = j < nv ? __ldg(src + j * st) : 0.0;
+    const long long o = b * T.s_dst + (long long)rr * T.dst_ld + c0;
+    if (nv < 8 && !T.pad) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < nv) conv_put<PREC>(T, o + j, v[j]);
+      continue;
+    }
+    if (PREC == MPSLCC_TF32) {
+      float4* d = reinterpret_cast<float4*>((float*)T.dst + o);
+      d[0] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+      d[1] = make_float4((float)v[4], (float)v[5], (float)v[6], (float)v[7]);
+      continue;
+    }
+    uint32_t w[3][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const Pieces x = split_pieces(v[2 * j], T.pattern >= 2), y = split_pieces(v[2 * j + 1], T.pattern >= 2);
+      w[0][j] = x.h | (uint32_t)y.h << 16;
+      w[1][j] = x.m | (uint32_t)y.m << 16;
+      w[2][j] = x.l | (uint32_t)y.l << 16;
+    }
+    uint16_t* d = (uint16_t*)T.dst + o;
+    const int nb = blocks_of(T.pattern);
+    for (int j = 0; j < nb; ++j) {
+      const int k = piece_of(T.pattern, j);
+      uint4 x;
+      x.x = k == 0 ? w[0][0] : (k == 1 ? w[1][0] : w[2][0]);
+      x.y = k == 0 ? w[0][1] : (k == 1 ? w[1][1] : w[2][1]);
+      x.z = k == 0 ? w[0][2] : (k == 1 ? w[1][2] : w[2][2]);
+      x.w = k == 0 ? w[0][3] : (k == 1 ? w[1][3] : w[2][3]);
+      *reinterpret_cast<uint4*>(d + j * T.soff) = x;
     }
   }
 }
@@ -1061,9 +1149,33 @@ void launch_tc(Ctx& c, int prec, const TcTask* d_tasks, int ntasks, long long to
   c.st.gemm_launches++;
 }
 
+// Tiles of a conversion list; tasks whose rows, pieces and batch entries all
+// start on 16-byte boundaries are written in groups of 8 columns.
+long long plan_conv(ConvTask* t, int n) {
+  long long tot = 0;
+  for (int i = 0; i < n; ++i) {
+    ConvTask& x = t[i];
+    const bool blocks = blocks_of(x.pattern) > 1;
+    x.vec = ((uintptr_t)x.dst & 15) == 0 && x.dst_ld % 8 == 0 && (x.batch == 1 || x.s_dst % 8 == 0) &&
+            (!blocks || x.soff % 8 == 0) && (long long)x.rows * ((x.cols + 7) / 8) < (1LL << 31);
+    MPSLCC_REQUIRE(x.vec || (long long)x.rows * x.cols < (1LL << 31), ST_INTERNAL, "conversion window too large");
+    MPSLCC_REQUIRE(!x.pad || x.vec, ST_INTERNAL, "padded conversion rows not on 16-byte boundaries");
+    x.tile0 = tot;
+    const long long items = (long long)x.batch * x.rows * (x.vec ? (x.cols + 7) / 8 : x.cols);
+    const long long per = x.vec ? CONV_T : (long long)CONV_T * CONV_E;
+    tot += (items + per - 1) / per;
+  }
+  return tot;
+}
+
+void launch_conv(int prec, const ConvTask* d, int n, long long tot, cudaStream_t s) {
+  const int grid = (int)std::min<long long>(tot, 152LL * 64);
+  if (kprec(prec) == MPSLCC_BF16) conv_kernel<MPSLCC_BF16><<<grid, CONV_T, 0, s>>>(d, n, tot);
+  else conv_kernel<MPSLCC_TF32><<<grid, CONV_T, 0, s>>>(d, n, tot);
+}
+
 void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
   if (t.empty()) return;
-  long long tot = 0;
   const int es = esize(prec);
   for (auto& x : t) {
     if (x.trans)
@@ -1074,19 +1186,16 @@ void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
                     "conv src");
     const long long blocks = x.pattern == 0 ? 0 : (x.pattern == 1 ? 1 : 5);  // extra split blocks
     c.check_bytes(x.dst,
-                  ((long long)(x.batch - 1) * x.s_dst + (long long)(x.rows - 1) * x.dst_ld + blocks * x.soff + x.cols) *
+                  ((long long)(x.batch - 1) * x.s_dst + (long long)(x.rows - 1) * x.dst_ld + blocks * x.soff +
+                   (x.pad ? pad8(x.cols) : x.cols)) *
                       es,
                   "conv dst");
-    x.tile0 = tot;
-    long long nel = (long long)x.rows * x.cols;
-    tot += (long long)x.batch * ((nel + CONV_CHUNK - 1) / CONV_CHUNK);
   }
+  const long long tot = plan_conv(t.data(), (int)t.size());
   dtasks.ensure(&c, t.size() * sizeof(ConvTask));
   cuda_check(cudaMemcpyAsync(dtasks.p, t.data(), t.size() * sizeof(ConvTask), cudaMemcpyHostToDevice, c.s()),
              "conv tasks");
-  int grid = (int)std::min<long long>(tot, 152LL * 16);
-  if (kprec(prec) == MPSLCC_BF16) conv_kernel<MPSLCC_BF16><<<grid, 256, 0, c.s()>>>((const ConvTask*)dtasks.p, (int)t.size(), tot);
-  else conv_kernel<MPSLCC_TF32><<<grid, 256, 0, c.s()>>>((const ConvTask*)dtasks.p, (int)t.size(), tot);
+  launch_conv(prec, (const ConvTask*)dtasks.p, (int)t.size(), tot, c.s());
   cuda_check(cudaGetLastError(), "conv launch");
   c.st.kernel_launches++;
 }
@@ -1273,7 +1382,7 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
   // phase 2), per run of channels with equal piece masks
   std::vector<ConvTask> cv;
   auto conv = [&](const double* src, int src_ld, void* dst, int dst_ld, int rows, int cols, int batch,
-                  long long s_src, long long s_dst, long long soff) {
+                  long long s_src, long long s_dst, long long soff, int pad) {
     ConvTask t;
     std::memset(&t, 0, sizeof(t));
     t.src = src;
@@ -1287,6 +1396,7 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
     t.s_dst = s_dst;
     t.pattern = six ? 2 : 0;
     t.soff = soff;
+    t.pad = pad;
     cv.push_back(t);
   };
   for (size_t bi = 0; bi < nbk; ++bi) {
@@ -1307,26 +1417,30 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
           const long ro = piece_off(lf.FLb, fb, so), co = piece_off(lf.FLk, fk, sn);
           conv(lf.data.d() + lf.off[bi] + ro * K + sg.koff + (long)w * sg.width + co, (int)K,
                (char*)S->lcat.p + (size_t)(S->lcat_off[bi] + ro * pitch + S->kblk[bi][g][sn] + (long)w * padp(dc)) * es,
-               (int)pitch, dr, dc, w1 - w, sg.width, padp(dc), S->K8[bi]);
+               (int)pitch, dr, dc, w1 - w, sg.width, padp(dc), S->K8[bi], 1);
         }
         w = w1;
       }
     }
   }
-  // ... and of R' (A side of phase 1), into the so-major stack rows
+  // ... and of R' (A side of phase 1), into the so-major stack rows.  A piece
+  // starts at any column: its window is widened to whole groups of 8 (what
+  // lies between is zero in the fused operator too), windows that meet join.
   for (const auto& u : S->u1) {
     const auto& st = rf.stk[u.si];
     const int rb = rf.FRb.d[rf.kb[st.bidx]], fk = rf.kk[st.kidx], rk = rf.FRk.d[fk];
     const long pitch = sp * pad8(rk);
+    std::vector<std::pair<long, long>> win;
     for (int sn = 0; sn < 4; ++sn) {
       if (!(u.in >> sn & 1)) continue;
-      const int dc = piece_dim(rf.FRk, fk, sn);
-      if (dc == 0) continue;
-      const long co = piece_off(rf.FRk, fk, sn);
-      conv(rf.base() + st.off + ((long)u.w0 * rb + u.boff) * rk + co, rk,
-           (char*)S->rstk.p + (size_t)(S->stk_off[u.si] + u.row0 * pitch + co) * es, (int)pitch, u.d, dc, u.w1 - u.w0,
-           (long long)rb * rk, (long long)u.d * pitch, pad8(rk));
+      const long dc = piece_dim(rf.FRk, fk, sn), co = piece_off(rf.FRk, fk, sn);
+      if (dc > 0) win.push_back({co & ~7L, pad8(co + dc)});
     }
+    for (const auto& x : merge_exact(win))
+      conv(rf.base() + st.off + ((long)u.w0 * rb + u.boff) * rk + x.first, rk,
+           (char*)S->rstk.p + (size_t)(S->stk_off[u.si] + u.row0 * pitch + x.first) * es, (int)pitch, u.d,
+           (int)(std::min<long>(x.second, rk) - x.first), u.w1 - u.w0, (long long)rb * rk, (long long)u.d * pitch,
+           pad8(rk), 1);
   }
   run_conv(c, layout, cv, S->conv);
   // per-call conversion of the input vector (B side of phase 1)
@@ -1347,6 +1461,7 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
       t.batch = 1;
       t.pattern = six ? 3 : 0;
       t.soff = pad8(rk);
+      t.pad = 1;
       S->xconv.push_back(t);
     }
   }
@@ -1726,9 +1841,9 @@ void tc_selftest(Ctx& c, int prec, int m, int n, int k, const double* A, const d
   std::vector<ConvTask> cv(2);
   std::memset(cv.data(), 0, sizeof(ConvTask) * 2);
   cv[0].src = dA.d(); cv[0].dst = lA.p; cv[0].rows = m; cv[0].cols = k; cv[0].src_ld = k; cv[0].dst_ld = (int)kk;
-  cv[0].batch = 1; cv[0].pattern = sp == 2 ? 1 : 0; cv[0].soff = k8;
+  cv[0].batch = 1; cv[0].pattern = sp == 2 ? 1 : 0; cv[0].soff = k8; cv[0].pad = 1;
   cv[1].src = dB.d(); cv[1].dst = lB.p; cv[1].rows = n; cv[1].cols = k; cv[1].src_ld = k; cv[1].dst_ld = (int)kk;
-  cv[1].batch = 1; cv[1].pattern = sp == 2 ? 1 : 0; cv[1].soff = k8;
+  cv[1].batch = 1; cv[1].pattern = sp == 2 ? 1 : 0; cv[1].soff = k8; cv[1].pad = 1;
   run_conv(c, prec, cv, conv);
   const int oes = mode == 1 ? 2 : 4;
   out.alloc(&c, (size_t)m * n * oes);
@@ -1827,24 +1942,17 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
   cuda_check(cudaGetDevice(&cur), "cudaGetDevice");
   MPSLCC_REQUIRE(cur == device, ST_ARG, "device must be the current device");
   char* base = (char*)noalloc_scratch(device);
-  // operand copies: zero padding columns, then convert
+  // operand copies; the conversion clears the padding columns
   cuda_check(cudaMemsetAsync(base + o_err, 0, 256, stream), "noalloc memset");
-  cuda_check(cudaMemsetAsync(base + o_a, 0, o_c - o_a, stream), "noalloc memset");
   ConvTask cv[2];
   std::memset(cv, 0, sizeof(cv));
   cv[0].src = dA; cv[0].dst = base + o_a; cv[0].rows = m; cv[0].cols = k; cv[0].src_ld = k; cv[0].dst_ld = (int)kk;
-  cv[0].batch = 1; cv[0].pattern = sp == 2 ? 1 : 0; cv[0].soff = k8;
+  cv[0].batch = 1; cv[0].pattern = sp == 2 ? 1 : 0; cv[0].soff = k8; cv[0].pad = 1;
   cv[1].src = dB; cv[1].dst = base + o_b; cv[1].rows = n; cv[1].cols = k; cv[1].src_ld = k; cv[1].dst_ld = (int)kk;
-  cv[1].batch = 1; cv[1].pattern = sp == 2 ? 1 : 0; cv[1].soff = k8;
-  long long tot = 0;
-  for (auto& x : cv) {
-    x.tile0 = tot;
-    tot += ((long long)x.rows * x.cols + CONV_CHUNK - 1) / CONV_CHUNK;
-  }
+  cv[1].batch = 1; cv[1].pattern = sp == 2 ? 1 : 0; cv[1].soff = k8; cv[1].pad = 1;
+  const long long tot = plan_conv(cv, 2);
   cuda_check(cudaMemcpyAsync(base + o_conv, cv, sizeof(cv), cudaMemcpyHostToDevice, stream), "noalloc tasks");
-  int cgrid = (int)std::min<long long>(tot, 152LL * 16);
-  if (kprec(prec) == MPSLCC_BF16) conv_kernel<MPSLCC_BF16><<<cgrid, 256, 0, stream>>>((const ConvTask*)(base + o_conv), 2, tot);
-  else conv_kernel<MPSLCC_TF32><<<cgrid, 256, 0, stream>>>((const ConvTask*)(base + o_conv), 2, tot);
+  launch_conv(prec, (const ConvTask*)(base + o_conv), 2, tot, stream);
   cuda_check(cudaGetLastError(), "noalloc conv");
   // one GEMM task writing FP32 rows of C
   TcTask t;
@@ -1947,6 +2055,7 @@ void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
     t.pattern = side;
     t.soff = kp;
     t.trans = trans;
+    t.pad = 1;
     cv.push_back(t);
     opoff[k] = off;
     return off;
@@ -1966,7 +2075,6 @@ void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
   }
   if (jobs.empty()) return;
   c.scratch_tc.ensure(&c, std::max<long>(tot, 8) * 2);
-  cuda_check(cudaMemsetAsync(c.scratch_tc.p, 0, std::max<long>(tot, 8) * 2, c.s()), "tc scratch zero");
   char* base = (char*)c.scratch_tc.p;
   for (auto& t : cv) t.dst = base + (uintptr_t)t.dst * 2;
   run_conv(c, MPSLCC_BF16, cv, c.tc_conv_tasks);
