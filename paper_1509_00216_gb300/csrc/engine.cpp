@@ -160,7 +160,7 @@ void run_gemms(Ctx& c, std::vector<GemmTask>& t) {
   for (const auto& x : t) validate_gemm(c, x);
   F64Plan p;
   plan_f64(t.data(), (int)t.size(), p);
-  if (p.tiles_tc + p.tiles_small == 0) return;
+  if (f64_plan_bytes(p) == 0) return;
   c.gtask.ensure(&c, f64_plan_bytes(p));
   upload_f64(p, c.gtask.p, c.s());
   run_f64(c, p, c.gtask.p);

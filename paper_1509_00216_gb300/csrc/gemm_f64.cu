@@ -6,7 +6,7 @@
 // run as exact integer products on the tensor cores (Ozaki's splitting): every
 // row of an operand is scaled by a power of two to 62-bit integers, each
 // integer is cut into eight balanced digits of eight bits, digits are exact in
-// BF16, and products of digit planes accumulate exactly in FP32 (at most 8 x
+// FP16, and products of digit planes accumulate exactly in FP32 (at most 8 x
 // 128 products of 2^14).  The 36 plane pairs whose weight is at least 2^-56 of
 // the largest are formed; pairs of equal weight share one accumulator, the
 // accumulators are combined in integers and rounded to FP64 once per 1024 K
@@ -14,14 +14,17 @@
 // what is lost is the rounding of an operand to 2^-62 of its row's largest
 // value and the pairs left out (2^-60 of a product of two such values).
 //
-// Tasks of few multiply-adds run on the FP64 pipe (gemm_f64_small_kernel).
+// Tasks of few multiply-adds run on the FP64 pipe (gemm_f64_pipe_kernel).
 //
 // Measured against the 64 x 64 FP64-pipe tiles that did all of this before
-// (3-band model, M1 = 500, middle position): sigma phases 27.0 + 28.8 ms ->
-// 3.8 + 3.4 ms, error against 64-bit contraction 2.4e-15 -> 1.0e-15; the
-// environment passes of the energies at M1 = 400, 790 ms -> 120 ms.
+// (3-band model, middle position, M1 = 500): sigma phases 27.0 + 28.8 ms ->
+// 2.5 + 3.4 ms, error against 64-bit contraction 2.4e-15 -> 1.0e-15; all
+// products of the energies at M1 = 400, 790 ms -> 49 ms.  A tile's time is its
+// chain (loads, cutting, products, drain, conversion, stores), of which the
+// integer pipe carries most; the tensor pipe is busy a tenth of it.
 #include <algorithm>
 #include <atomic>
+#include <vector>
 #include <cstring>
 
 #include "engine.hpp"
@@ -31,27 +34,34 @@ namespace mpslcc {
 
 namespace {
 
-constexpr int TM = 128, TN = 64;       // tensor-core tile (rows of X, rows of Y)
+constexpr int TM = 128;                // rows of X in a tensor-core tile
 constexpr int KB = 1024;               // K values per scaling block
-constexpr int KS = 32;                 // K values per step (half a 128-byte row of BF16)
+constexpr int KS = 32;                 // K values per step (64 bytes of FP16)
 constexpr int CHUNK = 4;               // steps between two drains: 128 K values
 constexpr int PLANES = 8;
-constexpr int THREADS = 512;
-constexpr int XPLANE = TM * 128, YPLANE = TN * 128;          // bytes of a digit plane (64 K values)
-constexpr int OPER = PLANES * (XPLANE + YPLANE);             // 192 KB
-constexpr int STG_LD = TN + 1;                               // staging pitch of the result tile, doubles
-constexpr int SMEM_TC = OPER + 1024 + KB * 4 + (TM + TN) * 4 + 64 + (int)sizeof(F64Task);
-constexpr int SM_T = 32;               // tile of the FP64-pipe kernel
 constexpr int MAX_DEV = 128;
 
-__device__ __forceinline__ int find_f64(const F64Task* t, int n, long long tile) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (t[mid].tile0 <= tile) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+// Two shapes.  TN = 64, one CTA of 16 warps per SM: two step buffers, so that
+// digits are cut while the previous step multiplies; 8 x 64 accumulator columns
+// take all of tensor memory.  TN = 32, two CTAs of 8 warps per SM, one step
+// buffer each: for short sums, whose time is the chain load - cut - multiply -
+// drain - write of a tile, one CTA's chain fills the other's gaps.
+template <int TN_> struct F64Cfg {
+  static constexpr int TN = TN_;
+  static constexpr int WARPS = TN == 64 ? 16 : 8, THREADS = 32 * WARPS, CTAS = TN == 64 ? 1 : 2;
+  static constexpr int NBUF = TN == 64 ? 2 : 1;
+  static constexpr int ROW = 64 * NBUF;                        // bytes of a plane's row
+  static constexpr int XPLANE = TM * ROW, YPLANE = TN * ROW;
+  static constexpr int OPER = PLANES * (XPLANE + YPLANE);      // 192 or 80 KB
+  static constexpr int XU = 16 / WARPS;                        // loader units of X per warp
+  static constexpr int YU0 = WARPS - TN / 8;                   // first warp that loads Y
+};
+struct F64Slot {
+  F64Task t;
+  int b, ks, ix, iy;
+};
+template <class F> constexpr int f64_smem() {
+  return F::OPER + 1024 + KB * 4 + (TM + F::TN) * 8 + 64 + 2 * (int)sizeof(F64Slot) + (TM + F::TN) * 8;
 }
 
 struct F64Tile { int b, ks, ix, iy; };
@@ -59,13 +69,51 @@ __device__ __forceinline__ F64Tile tile_of(const F64Task& T, long long tile) {
   const long long local = tile - T.tile0;
   const long long txy = (long long)T.tx * T.ty, per_b = txy * T.ksplit;
   F64Tile t;
-  t.b = (int)(local / per_b);
-  const long long r = local - (long long)t.b * per_b;
-  t.ks = (int)(r / txy);
-  const int q = (int)(r - (long long)t.ks * txy);
-  t.ix = q / T.ty;
-  t.iy = q - t.ix * T.ty;
+  unsigned q;
+  if (local < (1LL << 31) && per_b < (1LL << 31)) {   // 64-bit divisions cost hundreds of instructions
+    t.b = (int)((unsigned)local / (unsigned)per_b);
+    const unsigned r = (unsigned)local - (unsigned)t.b * (unsigned)per_b;
+    t.ks = (int)(r / (unsigned)txy);
+    q = r - (unsigned)t.ks * (unsigned)txy;
+  } else {
+    t.b = (int)(local / per_b);
+    const long long r = local - (long long)t.b * per_b;
+    t.ks = (int)(r / txy);
+    q = (unsigned)(r - (long long)t.ks * txy);
+  }
+  t.ix = (int)(q / (unsigned)T.ty);
+  t.iy = (int)(q - (unsigned)t.ix * (unsigned)T.ty);
   return t;
+}
+
+// Task of `tile`, found by a whole warp from task `prev` on (a CTA's tiles
+// ascend): the next 32 tasks, then 32-fold steps.
+__device__ __forceinline__ int warp_find(const F64Task* t, int n, long long tile, int prev) {
+  const int lane = threadIdx.x & 31;
+  int lo = prev, hi = min(n, prev + 33), step = 1;   // t[lo] starts at or before the tile
+  for (;;) {
+    const int i = lo + (lane + 1) * step;
+    const int c = __popc(__ballot_sync(0xffffffffu, i < hi && t[i].tile0 <= tile));
+    lo += c * step;
+    if (step == 1 && (c < 32 || lo + 1 >= n)) return lo;
+    hi = step == 1 ? n : min(hi, lo + step);
+    step = (hi - lo + 31) / 32;
+    if (step < 1) step = 1;
+  }
+}
+// Fills a slot with tile's task and coordinates (a whole warp); returns the task.
+__device__ __forceinline__ int fetch_slot(F64Slot* s, const F64Task* t, int n, long long tile, int prev) {
+  const int lane = threadIdx.x & 31;
+  const int i = warp_find(t, n, tile, prev);
+  static_assert(sizeof(F64Task) % 8 == 0 && sizeof(F64Task) <= 512, "task copy");
+#pragma unroll
+  for (int w = lane; w < (int)(sizeof(F64Task) / 8); w += 32) ((long long*)&s->t)[w] = ((const long long*)(t + i))[w];
+  __syncwarp();
+  if (lane == 0) {
+    const F64Tile c = tile_of(s->t, tile);
+    s->b = c.b; s->ks = c.ks; s->ix = c.ix; s->iy = c.iy;
+  }
+  return i;
 }
 
 // Offset of row i of a folded operand: rows run over (batch entry, row).
@@ -110,19 +158,29 @@ __device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t* v) {
 }
 
 // One loader unit: up to 32 x 8 or 8 x 32 elements of an operand tile; a
-// thread holds the eight K values q, q + 4, ..., q + 28 of one row's step.
+// thread holds eight K values of one row's step: q, q + 2, ..., q + 14 for q =
+// 0, 1, and 16 more for q = 2, 3 (so that a step of up to 16 values has an
+// empty second half).
 struct Unit {
   const double* p;
-  long long ks;
   int row, q;
   bool ok;
 };
 
-__device__ __forceinline__ void load_unit(const Unit& u, const int* tab, int nk, double (&v)[8]) {
+// Values below nk of the unit's row; tab holds the operand columns, or is null
+// where they are base, base + 1, ...
+__device__ __forceinline__ void load_unit(const Unit& u, long long ks, const int* tab, int base, int nk,
+                                          double (&v)[8]) {
+  const int q0 = u.q < 2 ? u.q : 14 + u.q;
+  const int left = u.ok ? nk - q0 : 0;
+  if (tab) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int k = u.q + 4 * j;
-    v[j] = (u.ok && k < nk) ? __ldg(u.p + (long long)tab[k] * u.ks) : 0.0;
+    for (int j = 0; j < 8; ++j) v[j] = 2 * j < left ? __ldg(u.p + (long long)tab[q0 + 2 * j] * ks) : 0.0;
+  } else {
+    const double* p = u.p + (base + q0) * ks;
+    const long long st = 2 * ks;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = 2 * j < left ? __ldg(p + j * st) : 0.0;
   }
 }
 
@@ -137,93 +195,125 @@ __device__ __forceinline__ uint32_t unit_max(const double (&v)[8], uint32_t m) {
   return m;
 }
 
-// v as an integer of 62 bits relative to the row exponent, offset by 128 in
-// every digit: byte i of the result is digit i plus 128.
+// v as an integer of 62 bits relative to the row exponent (cut towards zero:
+// 2^-61 of the row's largest value at most), offset by 128 in every digit:
+// byte i of the result is digit i plus 128.
 __device__ __forceinline__ unsigned long long digits(double v, int emax) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-  const int e = (hi >> 20) & 0x7ff;
+  const int d = min(emax - (int)((hi >> 20) & 0x7ffu), 63);   // 63 clears zeros too: emax >= 64
   unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  int d = min(emax - e, 62);
-  m <<= 10;                          // one guard bit below the 62-bit grid
-  m = ((m >> d) + 1) >> 1;           // round half up in magnitude
-  if (e == 0) m = 0;
-  const unsigned long long s = (unsigned long long)((long long)(int)hi >> 63);
-  return ((m ^ s) - s) + 0x8080808080808080ull;
+  m = (m << 9) >> d;
+  const long long s = (long long)((int)hi >> 31);
+  return (m ^ (unsigned long long)s) + (0x8080808080808080ull - (unsigned long long)s);
 }
 
-// Writes the unit's eight values as 16 bytes in each digit plane (128-byte
-// swizzle: 16-byte chunk index xor row within the 8-row group).
-__device__ __forceinline__ void store_unit(const Unit& u, const double (&v)[8], int emax, uint8_t* planes, int plane,
+// Exponent of a row scale (exponent of the row's largest value, times two, plus
+// one if its values are taken 2^512-fold).
+__device__ __forceinline__ int scale_exp(int scale) { return (scale >> 1) - ((scale & 1) << 9); }
+
+// Writes the unit's eight values as 16 bytes in each digit plane: rows of two
+// steps with 128-byte swizzle (16-byte chunk xor row mod 8), or rows of one
+// step with 64-byte swizzle (chunk xor row / 2 mod 4).  A digit's byte under
+// the FP16 exponent of 1024 is 1024 + digit + 128; one subtraction leaves it.
+// (Bound by the integer pipe: two byte permutations per pair of digits, where
+// BF16's shorter significand needed four operations.)
+template <int NBUF>
+__device__ __forceinline__ void store_unit(const Unit& u, double (&v)[8], int scale, uint8_t* planes, int plane,
                                            int half) {
-  unsigned long long t[8];
+  const int emax = scale >> 1;
+  if (scale & 1) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) t[j] = digits(v[j], emax);
-  uint8_t* dst = planes + u.row * 128 + (((half * 4 + u.q) ^ (u.row & 7)) << 4);
+    for (int j = 0; j < 8; ++j) v[j] *= 0x1p512;
+  }
+  uint32_t t0[8], t1[8];
 #pragma unroll
-  for (int p = 0; p < PLANES; ++p) {
-    const int dg = PLANES - 1 - p;   // plane 0 holds the most significant digit
-    uint32_t w[4];
+  for (int j = 0; j < 8; ++j) {
+    const unsigned long long t = digits(v[j], emax);
+    t0[j] = (uint32_t)t;
+    t1[j] = (uint32_t)(t >> 32);
+  }
+  uint8_t* dst = NBUF == 2 ? planes + u.row * 128 + (((half * 4 + u.q) ^ (u.row & 7)) << 4)
+                           : planes + u.row * 64 + ((u.q ^ ((u.row >> 1) & 3)) << 4);
+#pragma unroll
+  for (int p = 0; p < PLANES; p += 2) {
+    // planes p and p + 1 (plane 0 the most significant) are bytes s + 1 and s
+    // of the same word
+    const int s = (PLANES - 2 - p) & 3;
+    uint32_t w0[4], w1[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const uint32_t a = dg < 4 ? (uint32_t)t[2 * j] : (uint32_t)(t[2 * j] >> 32);
-      const uint32_t b = dg < 4 ? (uint32_t)t[2 * j + 1] : (uint32_t)(t[2 * j + 1] >> 32);
-      const int s = dg & 3;
-      // the digits plus 128 in the low bytes of two 16-bit halves
-      const uint32_t y = __byte_perm(a, b, s | (s + 4) << 8);
-      // BF16 128 + (y mod 128), minus 128 or 256: the digit, exactly
-      const uint32_t f = (y & 0x007f007fu) | 0x43004300u;
-      const uint32_t g = (y & 0x00800080u) ^ 0x43804380u;
-      uint32_t r;
-      asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(f), "r"(g));
-      w[j] = r;
+      const uint32_t a = p < 4 ? t1[2 * j] : t0[2 * j], b = p < 4 ? t1[2 * j + 1] : t0[2 * j + 1];
+      const uint32_t x = __byte_perm(a, b, s | (s + 4) << 4 | (s + 1) << 8 | (s + 5) << 12);   // a_s b_s a_s+1 b_s+1
+      const uint32_t lo = __byte_perm(x, 0x64646464u, 0x4140), hi = __byte_perm(x, 0x64646464u, 0x4342);
+      asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(w1[j]) : "r"(lo), "r"(0x64806480u));
+      asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(w0[j]) : "r"(hi), "r"(0x64806480u));
     }
-    *reinterpret_cast<uint4*>(dst + p * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(dst + p * plane) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
+    *reinterpret_cast<uint4*>(dst + (p + 1) * plane) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
   }
 }
 
 // hi 2^32 + lo, in units of 2^(eab - 2112), as FP64 rounded to nearest.
 __device__ __forceinline__ double to_f64(long long hi, long long lo, int eab) {
-  unsigned long long w0 = ((unsigned long long)hi << 32) + (unsigned long long)lo;
-  long long w1 = (hi >> 32) + (lo >> 63) + (w0 < (unsigned long long)lo ? 1 : 0);
-  const unsigned long long s = (unsigned long long)(w1 >> 63);
-  w0 ^= s;
-  w1 ^= (long long)s;
-  w0 -= s;
-  if (s && w0 == 0) ++w1;
-  int lz, top;
-  unsigned long long nrm;
-  if (w1 != 0) {
-    lz = __clzll(w1);
-    nrm = (unsigned long long)w1 << lz;
-    if (lz) nrm |= w0 >> (64 - lz);
-    top = 127 - lz;
-  } else {
-    if (w0 == 0) return 0.0;
-    lz = __clzll((long long)w0);
-    nrm = w0 << lz;
-    top = 63 - lz;
+  const long long h = hi + (lo >> 32);
+  uint32_t a2 = (uint32_t)((unsigned long long)h >> 32), a1 = (uint32_t)h, a0 = (uint32_t)lo;
+  const uint32_t neg = (uint32_t)((int)a2 >> 31);
+  // magnitude of the 96-bit value
+  asm("xor.b32 %0, %0, %3;\n xor.b32 %1, %1, %3;\n xor.b32 %2, %2, %3;\n"
+      "sub.cc.u32 %0, %0, %3;\n subc.cc.u32 %1, %1, %3;\n subc.u32 %2, %2, %3;"
+      : "+r"(a0), "+r"(a1), "+r"(a2)
+      : "r"(neg));
+  int e = eab + 95 - 1089;
+  if (a2 == 0) {
+    a2 = a1; a1 = a0; a0 = 0;
+    e -= 32;
+    if (a2 == 0) {
+      a2 = a1; a1 = 0;
+      e -= 32;
+      if (a2 == 0) return 0.0;
+    }
   }
-  const int e = eab + top - 1089;
-  const unsigned long long mant = (nrm >> 11) + ((nrm >> 10) & 1);   // in [2^52, 2^53]
+  const int lz = __clz((int)a2);
+  e -= lz;
+  const uint32_t m1 = __funnelshift_l(a1, a2, lz), m0 = __funnelshift_l(a0, a1, lz);
+  uint32_t rl = __funnelshift_r(m0, m1, 11), rh = m1 >> 11;   // 53 bits, then the rounding bit
+  asm("add.cc.u32 %0, %0, %2;\n addc.u32 %1, %1, 0;" : "+r"(rl), "+r"(rh) : "r"((m0 >> 10) & 1u));
   if (e < 1 || e > 2045) {
-    const double v = scalbn((double)mant, eab + top - 52 - 2112);
-    return s ? -v : v;
+    const double v = scalbn((double)(((unsigned long long)rh << 32) | rl), e - 1075);
+    return neg ? -v : v;
   }
-  return __longlong_as_double((long long)(((((unsigned long long)(e - 1)) << 52) + mant) | (s << 63)));
+  return __hiloint2double((int)((rh + ((uint32_t)(e - 1) << 20)) | (neg & 0x80000000u)), (int)rl);
 }
 
-__global__ void __launch_bounds__(THREADS, 1)
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
+// With MULTI = false every task sums at most one chunk (128 K values): the
+// accumulators go straight to the output, and the registers can hold two steps'
+// values.  With MULTI = true the chunks' sums stay in 64 registers a thread and
+// a step's values are loaded when they are cut; both kinds in one kernel
+// spilled registers to L2 in the cutting loop.
+template <int TN, bool MULTI>
+__global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
     gemm_f64_tc_kernel(const F64Task* __restrict__ tasks, int ntasks, long long total, int* err,
                        unsigned long long wait_ns) {
+  using F = F64Cfg<TN>;
+  constexpr int THREADS = F::THREADS, XU = F::XU, NBUF = F::NBUF;
+  constexpr bool PAIR = !MULTI && XU == 1;            // registers hold two steps' values
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* yplanes = smem + PLANES * XPLANE;
-  int* tab = (int*)(smem + OPER);                     // operand column of each K value of the block
+  uint8_t* yplanes = smem + PLANES * F::XPLANE;
+  int* tab = (int*)(smem + F::OPER);                  // operand column of each K value of the block
   uint32_t* rmax = (uint32_t*)(tab + KB);             // largest high word per row: X, then Y
-  uint64_t* bar = (uint64_t*)(rmax + TM + TN);        // [2] products of a half done, [1] drain
+  int* rscale = (int*)(rmax + TM + TN);               // the rows' scales
+  uint64_t* bar = (uint64_t*)(rscale + TM + TN);      // [2] products of a buffer done, [1] drain
   volatile uint32_t* tslot = (volatile uint32_t*)(bar + 3);
-  F64Task* task = (F64Task*)(bar + 8);                // the tile's task
-  double* stg = (double*)smem;                        // result tile (after the products)
+  F64Slot* slots = (F64Slot*)(bar + 8);               // this tile's task and the next one's
+  long long* coff = (long long*)(slots + 2);          // output offset of each column
+  long long* roff = coff + TN;                        // and of each row
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     mbar_init(&bar[0], 1);
@@ -234,100 +324,152 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32((const void*)tslot)),
-                 "r"(512)
+                 "r"(8 * TN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  int ti = 0;                                         // warp 1: task of the last slot filled
+  if (warp == 1 && blockIdx.x < total) ti = fetch_slot(&slots[0], tasks, ntasks, blockIdx.x, 0);
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tslot;
   const int quarter = warp & 3, colq = warp >> 2;     // this warp's part of a drain
+  const uint32_t tdrain = tmem + ((uint32_t)(quarter * 32) << 16) + colq * 16;
+  const int orow = quarter * 32 + lane;               // this thread's row of a drain
   uint32_t it = 0;                                    // steps issued so far
   bool abort = false;
+  int cur = 0;
 
-  for (long long tile = blockIdx.x; tile < total && !abort; tile += gridDim.x) {
-    if (tid < (int)(sizeof(F64Task) / 8))
-      ((long long*)task)[tid] = ((const long long*)(tasks + find_f64(tasks, ntasks, tile)))[tid];
-    __syncthreads();
-    const F64Task& T = *task;
-    const F64Tile tc = tile_of(T, tile);
-    const int x0 = tc.ix * TM, y0 = tc.iy * TN;
+  for (long long tile = blockIdx.x; tile < total && !abort; tile += gridDim.x, cur ^= 1) {
+    const F64Task& T = slots[cur].t;
+    const int x0 = slots[cur].ix * TM, y0 = slots[cur].iy * TN;
     const int nx = min(TM, T.mx - x0), ny = min(TN, T.my - y0);
-    const int k0 = tc.ks * T.kchunk, k1 = min(T.k, k0 + T.kchunk);
-    const double* X = T.x + (long long)tc.b * T.xub;
-    const double* Y = T.y + (long long)tc.b * T.yub;
-    double* C = T.c + (long long)tc.b * T.cub + (long long)tc.ks * T.sK;
-    // loader units: one of X per warp, one of Y in warps 8 .. 15
-    Unit ux, uy;
-    if (T.xks == 1) { ux.row = warp * 8 + (lane & 7); ux.q = lane >> 3; }
-    else { ux.row = (warp >> 2) * 32 + lane; ux.q = warp & 3; }
-    ux.ks = T.xks;
-    ux.ok = ux.row < nx;
-    ux.p = X + (ux.ok ? row_off(x0 + ux.row, T.nx, T.xrs, T.xbs) : 0);
-    const int w8 = warp & 7;
-    if (T.yks == 1) { uy.row = w8 * 8 + (lane & 7); uy.q = lane >> 3; }
-    else { uy.row = (w8 >> 2) * 32 + lane; uy.q = w8 & 3; }
-    uy.ks = T.yks;
-    uy.ok = warp >= 8 && uy.row < ny;
-    uy.p = Y + (uy.ok ? row_off(y0 + uy.row, T.ny, T.yrs, T.ybs) : 0);
+    const int k0 = slots[cur].ks * T.kchunk, k1 = min(T.k, k0 + T.kchunk);
+    const bool next = tile + gridDim.x < total;
+    bool fetched = false;
+    // loader units: 16 of X over all warps, TN / 8 of Y over the last ones
+    Unit ux[XU], uy;
+#pragma unroll
+    for (int u = 0; u < XU; ++u) {
+      const int n = warp + u * F::WARPS;
+      if (T.xks == 1) { ux[u].row = n * 8 + (lane & 7); ux[u].q = lane >> 3; }
+      else { ux[u].row = (n >> 2) * 32 + lane; ux[u].q = n & 3; }
+      ux[u].ok = ux[u].row < nx;
+      ux[u].p = T.x + (long long)slots[cur].b * T.xub + (ux[u].ok ? row_off(x0 + ux[u].row, T.nx, T.xrs, T.xbs) : 0);
+    }
+    const int wy = warp - F::YU0;
+    if (T.yks == 1) { uy.row = wy * 8 + (lane & 7); uy.q = lane >> 3; }
+    else { uy.row = (wy >> 2) * 32 + lane; uy.q = wy & 3; }
+    uy.ok = wy >= 0 && uy.row < ny;
+    uy.p = T.y + (long long)slots[cur].b * T.yub + (uy.ok ? row_off(y0 + uy.row, T.ny, T.yrs, T.ybs) : 0);
+    if (tid < ny) coff[tid] = row_off(y0 + tid, T.ny, T.cys, T.cyb);
+    if (tid >= THREADS - nx) roff[tid - (THREADS - nx)] = row_off(x0 + tid - (THREADS - nx), T.nx, T.cxs, T.cxb);
+    const bool mine = quarter * 32 < nx && colq * 16 < ny;
 
     int kb = k0;
     do {
       const int len = max(0, min(KB, k1 - kb));
       const int nst = (len + KS - 1) / KS;
       if (tid < TM + TN) rmax[tid] = 0;
-      for (int i = tid; i < len; i += THREADS) tab[i] = k_col(T, kb + i);
+      if (T.kr)
+        for (int i = tid; i < len; i += THREADS) tab[i] = k_col(T, kb + i);
       __syncthreads();
-      // row exponents of this block; the last step visited stays in registers
-      double vx[8], vy[8];
-      uint32_t mx = 0, my = 0;
-      for (int s = nst - 1; s >= 0; --s) {
-        load_unit(ux, tab + s * KS, len - s * KS, vx);
-        load_unit(uy, tab + s * KS, len - s * KS, vy);
-        mx = unit_max(vx, mx);
-        my = unit_max(vy, my);
+      struct Vals { double x[XU][8], y[8]; };
+      auto load = [&](int s, Vals& v) {
+        const int* tb = T.kr ? tab + s * KS : nullptr;
+#pragma unroll
+        for (int u = 0; u < XU; ++u) load_unit(ux[u], T.xks, tb, kb + s * KS, len - s * KS, v.x[u]);
+        load_unit(uy, T.yks, tb, kb + s * KS, len - s * KS, v.y);
+      };
+      // largest magnitude of each row over the block
+      uint32_t mx[XU] = {}, my = 0;
+      auto widest = [&](const Vals& v) {
+#pragma unroll
+        for (int u = 0; u < XU; ++u) mx[u] = unit_max(v.x[u], mx[u]);
+        my = unit_max(v.y, my);
+      };
+      Vals v0, v1;   // PAIR: the values of the next even and odd step
+      if (!PAIR) {
+        for (int s = nst - 1; s >= 0; --s) {
+          load(s, v0);
+          widest(v0);
+        }
+      } else {
+        for (int s = (nst - 1) & ~1; s >= 0; s -= 2) {
+          load(s, v0);
+          if (s + 1 < nst) load(s + 1, v1);
+          widest(v0);
+          if (s + 1 < nst) widest(v1);
+        }
       }
-      if (mx) atomicMax(&rmax[ux.row], mx);
+#pragma unroll
+      for (int u = 0; u < XU; ++u)
+        if (mx[u]) atomicMax(&rmax[ux[u].row], mx[u]);
       if (my) atomicMax(&rmax[TM + uy.row], my);
       __syncthreads();
-      // rows that hold an infinity, a NaN or nothing but values near the
-      // subnormal range go through plain multiply-adds
+      // Row scales.  A row with an infinity or a NaN sends the tile through
+      // plain multiply-adds; a row of nothing but values below 2^-959 (noise to
+      // the power of the chain's length is met in earnest) is taken 2^512-fold.
       bool bad = false;
       if (tid < TM + TN) {
         const uint32_t h = rmax[tid];
-        bad = (h >> 20) == 0x7ffu || (h != 0 && (h >> 20) < 64u);
+        bad = (h >> 20) == 0x7ffu;
+        int e = (int)(h >> 20), tiny = 0;
+        if (e < 64) {
+          tiny = h != 0;
+          e = tiny ? (int)((uint32_t)__double2hiint(__hiloint2double((int)h + 1, 0) * 0x1p512) >> 20) : 64;
+        }
+        rscale[tid] = e << 1 | tiny;
       }
       const bool plain = __syncthreads_or(bad);
-      long long ahi[16], alo[16];   // sums of accumulators 0 .. 3 and 4 .. 7
+      const int pm = put_mode(T, kb == k0);
+      double* C = T.c + (long long)slots[cur].b * T.cub + (long long)slots[cur].ks * T.sK;
+      long long ahi[MULTI ? 16 : 1], alo[MULTI ? 16 : 1];   // sums of accumulators 0 .. 3 and 4 .. 7
+      if (MULTI) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) ahi[j] = alo[j] = 0;
-      const bool mine = quarter * 32 < nx && colq * 16 < ny;
+        for (int j = 0; j < 16; ++j) ahi[j] = alo[j] = 0;
+      }
+      // accumulators of columns cb and cb + 1 of this thread's row, added to hi and lo
+      auto drain2 = [&](int cb, long long* hi, long long* lo) {
+        uint32_t v[8][2];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) tmem_ld2(tdrain + cb + g * TN, v[g]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          int c[8];
+#pragma unroll
+          for (int g = 0; g < 8; ++g) c[g] = __float2int_rn(__uint_as_float(v[g][j]));
+          // |c0| <= 2^19, |c2| <= 2^22: 256 times them plus the next fits 32 bits
+          hi[j] = mad_wide(c[0] * 256 + c[1], 1 << 16, mad_wide(c[2] * 256 + c[3], 1, hi[j]));
+          lo[j] = mad_wide(c[4], 1 << 24, mad_wide(c[5], 1 << 16, mad_wide(c[6], 256, mad_wide(c[7], 1, lo[j]))));
+        }
+      };
       if (!plain) {
-        const int ex = ux.ok ? (int)(rmax[ux.row] >> 20) : 0, ey = uy.ok ? (int)(rmax[TM + uy.row] >> 20) : 0;
-        for (int s = 0; s < nst; ++s, ++it) {
-          const uint32_t h = it & 1u;
+        auto step = [&](int s, Vals& v) -> bool {
+          const uint32_t h = NBUF == 2 ? it & 1u : 0u, use = NBUF == 2 ? it >> 1 : it;   // buffer, its use count
+          if (!PAIR && nst > 1) load(s, v);
           bool ok = true;
-          if (it >= 2) ok = mbar_wait(&bar[h], ((it >> 1) - 1) & 1u, err, 11, wait_ns);
+          if (use >= 1) ok = mbar_wait(&bar[h], (use - 1) & 1u, err, 11, wait_ns);
           if (ok) {
-            if (ux.ok) store_unit(ux, vx, ex, smem, XPLANE, h);
-            if (uy.ok) store_unit(uy, vy, ey, yplanes, YPLANE, h);
+#pragma unroll
+            for (int u = 0; u < XU; ++u)
+              if (ux[u].ok) store_unit<NBUF>(ux[u], v.x[u], rscale[ux[u].row], smem, F::XPLANE, h);
+            if (uy.ok) store_unit<NBUF>(uy, v.y, rscale[TM + uy.row], yplanes, F::YPLANE, h);
           }
-          if (s + 1 < nst) {
-            load_unit(ux, tab + (s + 1) * KS, len - (s + 1) * KS, vx);
-            load_unit(uy, tab + (s + 1) * KS, len - (s + 1) * KS, vy);
-          }
+          if (PAIR && s + 2 < nst) load(s + 2, v);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           fence_before();
-          if (!__syncthreads_and(ok)) { abort = true; break; }
-          const bool chunk_end = s + 1 == nst || (s & (CHUNK - 1)) == CHUNK - 1;
+          if (!__syncthreads_and(ok)) return false;
           if (tid == 0) {
             fence_after();
-            const uint64_t dx = sdesc(smem + h * 64), dy = sdesc(yplanes + h * 64);
-            constexpr uint64_t PX = XPLANE >> 4, PY = YPLANE >> 4;
+            const uint64_t dx = sdesc_k<F::ROW>(smem + h * 64), dy = sdesc_k<F::ROW>(yplanes + h * 64);
+            constexpr uint64_t PX = F::XPLANE >> 4, PY = F::YPLANE >> 4;
             const bool fresh = (s & (CHUNK - 1)) == 0;
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk) {
+              if (kk == 1 && len - s * KS <= KS / 2) break;   // empty second half
               const uint64_t a = dx + 2 * kk, b = dy + 2 * kk;
               // plane pair (i, j) adds to accumulator i + j <= 7: for one i the
               // Y planes lie one after the other, and so do their accumulators
@@ -335,82 +477,101 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
               for (int i = 0; i < PLANES; ++i) {
                 const int n = (PLANES - i) * TN;   // columns
-                umma<MPSLCC_BF16>(tmem + i * TN, a + i * PX, b, idesc<MPSLCC_BF16>(TM, n < 256 ? n : 256),
-                                  i == 0 ? keep : 1u);
+                umma<MPSLCC_BF16>(tmem + i * TN, a + i * PX, b, idesc_f16(TM, n < 256 ? n : 256), i == 0 ? keep : 1u);
                 if (n > 256)
-                  umma<MPSLCC_BF16>(tmem + i * TN + 256, a + i * PX, b + 4 * PY, idesc<MPSLCC_BF16>(TM, n - 256),
+                  umma<MPSLCC_BF16>(tmem + i * TN + 256, a + i * PX, b + (256 / TN) * PY, idesc_f16(TM, n - 256),
                                     i == 0 ? keep : 1u);
               }
             }
             umma_commit(&bar[h]);
           }
-          if (chunk_end) {
-            // all products up to this step are done: combine the weights
-            if (!mbar_wait(&bar[h], (it >> 1) & 1u, err, 12, wait_ns)) abort = true;
+          if (warp == 1 && next && !fetched) {   // while the products run
+            ti = fetch_slot(&slots[cur ^ 1], tasks, ntasks, tile + gridDim.x, ti);
+            fetched = true;
+          }
+          if (s + 1 == nst || (MULTI && (s & (CHUNK - 1)) == CHUNK - 1)) {
+            // all products up to this step are done
+            if (!mbar_wait(&bar[h], use & 1u, err, 12, wait_ns)) abort = true;
             fence_after();
-            if (mine) {
+            if (MULTI && mine) {
 #pragma unroll
-              for (int cb = 0; cb < 16; cb += 2) {
-                uint32_t v[8][2];
-                const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + colq * 16 + cb;
-#pragma unroll
-                for (int g = 0; g < 8; ++g) tmem_ld2(ta + g * TN, v[g]);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                  int c[8];
-#pragma unroll
-                  for (int g = 0; g < 8; ++g) c[g] = __float2int_rn(__uint_as_float(v[g][j]));
-                  ahi[cb + j] += (long long)c[0] * (1 << 24) + (long long)c[1] * (1 << 16) + (long long)c[2] * 256 + c[3];
-                  alo[cb + j] += (long long)c[4] * (1 << 24) + (long long)c[5] * (1 << 16) + (long long)c[6] * 256 + c[7];
-                }
-              }
+              for (int cb = 0; cb < 16; cb += 2) drain2(cb, ahi + (MULTI ? cb : 0), alo + (MULTI ? cb : 0));
             }
-            fence_before();
+            if (MULTI) fence_before();
+          }
+          ++it;
+          return true;
+        };
+        if (!PAIR) {
+          for (int s = 0; s < nst; ++s)
+            if (!step(s, v0)) { abort = true; break; }
+        } else {
+          for (int s = 0; s < nst; s += 2) {
+            if (!step(s, v0)) { abort = true; break; }
+            if (s + 1 < nst && !step(s + 1, v1)) { abort = true; break; }
           }
         }
-        abort = __syncthreads_or(abort);
-        if (abort) break;
+        // A warp holds 32 rows (one a lane) of 16 columns.  Where rows are
+        // contiguous in memory it stores them column by column; else it turns
+        // its piece in shared memory (its own part: the products are done) and
+        // stores two rows of 16 columns at a time, instead of 32 rows of one.
         if (mine) {
-          const int exr = (int)(rmax[quarter * 32 + lane] >> 20);
+          const int exr = scale_exp(rscale[orow]);
+          const bool lanes = T.cxs == 1;
+          double* r = C + (orow < nx ? roff[orow] : 0);
+          double* st = (double*)smem + warp * (32 * 17);
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            stg[(quarter * 32 + lane) * STG_LD + colq * 16 + j] =
-                to_f64(ahi[j], alo[j], exr + (int)(rmax[TM + colq * 16 + j] >> 20));
+          for (int cb = 0; cb < 16; cb += 2) {
+            long long hi[2], lo[2];
+            if (MULTI) {
+#pragma unroll
+              for (int j = 0; j < 2; ++j) { hi[j] = ahi[cb + j]; lo[j] = alo[cb + j]; }
+            } else {
+              hi[0] = hi[1] = lo[0] = lo[1] = 0;
+              if (nst > 0) drain2(cb, hi, lo);
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const int col = colq * 16 + cb + j;
+              const double x = to_f64(hi[j], lo[j], exr + scale_exp(rscale[TM + col]));
+              if (!lanes) st[lane * 17 + cb + j] = x;
+              else if (col < ny && orow < nx) put(T, pm, r + coff[col], x);
+            }
+          }
+          if (!lanes) {
+            __syncwarp();
+            const int col = colq * 16 + (lane & 15);
+            double* c = C + (col < ny ? coff[col] : 0);
+#pragma unroll 4
+            for (int i = lane >> 4; i < 32; i += 2) {
+              const int row = quarter * 32 + i;
+              if (row < nx && col < ny) put(T, pm, c + roff[row], st[i * 17 + (lane & 15)]);
+            }
+          }
         }
+        if (!MULTI) fence_before();
       } else {
+        const double* X = T.x + (long long)slots[cur].b * T.xub;
+        const double* Y = T.y + (long long)slots[cur].b * T.yub;
         for (int e = tid; e < nx * ny; e += THREADS) {
           const int i = e / ny, j = e - i * ny;
           const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
           const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
           double s = 0.0;
-          for (int k = 0; k < len; ++k) s = fma(px[tab[k] * T.xks], py[tab[k] * T.yks], s);
-          stg[i * STG_LD + j] = s;
+          for (int k = 0; k < len; ++k) {
+            const int col = T.kr ? tab[k] : kb + k;
+            s = fma(px[(long long)col * T.xks], py[(long long)col * T.yks], s);
+          }
+          put(T, pm, C + roff[i] + coff[j], s);
         }
       }
-      __syncthreads();
-      // write-out along the direction that is contiguous in memory
-      const int pm = put_mode(T, kb == k0);
-      if (T.cys == 1) {
-        const bool o0 = lane < ny, o1 = lane + 32 < ny;
-        const long long c0 = o0 ? row_off(y0 + lane, T.ny, 1, T.cyb) : 0;
-        const long long c1 = o1 ? row_off(y0 + lane + 32, T.ny, 1, T.cyb) : 0;
-        for (int i = warp; i < nx; i += THREADS / 32) {
-          double* r = C + row_off(x0 + i, T.nx, T.cxs, T.cxb);
-          if (o0) put(T, pm, r + c0, stg[i * STG_LD + lane]);
-          if (o1) put(T, pm, r + c1, stg[i * STG_LD + lane + 32]);
-        }
-      } else {
-        for (int i0 = 0; i0 < nx; i0 += 32) {
-          const int i = i0 + lane;
-          const long long ci = i < nx ? row_off(x0 + i, T.nx, T.cxs, T.cxb) : 0;
-          for (int j = warp; j < ny; j += THREADS / 32)
-            if (i < nx) put(T, pm, C + ci + row_off(y0 + j, T.ny, T.cys, T.cyb), stg[i * STG_LD + j]);
-        }
+      if (warp == 1 && next && !fetched && kb + KB >= k1) {
+        ti = fetch_slot(&slots[cur ^ 1], tasks, ntasks, tile + gridDim.x, ti);
+        fetched = true;
       }
-      __syncthreads();
+      abort = __syncthreads_or(abort);
       kb += KB;
-    } while (kb < k1);
+    } while (kb < k1 && !abort);
   }
   if (abort && tid == 0) {
     // products already issued read shared and tensor memory: wait for them
@@ -420,20 +581,85 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   fence_after();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(8 * TN) : "memory");
 }
 
 // ---------------------------------------------------------------------------
 // FP64-pipe kernel: 32 x 32 output tiles, outputs dense over the threads (no
-// multiply-add is issued for padding), each summed in ascending K.
+// multiply-add is issued for padding), or thin tiles; each output is summed in
+// ascending K.  (One warp a tile without shared memory, 32 of them on an SM,
+// measured slower: 18.9 against 15.5 ms over the energies at M1 = 400, and 3x
+// on long sums of few outputs, whose loads then lie on the chain.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gemm_f64_small_kernel(const F64Task* __restrict__ tasks, int ntasks,
+constexpr int SM_T = 32, THIN_X = 8, THIN_Y = 256, THIN_K = 64;
+
+// A tile of up to 8 rows of X (kept in shared memory) and 256 rows of Y, one a
+// thread: Y is read once, coalesced where its rows are contiguous.  Sums of a
+// few matrices with coefficients (the operators' dense blocks) are of this
+// form: 8 x k multiply-adds per value read.  As 128-row tensor-core tiles 2 %
+// full they took 35 of the energies' 88 ms at M1 = 400.
+template <int N>
+__device__ __forceinline__ void thin_sum(const double* xs, const double* y, long long yks, const int* kcol, int nk,
+                                         double (&acc)[THIN_X]) {
+#pragma unroll 4
+  for (int q = 0; q < nk; ++q) {
+    const double v = __ldg(y + (long long)kcol[q] * yks);
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = fma(xs[q * THIN_X + i], v, acc[i]);
+  }
+}
+
+__device__ __forceinline__ void thin_tile(const F64Task& T, const F64Tile& tc, double* xs, int* kcol) {
+  const int tid = threadIdx.x;
+  const int x0 = tc.ix * THIN_X, y0 = tc.iy * THIN_Y;
+  const int nx = min(THIN_X, T.mx - x0), ny = min(THIN_Y, T.my - y0);
+  const int k0 = tc.ks * T.kchunk, k1 = min(T.k, k0 + T.kchunk);
+  const double* X = T.x + (long long)tc.b * T.xub;
+  double* C = T.c + (long long)tc.b * T.cub + (long long)tc.ks * T.sK;
+  const bool ok = tid < ny;
+  const double* y = T.y + (long long)tc.b * T.yub + (ok ? row_off(y0 + tid, T.ny, T.yrs, T.ybs) : 0);
+  double acc[THIN_X];
+#pragma unroll
+  for (int i = 0; i < THIN_X; ++i) acc[i] = 0.0;
+  for (int kk = k0; kk < k1; kk += THIN_K) {
+    const int nk = min(THIN_K, k1 - kk);
+    if (tid < nk) kcol[tid] = k_col(T, kk + tid);
+    __syncthreads();
+    for (int e = tid; e < nk * THIN_X; e += 256) {
+      const int q = e / THIN_X, i = e - q * THIN_X;
+      xs[e] = i < nx ? X[row_off(x0 + i, T.nx, T.xrs, T.xbs) + (long long)kcol[q] * T.xks] : 0.0;
+    }
+    __syncthreads();
+    if (ok) {
+      if (nx == 1) thin_sum<1>(xs, y, T.yks, kcol, nk, acc);
+      else if (nx == 2) thin_sum<2>(xs, y, T.yks, kcol, nk, acc);
+      else if (nx <= 4) thin_sum<4>(xs, y, T.yks, kcol, nk, acc);
+      else thin_sum<8>(xs, y, T.yks, kcol, nk, acc);
+    }
+    __syncthreads();
+  }
+  if (!ok) return;
+  const int pm = put_mode(T, true);
+  const long long c = row_off(y0 + tid, T.ny, T.cys, T.cyb);
+#pragma unroll
+  for (int i = 0; i < THIN_X; ++i)
+    if (i < nx) put(T, pm, C + row_off(x0 + i, T.nx, T.cxs, T.cxb) + c, acc[i]);
+}
+
+__global__ void __launch_bounds__(256) gemm_f64_pipe_kernel(const F64Task* __restrict__ tasks, int ntasks,
                                                              long long total) {
   __shared__ double xs[SM_T][SM_T + 1], ys[SM_T][SM_T + 1];   // [k][row]
+  __shared__ int kcol[THIN_K];
   const int tid = threadIdx.x;
+  int ti = 0;
   for (long long tile = blockIdx.x; tile < total; tile += gridDim.x) {
-    const F64Task T = tasks[find_f64(tasks, ntasks, tile)];
+    ti = warp_find(tasks, ntasks, tile, ti);
+    const F64Task T = tasks[ti];
     const F64Tile tc = tile_of(T, tile);
+    if (T.thin) {
+      thin_tile(T, tc, &xs[0][0], kcol);
+      continue;
+    }
     const int x0 = tc.ix * SM_T, y0 = tc.iy * SM_T;
     const int nx = min(SM_T, T.mx - x0), ny = min(SM_T, T.my - y0);
     const int k0 = tc.ks * T.kchunk, k1 = min(T.k, k0 + T.kchunk);
@@ -496,143 +722,219 @@ inline long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
 
 }  // namespace
 
-// A task in the kernels' form.  A batch that shares one operand becomes rows
-// of the other (their tiles then fill up whatever the batch's own size), and
-// the operand with more rows lies along the tile's long side.
-static F64Task make_f64_task(const GemmTask& g) {
+// Rows and K of a task in the kernels' form.  A batch that shares one operand
+// becomes rows of the other (their tiles then fill up whatever the batch's own
+// size): fold 1 along A's rows, 2 along B's.
+struct F64Dims {
+  long long ma, mb;   // rows of op(A), columns of op(B), folded
+  int fold, k, kc, batch, ksplit;
+};
+static F64Dims f64_dims(const GemmTask& g) {
+  F64Dims d;
+  const long long big = 1LL << 30;
+  d.ma = g.m;
+  d.mb = g.n;
+  d.batch = g.batch;
+  d.fold = 0;
+  if (g.batch > 1 && g.sB == 0 && g.batch * d.ma < big) { d.fold = 1; d.ma *= g.batch; d.batch = 1; }
+  else if (g.batch > 1 && g.sA == 0 && g.batch * d.mb < big) { d.fold = 2; d.mb *= g.batch; d.batch = 1; }
+  d.k = g.kr ? g.kv : g.k;
+  d.ksplit = std::max(1, g.ksplit);
+  d.kc = (int)(cdiv(cdiv(std::max(d.k, 1), d.ksplit), 16) * 16);
+  return d;
+}
+
+// How a task runs on the FP64 pipe or on the tensor cores: its operands as given
+// or exchanged, with the estimated SM clocks of the whole task and the longest
+// tile.
+struct F64Form {
+  double clocks, tile;
+  int swap, bx, by;   // exchanged operands; tile
+  bool thin;
+};
+
+// A multiply-add instruction of the FP64 pipe takes 16 clocks a warp whatever
+// its operands.
+static F64Form pipe_form(const F64Dims& d) {
+  const double kc = std::max(1, std::min(d.k, d.kc));
+  const double reps = (double)d.batch * d.ksplit;
+  const double o = (double)std::min<long long>(d.ma, SM_T) * std::min<long long>(d.mb, SM_T);
+  const double sq = 700.0 + (300.0 / SM_T) * (kc + SM_T) + 0.5 * kc * (o + 31.0);
+  F64Form f{sq * reps * cdiv(d.ma, SM_T) * cdiv(d.mb, SM_T), sq, 0, SM_T, SM_T, false};
+  for (int w = 0; w < 2; ++w) {
+    const long long x = w ? d.mb : d.ma, y = w ? d.ma : d.mb;
+    const int n = x == 1 ? 1 : (x == 2 ? 2 : (x <= 4 ? 4 : 8));
+    const double t = 400.0 + std::max(0.5 * kc * n * (std::min<long long>(y, THIN_Y) + 31), 60.0 * (kc + n));
+    const double all = t * reps * cdiv(x, THIN_X) * cdiv(y, THIN_Y);
+    if (all < f.clocks) f = {all, t, w, THIN_X, THIN_Y, true};
+  }
+  return f;
+}
+
+// Tensor-core tile: set-up, a step's products and barriers, the cutting of its
+// rows' digits, the drain and the write-out of its 32 x 16 pieces.  Measured
+// with clocks on the device at K = 56, M1 = 500: about 45000 a full tile of 128
+// x 64.
+static F64Form tc_form(const F64Dims& d, const GemmTask& g, int tn) {
+  const double kc = std::max(1, std::min(d.k, d.kc)), steps = (double)(((long long)kc + KS - 1) / KS);
+  F64Form best{1e300, 0, 0, TM, tn, false};
+  for (int w = 0; w < 2; ++w) {
+    const long long x = w ? d.mb : d.ma, y = w ? d.ma : d.mb;
+    const double tx = (double)cdiv(x, TM), ty = (double)cdiv(y, tn);
+    const double px = 0.5 + x / 32.0, py = 0.5 + y / 16.0;   // pieces along each side, all tiles
+    const bool lanes = (w ? 1 : g.ldc) == 1;                  // rows contiguous in memory
+    const double tile = tn == 64 ? 8500.0 + 4200.0 * steps : 4500.0 + 2200.0 * steps;
+    const double rows = steps * (steps > 1 ? 140.0 : 80.0) * (ty * x + tx * y) / 8.0;
+    const double out = px * py * (330.0 * ((long long)(kc / 128) + 1) + (lanes ? 300.0 : 450.0));
+    const double all = (tx * ty * tile + rows + out) * d.batch * d.ksplit;
+    if (all < best.clocks) best = {all, tile, w, TM, tn, false};
+  }
+  return best;
+}
+
+static bool is_long(const F64Dims& d) { return std::min(d.k, d.kc) > KS * CHUNK; }
+
+static F64Task make_task(const GemmTask& g, const F64Dims& d, const F64Form& f) {
   F64Task t;
   std::memset(&t, 0, sizeof(t));
   const bool ta = g.flags & GEMM_TA, tb = g.flags & GEMM_TB;
   t.x = g.A; t.y = g.B; t.c = g.C;
   t.xrs = ta ? 1 : g.lda; t.xks = ta ? g.lda : 1;
   t.yrs = tb ? g.ldb : 1; t.yks = tb ? 1 : g.ldb;
-  t.nx = t.mx = g.m;
-  t.ny = t.my = g.n;
+  t.nx = g.m; t.mx = (int)d.ma;
+  t.ny = g.n; t.my = (int)d.mb;
   t.cxs = g.ldc; t.cys = 1;
-  t.batch = g.batch;
-  const long long big = 1LL << 30;
-  if (g.batch > 1 && g.sB == 0 && (long long)g.batch * g.m < big) {
-    t.mx = g.batch * g.m; t.xbs = g.sA; t.cxb = g.sC; t.batch = 1;
-  } else if (g.batch > 1 && g.sA == 0 && (long long)g.batch * g.n < big) {
-    t.my = g.batch * g.n; t.ybs = g.sB; t.cyb = g.sC; t.batch = 1;
-  } else {
-    t.xub = g.sA; t.yub = g.sB; t.cub = g.sC;
-  }
-  t.k = g.kr ? g.kv : g.k;
+  t.batch = d.batch;
+  if (d.fold == 1) { t.xbs = g.sA; t.cxb = g.sC; }
+  else if (d.fold == 2) { t.ybs = g.sB; t.cyb = g.sC; }
+  else { t.xub = g.sA; t.yub = g.sB; t.cub = g.sC; }
+  t.k = d.k;
   t.kr = g.kr;
   t.nkr = g.nkr;
   t.alpha = g.alpha;
   t.beta = g.beta;
-  t.ksplit = std::max(1, g.ksplit);
+  t.ksplit = d.ksplit;
   MPSLCC_REQUIRE(t.ksplit == 1 || g.sK > 0, ST_INTERNAL, "FP64 task split over K without partial offsets");
   t.sK = t.ksplit > 1 ? g.sK : 0;
-  t.kchunk = (int)(cdiv(cdiv(std::max(t.k, 1), t.ksplit), 16) * 16);
-  if (cdiv(t.my, TM) * cdiv(t.mx, TN) < cdiv(t.mx, TM) * cdiv(t.my, TN)) {
+  t.kchunk = d.kc;
+  if (f.swap) {
     std::swap(t.x, t.y);
     std::swap(t.xrs, t.yrs); std::swap(t.xks, t.yks); std::swap(t.xbs, t.ybs); std::swap(t.xub, t.yub);
     std::swap(t.nx, t.ny); std::swap(t.mx, t.my);
     std::swap(t.cxs, t.cys); std::swap(t.cxb, t.cyb);
   }
+  t.thin = f.thin;
+  t.tx = (int)cdiv(t.mx, f.bx);
+  t.ty = (int)cdiv(t.my, f.by);
   return t;
-}
-
-// Estimated SM clocks of a task's largest tile: a multiply-add instruction of
-// the FP64 pipe takes 16 clocks a warp; a tensor-core tile takes about 4000
-// for its set-up and write-out, 2400 a step of 32 K values and 1500 a drain
-// whatever part of it is used.
-static double pipe_clocks(const F64Task& t) {
-  const long long kc = std::max(1, std::min(t.k, t.kchunk));
-  return 1500.0 + 600.0 * cdiv(kc, SM_T) +
-         16.0 * kc * cdiv(std::min<long long>(t.mx, SM_T) * std::min<long long>(t.my, SM_T), 32);
-}
-static double tc_clocks(const F64Task& t) {
-  const long long kc = std::max(1, std::min(t.k, t.kchunk));
-  return 4000.0 * cdiv(kc, KB) + 2400.0 * cdiv(kc, KS) + 1500.0 * cdiv(kc, KS * CHUNK);
-}
-static long long tiles_of(const F64Task& t, int bx, int by) {
-  return (long long)t.batch * t.ksplit * cdiv(t.mx, bx) * cdiv(t.my, by);
 }
 
 // A launch whose multiply-adds keep the FP64 pipes busy for no longer than a
 // tensor-core launch takes to fill and drain (about 10 us; 30 us for the
 // longest tile) runs there whole: one launch instead of two, and its sums are
 // plain FP64 chains.
-static bool pipe_launch(const std::vector<F64Task>& t) {
-  double sum = 0;
-  for (const auto& x : t) {
-    const double c = pipe_clocks(x);
-    if (c > 60e3) return false;
-    sum += c * tiles_of(x, SM_T, SM_T);
+static bool short_launch(double clocks, double longest) { return clocks <= 152 * 20e3 && longest <= 60e3; }
+
+static bool f64_empty(const GemmTask& g) { return g.m <= 0 || g.n <= 0 || g.batch <= 0; }
+
+bool f64_on_pipe(const GemmTask* g, int n) {
+  double sum = 0, longest = 0;
+  for (int i = 0; i < n; ++i) {
+    if (f64_empty(g[i])) continue;
+    const F64Form f = pipe_form(f64_dims(g[i]));
+    sum += f.clocks;
+    longest = std::max(longest, f.tile);
   }
-  return sum <= 152 * 20e3;
+  return short_launch(sum, longest);
 }
 
-static std::vector<F64Task> f64_tasks(const GemmTask* g, int n) {
-  std::vector<F64Task> v;
-  v.reserve(n);
-  for (int i = 0; i < n; ++i)
-    if (g[i].m > 0 && g[i].n > 0 && g[i].batch > 0) v.push_back(make_f64_task(g[i]));
-  return v;
-}
-
-bool f64_on_pipe(const GemmTask* g, int n) { return pipe_launch(f64_tasks(g, n)); }
-
-// Splits a task list between the two kernels (the one with fewer estimated
-// clocks over the task's tiles) and fills the tile counts.
+// Splits a task list between the kernels, by estimated clocks, and fills the
+// tile counts.  The short sums of a launch share one tile shape; long ones take
+// 128 x 32 (two CTAs per SM overlap the cutting and the drains: 2.8 against 3.4
+// ms for phase 2 of the M1 = 500 sigma, K = 2900).
 void plan_f64(const GemmTask* g, int n, F64Plan& p) {
   p = F64Plan();
-  const std::vector<F64Task> v = f64_tasks(g, n);
-  const bool all_small = pipe_launch(v);
-  for (F64Task t : v) {
-    const bool small =
-        all_small || pipe_clocks(t) * tiles_of(t, SM_T, SM_T) <= tc_clocks(t) * tiles_of(t, TM, TN);
-    const int bx = small ? SM_T : TM, by = small ? SM_T : TN;
-    t.tx = (int)cdiv(t.mx, bx);
-    t.ty = (int)cdiv(t.my, by);
-    long long& tot = small ? p.tiles_small : p.tiles_tc;
-    t.tile0 = tot;
-    tot += (long long)t.batch * t.ksplit * t.tx * t.ty;
-    (small ? p.small : p.tc).push_back(t);
+  struct Opt { F64Dims d; F64Form pipe, tc[2]; };
+  std::vector<Opt> o((size_t)n);
+  double sum = 0, longest = 0, cost[2] = {0, 0};
+  for (int i = 0; i < n; ++i) {
+    if (f64_empty(g[i])) continue;
+    o[i].d = f64_dims(g[i]);
+    o[i].pipe = pipe_form(o[i].d);
+    sum += o[i].pipe.clocks;
+    longest = std::max(longest, o[i].pipe.tile);
   }
-  p.n_tc = (int)p.tc.size();
-  p.n_small = (int)p.small.size();
+  const bool all_pipe = short_launch(sum, longest);
+  if (!all_pipe) {
+    for (int i = 0; i < n; ++i) {
+      if (f64_empty(g[i])) continue;
+      for (int w = 0; w < 2; ++w) {
+        o[i].tc[w] = tc_form(o[i].d, g[i], w || is_long(o[i].d) ? 32 : 64);
+        cost[w] += std::min(o[i].pipe.clocks, o[i].tc[w].clocks);
+      }
+    }
+    p.tn = cost[1] < cost[0] ? 32 : 64;
+  }
+  const int w = p.tn == 32 ? 1 : 0;
+  for (int i = 0; i < n; ++i) {
+    if (f64_empty(g[i])) continue;
+    const bool pipe = all_pipe || o[i].pipe.clocks <= o[i].tc[w].clocks;
+    const int list = pipe ? F64_PIPE : (is_long(o[i].d) ? F64_LONG : F64_SHORT);
+    F64Task t = make_task(g[i], o[i].d, pipe ? o[i].pipe : o[i].tc[w]);
+    t.tile0 = p.tiles[list];
+    p.tiles[list] += (long long)t.batch * t.ksplit * t.tx * t.ty;
+    p.t[list].push_back(t);
+  }
+  for (int l = 0; l < F64_LISTS; ++l) p.n[l] = (int)p.t[l].size();
 }
 
-size_t f64_plan_bytes(const F64Plan& p) { return (p.tc.size() + p.small.size()) * sizeof(F64Task); }
+size_t f64_plan_bytes(const F64Plan& p) {
+  size_t n = 0;
+  for (const auto& l : p.t) n += l.size();
+  return n * sizeof(F64Task);
+}
 
 // Copies the plan's tasks to device memory at d (f64_plan_bytes of it).
 void upload_f64(const F64Plan& p, void* d, cudaStream_t s) {
-  if (!p.tc.empty())
-    cuda_check(cudaMemcpyAsync(d, p.tc.data(), p.tc.size() * sizeof(F64Task), cudaMemcpyHostToDevice, s),
-               "upload FP64 tasks");
-  if (!p.small.empty())
-    cuda_check(cudaMemcpyAsync((char*)d + p.tc.size() * sizeof(F64Task), p.small.data(),
-                               p.small.size() * sizeof(F64Task), cudaMemcpyHostToDevice, s),
-               "upload FP64 tasks");
+  for (const auto& l : p.t) {
+    if (l.empty()) continue;
+    cuda_check(cudaMemcpyAsync(d, l.data(), l.size() * sizeof(F64Task), cudaMemcpyHostToDevice, s), "upload FP64 tasks");
+    d = (char*)d + l.size() * sizeof(F64Task);
+  }
+}
+
+template <int TN, bool MULTI>
+static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, int sms, int* err, cudaStream_t s) {
+  using F = F64Cfg<TN>;
+  static std::atomic<bool> attr[MAX_DEV];
+  MPSLCC_REQUIRE(device >= 0 && device < MAX_DEV, ST_ARG, "device ordinal out of range");
+  if (!attr[device].load(std::memory_order_acquire)) {
+    cuda_check(cudaFuncSetAttribute(gemm_f64_tc_kernel<TN, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    f64_smem<F>()),
+               "smem attr");
+    attr[device].store(true, std::memory_order_release);
+  }
+  const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, sms) * F::CTAS);
+  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F>(), s>>>(d, n, tiles, err, WAIT_NS);
 }
 
 int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s) {
-  int n = 0;
-  MPSLCC_REQUIRE((l.tiles_tc > 0) == (l.n_tc > 0) && (l.tiles_small > 0) == (l.n_small > 0), ST_INTERNAL,
-                 "FP64 task list without its counts");
-  if (l.tiles_tc > 0) {
-    static std::atomic<bool> attr[MAX_DEV];
-    MPSLCC_REQUIRE(device >= 0 && device < MAX_DEV, ST_ARG, "device ordinal out of range");
-    if (!attr[device].load(std::memory_order_acquire)) {
-      cuda_check(cudaFuncSetAttribute(gemm_f64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_TC),
-                 "smem attr");
-      attr[device].store(true, std::memory_order_release);
-    }
-    const int grid = (int)std::min<long long>(l.tiles_tc, std::max(1, sms));
-    gemm_f64_tc_kernel<<<grid, THREADS, SMEM_TC, s>>>((const F64Task*)d, l.n_tc, l.tiles_tc, err, WAIT_NS);
-    ++n;
+  int launches = 0;
+  const F64Task* t = (const F64Task*)d;
+  for (int i = 0; i < F64_LISTS; ++i) {
+    const int n = l.n[i];
+    const long long tiles = l.tiles[i];
+    MPSLCC_REQUIRE((tiles > 0) == (n > 0), ST_INTERNAL, "FP64 task list without its counts");
+    if (n == 0) continue;
+    if (i == F64_PIPE)
+      gemm_f64_pipe_kernel<<<(int)std::min<long long>(tiles, 152LL * 8), 256, 0, s>>>(t, n, tiles);
+    else if (i == F64_SHORT && l.tn == 32) launch_f64_tc<32, false>(t, n, tiles, device, sms, err, s);
+    else if (i == F64_SHORT) launch_f64_tc<64, false>(t, n, tiles, device, sms, err, s);
+    else launch_f64_tc<32, true>(t, n, tiles, device, sms, err, s);
+    t += n;
+    ++launches;
   }
-  if (l.tiles_small > 0) {
-    const int grid = (int)std::min<long long>(l.tiles_small, 152LL * 8);
-    gemm_f64_small_kernel<<<grid, 256, 0, s>>>((const F64Task*)d + l.n_tc, l.n_small, l.tiles_small);
-    ++n;
-  }
-  return n;
+  return launches;
 }
 
 }  // namespace mpslcc

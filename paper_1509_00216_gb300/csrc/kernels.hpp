@@ -58,18 +58,20 @@ struct F64Task {
   double alpha, beta;
   int nx, mx, ny, my, k, ksplit, kchunk, batch;
   const int* kr;
-  int nkr, tx, ty;
+  int nkr, tx, ty, thin;
   long long tile0;
 };
 
-// Task lists of one launch pair: tensor-core tasks first, then the small
-// ones that run on the FP64 pipe.
+// Task lists of one grouped product, one launch each: sums of up to 128 K
+// values on the tensor cores, longer ones, and those on the FP64 pipe.
+enum { F64_SHORT, F64_LONG, F64_PIPE, F64_LISTS };
 struct F64Launch {
-  int n_tc = 0, n_small = 0;
-  long long tiles_tc = 0, tiles_small = 0;
+  int n[F64_LISTS] = {0, 0, 0};
+  long long tiles[F64_LISTS] = {0, 0, 0};
+  int tn = 64;               // columns of a short sum's tile: 64 or 32 (long sums: 32)
 };
 struct F64Plan : F64Launch {
-  std::vector<F64Task> tc, small;
+  std::vector<F64Task> t[F64_LISTS];
 };
 // Whether a launch of these tasks is so short that it runs on the FP64 pipe whole.
 bool f64_on_pipe(const GemmTask* g, int n);

@@ -73,6 +73,19 @@ __device__ __forceinline__ uint64_t sdesc(const void* p) {
   return d;
 }
 
+// The same for rows of ROW = 128 bytes, or of 64 bytes with 64-byte swizzle
+// (8-row groups of 512 bytes).
+template <int ROW>
+__device__ __forceinline__ uint64_t sdesc_k(const void* p) {
+  static_assert(ROW == 128 || ROW == 64, "operand row bytes");
+  uint64_t d = ((uint64_t)smem_u32(p) >> 4) & 0x3FFFull;
+  d |= 1ull << 16;
+  d |= (uint64_t)(8 * ROW >> 4) << 32;
+  d |= 1ull << 46;
+  d |= (ROW == 128 ? 2ull : 4ull) << 61;   // SWIZZLE_128B or SWIZZLE_64B
+  return d;
+}
+
 template <int PREC>
 __device__ __forceinline__ uint32_t idesc(int M, int N) {
   uint32_t f = PREC == MPSLCC_BF16 ? 1u : 2u;  // BF16 or TF32 operands
@@ -82,6 +95,11 @@ __device__ __forceinline__ uint32_t idesc(int M, int N) {
   d |= (uint32_t)(N >> 3) << 17;
   d |= (uint32_t)(M >> 4) << 24;
   return d;
+}
+
+// FP16 operands, FP32 accumulator (issued by umma<MPSLCC_BF16>: the same kind::f16).
+__device__ __forceinline__ uint32_t idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 template <int PREC>
