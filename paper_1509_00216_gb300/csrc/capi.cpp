@@ -140,11 +140,24 @@ mpslcc_status mpslcc_create(mpslcc_ctx** out, const mpslcc_opts* opts) {
     }
     MPSLCC_REQUIRE(cusolverDnCreate(&c.solver) == CUSOLVER_STATUS_SUCCESS, ST_CUDA, "cusolverDnCreate failed");
     cusolverDnSetStream(c.solver, c.stream);
-    int* flag = nullptr;
-    cuda_check(cudaHostAlloc((void**)&flag, sizeof(int), cudaHostAllocMapped), "flag");
-    *flag = 0;
-    c.f64_flag = flag;
-    cuda_check(cudaHostGetDevicePointer((void**)&c.f64_flag_dev, flag, 0), "flag address");
+    Ctx::HostOut* out = nullptr;
+    cuda_check(cudaHostAlloc((void**)&out, sizeof(*out), cudaHostAllocMapped), "host results");
+    std::memset(out, 0, sizeof(*out));
+    c.out = out;
+    cuda_check(cudaHostGetDevicePointer((void**)&c.out_dev, out, 0), "host results address");
+    if (!c.opts.alloc) {
+      // The context's own pool.  It keeps up to 4 GiB between synchronisations
+      // (the device's default pool keeps nothing: every buffer of every step was
+      // mapped anew) and is given back with the context.
+      cudaMemPoolProps props;
+      std::memset(&props, 0, sizeof(props));
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = c.device;
+      cuda_check(cudaMemPoolCreate(&c.pool, &props), "memory pool");
+      unsigned long long keep = 4ull << 30;
+      cuda_check(cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &keep), "memory pool threshold");
+    }
     for (cudaEvent_t* e : {&c.ev0, &c.ev1, &c.ev_p0, &c.ev_p1, &c.ev_p2}) cuda_check(cudaEventCreate(e), "event");
   });
   if (st != MPSLCC_OK) {
@@ -169,7 +182,7 @@ mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
     c.ofam.clear();
     for (auto& b : c.boxes) b.release();
     for (DBuf* b : {&c.red, &c.red_out, &c.red_ticket, &c.gtask, &c.ctask, &c.eig_work, &c.eig_w, &c.eig_info, &c.scratch_a,
-                    &c.scratch_b, &c.scratch_tc, &c.tc_conv_tasks, &c.tc_gemm_tasks, &c.tc_err})
+                    &c.scratch_b, &c.scratch_tc, &c.tc_conv_tasks, &c.tc_gemm_tasks})
       b->release();
     for (int s = 0; s < Ctx::NEIG; ++s) c.eig_ws[s].release();
     cudaStreamSynchronize(c.stream);
@@ -179,7 +192,7 @@ mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
       if (c.eig_ev[s]) cudaEventDestroy(c.eig_ev[s]);
     }
     if (c.eig_fork) cudaEventDestroy(c.eig_fork);
-    if (c.f64_flag) cudaFreeHost((void*)c.f64_flag);
+    if (c.out) cudaFreeHost((void*)c.out);
     if (c.solver) cusolverDnDestroy(c.solver);
     for (cudaEvent_t e : {c.ev0, c.ev1, c.ev_p0, c.ev_p1, c.ev_p2})
       if (e) cudaEventDestroy(e);
@@ -187,6 +200,7 @@ mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
       cudaStreamDestroy(c.stream);
       c.stream = nullptr;   // a buffer released after this point is freed synchronously
     }
+    if (c.pool) cudaMemPoolDestroy(c.pool);   // goes away with its last buffer
   }
   delete ctx;
   return MPSLCC_OK;

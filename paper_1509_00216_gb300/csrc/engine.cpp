@@ -49,7 +49,14 @@ void DBuf::alloc(Ctx* ctx, size_t nbytes) {
     p = ctx->opts.alloc(nbytes, ctx->opts.alloc_user);
     if (!p) throw Error(ST_NOMEM, "device allocation failed (" + std::to_string(nbytes) + " bytes)");
   } else {
-    cudaError_t e = cudaMallocAsync(&p, nbytes, ctx->stream);
+    cudaError_t e = ctx->pool ? cudaMallocFromPoolAsync(&p, nbytes, ctx->pool, ctx->stream)
+                              : cudaMallocAsync(&p, nbytes, ctx->stream);
+    if (e != cudaSuccess && ctx->pool) {   // give back what the pool keeps, and try once more
+      cudaGetLastError();
+      cudaStreamSynchronize(ctx->stream);
+      cudaMemPoolTrimTo(ctx->pool, 0);
+      e = cudaMallocFromPoolAsync(&p, nbytes, ctx->pool, ctx->stream);
+    }
     if (e != cudaSuccess) {
       p = nullptr;
       bytes = 0;
@@ -60,33 +67,35 @@ void DBuf::alloc(Ctx* ctx, size_t nbytes) {
   ctx->allocs[(uintptr_t)p] = nbytes;
 }
 
+bool Ctx::live(uintptr_t a, uintptr_t b) const {
+  for (const Live& r : recent)
+    if (a >= r.a && b <= r.b) return true;
+  auto it = allocs.upper_bound(a);
+  if (it == allocs.begin()) return false;
+  --it;
+  if (b > it->first + it->second) return false;
+  recent[recent_next++ % recent.size()] = {it->first, it->first + it->second};
+  return true;
+}
+
 void Ctx::check_range(const void* ptr, long long first, long long last, const char* what) const {
   if (last < first) return;
   uintptr_t a = (uintptr_t)ptr + (uintptr_t)(first * 8), b = (uintptr_t)ptr + (uintptr_t)(last * 8 + 8);
   if (first < 0) a = (uintptr_t)ptr - (uintptr_t)(-first * 8);
-  auto it = allocs.upper_bound(a);
-  bool ok = false;
-  if (it != allocs.begin()) {
-    --it;
-    ok = a >= it->first && b <= it->first + it->second;
-  }
-  if (!ok) throw Error(ST_INTERNAL, std::string("device access out of bounds in ") + what);
+  if (!live(a, b)) throw Error(ST_INTERNAL, std::string("device access out of bounds in ") + what);
 }
 
 void Ctx::check_bytes(const void* ptr, long long nbytes, const char* what) const {
   if (nbytes <= 0) return;
   uintptr_t a = (uintptr_t)ptr, b = a + (uintptr_t)nbytes;
-  auto it = allocs.upper_bound(a);
-  bool ok = false;
-  if (it != allocs.begin()) {
-    --it;
-    ok = a >= it->first && b <= it->first + it->second;
-  }
-  if (!ok) throw Error(ST_INTERNAL, std::string("device access out of bounds in ") + what);
+  if (!live(a, b)) throw Error(ST_INTERNAL, std::string("device access out of bounds in ") + what);
 }
 
 void DBuf::release() {
-  if (p && c) c->allocs.erase((uintptr_t)p);
+  if (p && c) {
+    c->allocs.erase((uintptr_t)p);
+    c->recent.fill({0, 0});
+  }
   if (p && c) {
     if (c->opts.free) c->opts.free(p, bytes, c->opts.alloc_user);
     else if (c->stream || !c->own_stream) cudaFreeAsync(p, c->stream);
@@ -104,9 +113,7 @@ Fused fuse_left(const Sectors& b, const std::vector<int>& mask) {
   for (auto& kv : m) {
     int off = 0;
     for (auto& p : kv.second) { p.off = off; off += p.dim; }
-    f.q.push_back(kv.first);
-    f.d.push_back(off);
-    f.pc.push_back(kv.second);
+    f.add(kv.first, off, std::move(kv.second));
   }
   return f;
 }
@@ -119,9 +126,7 @@ Fused fuse_right(const std::vector<int>& mask, const Sectors& b) {
   for (auto& kv : m) {
     int off = 0;
     for (auto& p : kv.second) { p.off = off; off += p.dim; }
-    f.q.push_back(kv.first);
-    f.d.push_back(off);
-    f.pc.push_back(kv.second);
+    f.add(kv.first, off, std::move(kv.second));
   }
   return f;
 }
@@ -168,16 +173,16 @@ void run_gemms(Ctx& c, std::vector<GemmTask>& t) {
 
 void run_f64(Ctx& c, const F64Launch& l, const void* d) {
   const int sms = std::max(1, sm_count_dev(c.device) - std::max(0, c.tc_sm_reserve));
-  const int n = launch_f64(l, d, c.device, sms, c.f64_flag_dev, c.s());
+  const int n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s());
   cuda_check(cudaGetLastError(), "gemm_f64 launch");
   c.st.gemm_launches += n;
   c.st.kernel_launches += n;
 }
 
 void check_f64(Ctx& c) {
-  const int h = c.f64_flag ? *c.f64_flag : 0;
+  const int h = c.out ? c.out->flag[0] : 0;
   if (!h) return;
-  *c.f64_flag = 0;
+  c.out->flag[0] = 0;
   throw Error(ST_TIMEOUT, "FP64 product gave up waiting on an mbarrier (code " + std::to_string(h) + ")");
 }
 
@@ -210,14 +215,8 @@ static unsigned int* dot_ticket(Ctx& c) {
 }
 
 double dev_dot(Ctx& c, const double* x, const double* y, long n) {
-  if (n <= 0) return 0.0;
-  unsigned int* tk = dot_ticket(c);
-  launch_dot_fused(x, y, nullptr, nullptr, n, c.red_out.d(), c.red.d(), tk, c.s());
-  c.st.kernel_launches++;
-  double r = 0;
-  cuda_check(cudaMemcpyAsync(&r, c.red_out.p, sizeof(double), cudaMemcpyDeviceToHost, c.s()), "dot d2h");
-  cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
-  check_f64(c);
+  double r = 0, r2 = 0;
+  dev_dot2(c, x, y, nullptr, nullptr, n, &r, &r2);
   return r;
 }
 
@@ -226,14 +225,12 @@ void dev_dot2(Ctx& c, const double* x1, const double* y1, const double* x2, cons
   *r1 = *r2 = 0.0;
   if (n <= 0) return;
   unsigned int* tk = dot_ticket(c);
-  launch_dot_fused(x1, y1, x2, y2, n, c.red_out.d(), c.red.d(), tk, c.s());
+  launch_dot_fused(x1, y1, x2, y2, n, c.out_dev->red, c.red.d(), tk, c.s());
   c.st.kernel_launches++;
-  double r[2] = {0, 0};
-  cuda_check(cudaMemcpyAsync(r, c.red_out.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "dot d2h");
   cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
   check_f64(c);
-  *r1 = r[0];
-  *r2 = r[1];
+  *r1 = c.out->red[0];
+  if (x2) *r2 = c.out->red[1];
 }
 
 void dev_project(Ctx& c, const double* u, double* v, long n) {
@@ -410,18 +407,6 @@ std::vector<uint16_t> fused_piece_masks(const Mpo& W, int p, bool left) {
   std::vector<uint16_t> m((size_t)b.n, 0);
   for (const auto& e : W.site[p].e) m[left ? e.w1 : e.w0] |= (uint16_t)(1u << (4 * e.so + e.si));
   return m;
-}
-
-int piece_dim(const Fused& F, int f, int s) {
-  for (const auto& p : F.pc[f])
-    if (p.s == s || p.s < 0) return p.dim;
-  return 0;
-}
-
-int piece_off(const Fused& F, int f, int s) {
-  for (const auto& p : F.pc[f])
-    if (p.s == s || p.s < 0) return p.off;
-  return 0;
 }
 
 static std::vector<int> class_list(const MpoBond& b) {
@@ -852,9 +837,7 @@ static void make_right_env(Ctx& c, Family& F, int l, const std::vector<QN>& kbq,
   auto bond_space = [](const Sectors& s) {
     Fused f;
     for (int i = 0; i < s.size(); ++i) {
-      f.q.push_back(s.q[i]);
-      f.d.push_back(s.d[i]);
-      f.pc.push_back({Piece{i, -1, s.d[i], 0}});
+      f.add(s.q[i], s.d[i], {Piece{i, -1, s.d[i], 0}});
     }
     return f;
   };
@@ -942,11 +925,58 @@ void make_sigma_plan1(Ctx& c, Family& F, int l, SigmaPlan& P) {
   finish_sigma_plan(c, P);
 }
 
-// Intermediate buffers and the task lists of both sigma phases of a plan
-// whose fused left operator and right operator are in place.
+// Flops of a plan whose fused left operator and right operator are in place.
 static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
   const LeftFused& lf = P.lf;
   const RightFused& rf = P.rf;
+  P.f64_ready = false;
+  // Algorithmic flops: a channel's fused block is non-zero only on the local
+  // pieces (s_out, s_in) its site tensor reaches, so both phases count the
+  // block products piece by piece (and both the FP64 and the tensor-core
+  // tasks multiply only those pieces).
+  const Mpo& W = *P.fam->mpo;
+  const std::vector<uint16_t> mL = fused_piece_masks(W, lf.p, true);
+  const std::vector<uint16_t> mR = rf.ext ? std::vector<uint16_t>() : fused_piece_masks(W, rf.p, false);
+  // Sector pairs sum over runs of channels with equal masks.
+  auto class_flops = [&](const std::vector<uint16_t>& m, int c0, int nw, const Fused& Fb, int fb, const Fused& Fk, int fk) {
+    double f = 0;
+    for (int w = 0; w < nw;) {
+      const uint16_t mask = m[c0 + w];
+      int w1 = w + 1;
+      while (w1 < nw && m[c0 + w1] == mask) ++w1;
+      double g = 0;
+      for (int b = 0; b < 16; ++b)
+        if (mask >> b & 1) g += 2.0 * piece_dim(Fb, fb, b >> 2) * piece_dim(Fk, fk, b & 3);
+      f += g * (w1 - w);
+      w = w1;
+    }
+    return f;
+  };
+  double fl = 0;
+  for (const auto& S : rf.stk) {
+    const int fb = rf.kb[S.bidx], fk = rf.kk[S.kidx];
+    const double dl = lf.FLk.d[lf.kk[S.kidx]];
+    if (rf.ext) fl += 2.0 * S.nw * (double)rf.FRb.d[fb] * rf.FRk.d[fk] * dl;
+    else fl += dl * class_flops(mR, W.bond[rf.p].class_start[S.cls], S.nw, rf.FRb, fb, rf.FRk, fk);
+  }
+  for (size_t bi = 0; bi < P.mid_b.size(); ++bi) {
+    const double dr = rf.FRb.d[rf.kb[bi]];
+    for (const auto& sg : lf.seg[bi])
+      fl += dr * class_flops(mL, W.bond[lf.p + 1].class_start[sg.cls], sg.nw, lf.FLb, lf.kb[bi], lf.FLk, lf.kk[sg.kidx]);
+  }
+  P.flops = fl;
+  (void)c;
+}
+
+// Intermediate buffers and the task lists of both FP64 sigma phases, built
+// when a plan's first FP64 product needs them (the tensor-core products have
+// their own: T alone is some GB at M1 = 1500).
+static void prepare_f64_sigma(Ctx& c, SigmaPlan& P) {
+  const LeftFused& lf = P.lf;
+  const RightFused& rf = P.rf;
+  const Mpo& W = *P.fam->mpo;
+  const std::vector<uint16_t> mL = fused_piece_masks(W, lf.p, true);
+  const std::vector<uint16_t> mR = rf.ext ? std::vector<uint16_t>() : fused_piece_masks(W, rf.p, false);
   P.tt_off.assign(P.mid_b.size(), 0);
   long tts = 0;
   for (size_t bi = 0; bi < P.mid_b.size(); ++bi) {
@@ -961,38 +991,6 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
   P.xin.release();
   P.xin.alloc(&c, std::max(P.nk, 1L) * sizeof(double));
   std::vector<GemmTask> t1, t2;
-  // Algorithmic flops: a channel's fused block is non-zero only on the local
-  // pieces (s_out, s_in) its site tensor reaches, so both phases count the
-  // block products piece by piece (and both the FP64 and the tensor-core
-  // tasks multiply only those pieces).
-  const Mpo& W = *P.fam->mpo;
-  const std::vector<uint16_t> mL = fused_piece_masks(W, lf.p, true);
-  const std::vector<uint16_t> mR = rf.ext ? std::vector<uint16_t>() : fused_piece_masks(W, rf.p, false);
-  auto piece_flops = [](const Fused& Fb, int fb, const Fused& Fk, int fk, uint16_t mask, double other) {
-    double f = 0;
-    for (int b = 0; b < 16; ++b)
-      if (mask >> b & 1) f += 2.0 * piece_dim(Fb, fb, b >> 2) * piece_dim(Fk, fk, b & 3) * other;
-    return f;
-  };
-  double fl = 0;
-  for (const auto& S : rf.stk) {
-    const int fb = rf.kb[S.bidx], fk = rf.kk[S.kidx];
-    const double dl = lf.FLk.d[lf.kk[S.kidx]];
-    if (rf.ext) {
-      fl += 2.0 * S.nw * (double)rf.FRb.d[fb] * rf.FRk.d[fk] * dl;
-      continue;
-    }
-    const int c0 = W.bond[rf.p].class_start[S.cls];
-    for (int w = 0; w < S.nw; ++w) fl += piece_flops(rf.FRb, fb, rf.FRk, fk, mR[c0 + w], dl);
-  }
-  for (size_t bi = 0; bi < P.mid_b.size(); ++bi) {
-    const int fb = lf.kb[bi];
-    const double dr = rf.FRb.d[rf.kb[bi]];
-    for (const auto& sg : lf.seg[bi]) {
-      const int c0 = W.bond[lf.p + 1].class_start[sg.cls], fk = lf.kk[sg.kidx];
-      for (int w = 0; w < sg.nw; ++w) fl += piece_flops(lf.FLb, fb, lf.FLk, fk, mL[c0 + w], dr);
-    }
-  }
   // Phase 1: T_w^T = R'_w psi^T per unit — the rows of one R' stack with bra
   // local state so for a run of channels whose pieces (so, .) agree, batched
   // over those channels — summing only over the ket pieces the unit reaches
@@ -1166,7 +1164,6 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
                "upload split segments");
   for (const auto& x : t1) validate_gemm(c, x);
   for (const auto& x : t2) validate_gemm(c, x);
-  P.flops = fl;
   F64Plan p1, p2;
   plan_f64(t1.data(), (int)t1.size(), p1);
   plan_f64(t2.data(), (int)t2.size(), p2);
@@ -1179,6 +1176,7 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
   upload_f64(p1, P.tasks1.p, c.s());
   upload_f64(p2, P.tasks2.p, c.s());
   cuda_check(cudaStreamSynchronize(c.s()), "sigma plan sync");
+  P.f64_ready = true;
 }
 
 void sigma_apply(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
@@ -1186,6 +1184,7 @@ void sigma_apply(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
     tc_sigma(c, P, x, y, prec);
     return;
   }
+  if (!P.f64_ready) prepare_f64_sigma(c, P);
   if (P.nk > 0)
     cuda_check(cudaMemcpyAsync(P.xin.p, x, P.nk * sizeof(double), cudaMemcpyDeviceToDevice, c.s()), "sigma in");
   cudaEventRecord(c.ev_p0, c.s());

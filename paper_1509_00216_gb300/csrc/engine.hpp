@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cusolverDn.h>
 
+#include <array>
 #include <map>
 #include <memory>
 #include <string>
@@ -53,6 +54,19 @@ struct Fused {
   std::vector<QN> q;
   std::vector<int> d;
   std::vector<std::vector<Piece>> pc;
+  // per sector: dimension and offset of the piece of each local state (0 if it
+  // has none; a bare bond sector's one piece stands for every state)
+  std::vector<std::array<int, 4>> pd, po;
+  void add(const QN& key, int dim, std::vector<Piece> pieces) {
+    std::array<int, 4> dd{0, 0, 0, 0}, oo{0, 0, 0, 0};
+    for (const auto& p : pieces)
+      for (int s = p.s < 0 ? 0 : p.s; s <= (p.s < 0 ? 3 : p.s); ++s) { dd[s] = p.dim; oo[s] = p.off; }
+    q.push_back(key);
+    d.push_back(dim);
+    pc.push_back(std::move(pieces));
+    pd.push_back(dd);
+    po.push_back(oo);
+  }
   int find(const QN& x) const {
     auto it = std::lower_bound(q.begin(), q.end(), x);
     if (it == q.end() || !(*it == x)) return -1;
@@ -178,6 +192,7 @@ struct SigmaPlan {
   DBuf xin;
   DBuf tasks1, tasks2;
   F64Launch l1, l2;
+  bool f64_ready = false;              // the FP64 tasks and buffers are in place
   // FP64 phase 2: per-split partial products and the segments of their
   // fixed-order sum into sigma
   DBuf ypart, segs;
@@ -236,6 +251,11 @@ struct Ctx {
   // live device allocations (start -> bytes), used to validate every task's
   // address range on the host before a launch
   std::map<uintptr_t, size_t> allocs;
+  // the last few allocations that a check fell into (cleared when one goes away)
+  struct Live { uintptr_t a, b; };
+  mutable std::array<Live, 8> recent{};
+  mutable unsigned recent_next = 0;
+  bool live(uintptr_t a, uintptr_t b) const;
   void check_range(const void* p, long long first, long long last, const char* what) const;
   void check_bytes(const void* p, long long nbytes, const char* what) const;
 
@@ -246,10 +266,13 @@ struct Ctx {
   mpslcc_opts opts{};
   std::string err;
   cusolverDnHandle_t solver = nullptr;
-  // set (to a code) by an FP64 tensor-core product whose wait ran out; pinned
-  // host memory that the device writes, so that reading it costs no copy
-  volatile int* f64_flag = nullptr;
-  int* f64_flag_dev = nullptr;
+  // Pinned host memory that the device writes, so that reading it costs no copy:
+  // codes of FP64 [0] and other [1] tensor-core products whose wait ran out,
+  // and the results of reductions.
+  struct HostOut { int flag[2]; double red[256]; };
+  volatile HostOut* out = nullptr;
+  HostOut* out_dev = nullptr;
+  cudaMemPool_t pool = nullptr;   // of the stream-ordered allocations (no caller allocator)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_p0 = nullptr, ev_p1 = nullptr, ev_p2 = nullptr;
 
   // problem
@@ -314,7 +337,7 @@ struct Ctx {
   cudaEvent_t eig_ev[NEIG] = {}, eig_fork = nullptr;
   DBuf eig_ws[NEIG];
   DBuf scratch_a, scratch_b;
-  DBuf scratch_tc, tc_conv_tasks, tc_gemm_tasks, tc_err;
+  DBuf scratch_tc, tc_conv_tasks, tc_gemm_tasks;
   // precision of the per-site FP64 GEMM tasks (fusion, renormalisation,
   // truncation): MPSLCC_FP64, or MPSLCC_BF16X3 inside mixed-precision sweeps
   int gemm_prec = MPSLCC_FP64;
@@ -388,8 +411,8 @@ void env_update_right(Ctx& c, Family& F, int p, const RightFused& rf);
 std::vector<uint16_t> fused_piece_masks(const Mpo& W, int p, bool left);
 // Dimension of the piece of local state s in sector f of a fused space (0 if
 // the sector has none); a piece of state -1 (a bare bond sector) matches any s.
-int piece_dim(const Fused& F, int f, int s);
-int piece_off(const Fused& F, int f, int s);
+inline int piece_dim(const Fused& F, int f, int s) { return F.pd[f][s]; }
+inline int piece_off(const Fused& F, int f, int s) { return F.po[f][s]; }
 
 void two_site_middle(const MPS& m, int l, std::vector<QN>& mid, std::vector<long>& off, long& n);
 void one_site_middle(const MPS& m, int l, std::vector<QN>& mid, std::vector<long>& off, long& n);

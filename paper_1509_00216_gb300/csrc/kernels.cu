@@ -189,6 +189,16 @@ __global__ void lincomb_kernel(long n, int m, const double* __restrict__ V, long
   }
 }
 
+struct LincombArgs { double c[LINCOMB_ARGS]; };
+__global__ void lincomb_args_kernel(long n, int m, const double* __restrict__ V, long ld,
+                                    const __grid_constant__ LincombArgs coef, double* __restrict__ out) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int j = 0; j < m; ++j) s = fma(coef.c[j], V[j * ld + i], s);
+    out[i] = s;
+  }
+}
+
 __global__ void gather_kernel(const GatherTask* __restrict__ t, int max_elems) {
   const GatherTask T = t[blockIdx.y];
   const long nel = (long)T.nw * T.n;
@@ -317,6 +327,11 @@ void launch_precond(long n, const double* x, const double* d, double shift, doub
 }
 void launch_lincomb(long n, int m, const double* V, long ld, const double* coef, double* out, cudaStream_t s) {
   lincomb_kernel<<<elem_grid(n), 256, 0, s>>>(n, m, V, ld, coef, out);
+}
+void launch_lincomb_args(long n, int m, const double* V, long ld, const double* coef, double* out, cudaStream_t s) {
+  LincombArgs a;
+  for (int j = 0; j < LINCOMB_ARGS; ++j) a.c[j] = j < m ? coef[j] : 0.0;
+  lincomb_args_kernel<<<elem_grid(n), 256, 0, s>>>(n, m, V, ld, a, out);
 }
 void launch_gather(const GatherTask* d_tasks, int ntasks, int max_elems, cudaStream_t s) {
   if (ntasks <= 0) return;

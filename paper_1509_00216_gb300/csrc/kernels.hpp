@@ -105,6 +105,9 @@ void launch_precond(long n, const double* x, const double* d, double shift, doub
 // out[i] = sum_j coef[j] * V[j*ld + i] for j < m (linear combination of basis vectors)
 void launch_lincomb(long n, int m, const double* V, long ld, const double* d_coef, double* out,
                     cudaStream_t s);
+// The same with the coefficients (host, m <= LINCOMB_ARGS) as launch arguments.
+constexpr int LINCOMB_ARGS = 64;
+void launch_lincomb_args(long n, int m, const double* V, long ld, const double* coef, double* out, cudaStream_t s);
 // proj[j] = <V_j, x> for j < m (batched dots), written to d_out[0..m)
 void launch_multidot(long n, int m, const double* V, long ld, const double* x, double* d_out,
                      double* d_partial, cudaStream_t s);

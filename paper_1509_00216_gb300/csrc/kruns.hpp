@@ -20,28 +20,35 @@ struct KRun {
 // down to 8) before the open run's last step ends joins that run, so no
 // column is read by two runs; the columns a run reads outside the ranges must
 // be zero in one operand, so that they add nothing.
-inline std::vector<KRun> merge_runs(std::vector<std::pair<long, long>>& r, int KT) {
-  std::sort(r.begin(), r.end());
-  std::vector<KRun> out;
-  long de = 0;   // end of the data the open run must cover
-  for (const auto& x : r) {
-    if (x.second <= x.first) continue;
-    const long a8 = x.first & ~7L;
-    if (!out.empty() && a8 < out.back().kx + out.back().steps * KT) {
-      de = std::max(de, x.second);
-      out.back().steps = (de - out.back().kx + KT - 1) / KT;
+struct RunBuilder {   // the ranges one by one, in ascending order
+  int KT;
+  std::vector<KRun> runs;
+  long de = 0;        // end of the data the open run must cover
+  explicit RunBuilder(int KT_) : KT(KT_) {}
+  void add(long a, long b) {
+    if (b <= a) return;
+    const long a8 = a & ~7L;
+    if (!runs.empty() && a8 < runs.back().kx + runs.back().steps * KT) {
+      de = std::max(de, b);
+      runs.back().steps = (de - runs.back().kx + KT - 1) / KT;
     } else {
-      out.push_back({a8, (x.second - a8 + KT - 1) / KT});
-      de = x.second;
+      runs.push_back({a8, (b - a8 + KT - 1) / KT});
+      de = b;
     }
   }
-  return out;
+};
+
+inline std::vector<KRun> merge_runs(std::vector<std::pair<long, long>>& r, int KT) {
+  std::sort(r.begin(), r.end());
+  RunBuilder out(KT);
+  for (const auto& x : r) out.add(x.first, x.second);
+  return std::move(out.runs);
 }
 
 // The same ranges merged exactly (sorted, disjoint, neither overlapping nor
 // touching), for kernels that read element by element (the FP64 path).
 inline std::vector<std::pair<long, long>> merge_exact(std::vector<std::pair<long, long>>& r) {
-  std::sort(r.begin(), r.end());
+  if (!std::is_sorted(r.begin(), r.end())) std::sort(r.begin(), r.end());
   std::vector<std::pair<long, long>> m;
   for (const auto& x : r) {
     if (x.second <= x.first) continue;

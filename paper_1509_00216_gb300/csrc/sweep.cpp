@@ -41,17 +41,26 @@ std::vector<double> multidot(Ctx& c, const double* V, long ld, int m, const doub
   std::vector<double> out(m);
   if (m == 0) return out;
   c.red.ensure(&c, std::max<size_t>(4096, (size_t)m * 64) * sizeof(double));
-  c.red_out.ensure(&c, std::max(256, m) * sizeof(double));
-  launch_multidot(n, m, V, ld, x, c.red_out.d(), c.red.d(), c.s());
+  const bool host = m <= 256;   // results straight to pinned host memory
+  if (!host) c.red_out.ensure(&c, m * sizeof(double));
+  launch_multidot(n, m, V, ld, x, host ? c.out_dev->red : c.red_out.d(), c.red.d(), c.s());
   c.st.kernel_launches += 2;
-  cuda_check(cudaMemcpyAsync(out.data(), c.red_out.p, m * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "mdot");
+  if (!host)
+    cuda_check(cudaMemcpyAsync(out.data(), c.red_out.p, m * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "mdot");
   cuda_check(cudaStreamSynchronize(c.s()), "mdot sync");
   check_f64(c);
+  if (host)
+    for (int j = 0; j < m; ++j) out[j] = c.out->red[j];
   return out;
 }
 
 // out = sum_j coef[j] V_j
 void lincomb(Ctx& c, const double* V, long ld, int m, const std::vector<double>& coef, double* out, long n) {
+  if (m <= LINCOMB_ARGS) {   // coefficients as launch arguments
+    launch_lincomb_args(n, m, V, ld, coef.data(), out, c.s());
+    c.st.kernel_launches++;
+    return;
+  }
   c.red_out.ensure(&c, std::max(256, m) * sizeof(double));
   cuda_check(cudaMemcpyAsync(c.red_out.p, coef.data(), m * sizeof(double), cudaMemcpyHostToDevice, c.s()), "coef");
   launch_lincomb(n, m, V, ld, c.red_out.d(), out, c.s());

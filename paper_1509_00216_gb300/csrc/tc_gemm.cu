@@ -718,7 +718,10 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
 
 // window conversion FP64 -> BF16 / FP32 with batched strides
 struct ConvTask {
-  const double* src;
+  union {
+    const double* src;
+    long long src_off;  // elements from the launch's base
+  };
   void* dst;
   int rows, cols, src_ld, dst_ld, batch;
   long long s_src, s_dst;
@@ -840,7 +843,9 @@ __device__ __forceinline__ void conv_put(const ConvTask& T, long long o, double 
 // time, 16 in sequence, with 2-byte stores and FP64-pipe arithmetic: 7.9 ms
 // for the operators of the M1 = 1500 position, now 3.0 ms.
 template <int PREC>
-__global__ void __launch_bounds__(CONV_T) conv_kernel(const ConvTask* __restrict__ t, int ntasks, long long total) {
+__global__ void __launch_bounds__(CONV_T) conv_kernel(const ConvTask* __restrict__ t, int ntasks, long long total,
+                                                      const double* base) {
+  // sources are addresses, or (base given) offsets from it
   for (long long tile = blockIdx.x; tile < total; tile += gridDim.x) {
     int lo = 0, hi = ntasks - 1;
     while (lo < hi) {
@@ -848,7 +853,8 @@ __global__ void __launch_bounds__(CONV_T) conv_kernel(const ConvTask* __restrict
       if (t[mid].tile0 <= tile) lo = mid;
       else hi = mid - 1;
     }
-    const ConvTask T = t[lo];
+    ConvTask T = t[lo];
+    if (base) T.src = base + T.src_off;
     const long long local = tile - T.tile0;
     if (!T.vec) {
       const long long per = (long long)T.rows * T.cols;
@@ -1071,11 +1077,9 @@ TcTask make_task(Ctx& c, int prec, const void* A, long lda, const void* B, long 
   t.tn = (n + t.ntile - 1) / t.ntile;
   // output range check
   const int es = (mode == 1 || mode == 3 || mode == 5) ? 2 : (mode == 4 ? 8 : 4);
+  // the furthest row is the last one, or the last of the full row batches
   long long last = (long long)((m - 1) / rpb) * bstride + (long long)((m - 1) % rpb) * ldc + (n - 1);
-  for (int r = 0; r < std::min(m, rpb); ++r) {
-    long long l2 = (long long)((m - 1 - r) / rpb) * bstride + (long long)((m - 1 - r) % rpb) * ldc + (n - 1);
-    last = std::max(last, l2);
-  }
+  if (m >= rpb) last = std::max(last, (long long)(m / rpb - 1) * bstride + (long long)(rpb - 1) * ldc + (n - 1));
   if (mode == 3) last += soff;
   if (mode == 5) last += 5 * soff;
   last += (long long)(batch - 1) * t.cbatch;
@@ -1168,10 +1172,20 @@ long long plan_conv(ConvTask* t, int n) {
   return tot;
 }
 
-void launch_conv(int prec, const ConvTask* d, int n, long long tot, cudaStream_t s) {
+void launch_conv(int prec, const ConvTask* d, int n, long long tot, cudaStream_t s, const double* base = nullptr) {
   const int grid = (int)std::min<long long>(tot, 152LL * 64);
-  if (kprec(prec) == MPSLCC_BF16) conv_kernel<MPSLCC_BF16><<<grid, CONV_T, 0, s>>>(d, n, tot);
-  else conv_kernel<MPSLCC_TF32><<<grid, CONV_T, 0, s>>>(d, n, tot);
+  if (grid <= 0) return;
+  if (kprec(prec) == MPSLCC_BF16) conv_kernel<MPSLCC_BF16><<<grid, CONV_T, 0, s>>>(d, n, tot, base);
+  else conv_kernel<MPSLCC_TF32><<<grid, CONV_T, 0, s>>>(d, n, tot, base);
+}
+
+void check_conv_dst(Ctx& c, const ConvTask& x, int es) {
+  const long long blocks = x.pattern == 0 ? 0 : (x.pattern == 1 ? 1 : 5);  // extra split blocks
+  c.check_bytes(x.dst,
+                ((long long)(x.batch - 1) * x.s_dst + (long long)(x.rows - 1) * x.dst_ld + blocks * x.soff +
+                 (x.pad ? pad8(x.cols) : x.cols)) *
+                    es,
+                "conv dst");
 }
 
 void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
@@ -1184,12 +1198,7 @@ void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
     else
       c.check_range(x.src, 0, (long long)(x.batch - 1) * x.s_src + (long long)(x.rows - 1) * x.src_ld + x.cols - 1,
                     "conv src");
-    const long long blocks = x.pattern == 0 ? 0 : (x.pattern == 1 ? 1 : 5);  // extra split blocks
-    c.check_bytes(x.dst,
-                  ((long long)(x.batch - 1) * x.s_dst + (long long)(x.rows - 1) * x.dst_ld + blocks * x.soff +
-                   (x.pad ? pad8(x.cols) : x.cols)) *
-                      es,
-                  "conv dst");
+    check_conv_dst(c, x, es);
   }
   const long long tot = plan_conv(t.data(), (int)t.size());
   dtasks.ensure(&c, t.size() * sizeof(ConvTask));
@@ -1200,12 +1209,14 @@ void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
   c.st.kernel_launches++;
 }
 
-void check_err(Ctx& c, DBuf& err) {
-  int h = 0;
-  cuda_check(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, c.s()), "tc err d2h");
+int* tc_flag(Ctx& c) { return &c.out_dev->flag[1]; }
+
+// Waits for the stream; throws if a tensor-core product gave up.
+void check_err(Ctx& c) {
   cuda_check(cudaStreamSynchronize(c.s()), "tc sync");
+  const int h = c.out->flag[1];
   if (h) {
-    cudaMemsetAsync(err.p, 0, sizeof(int), c.s());
+    c.out->flag[1] = 0;
     throw Error(ST_TIMEOUT, "tensor-core kernel gave up waiting on an mbarrier (code " + std::to_string(h) + ")");
   }
 }
@@ -1224,7 +1235,7 @@ long rows_p(const Fused& F, int f, int s) {
 struct TcState {
   int layout = -1;      // operand precision class: TF32, BF16 or BF16X3 (the
                         // three-piece six-block layout, serving BF16X3 and BF16X6)
-  DBuf lcat, rstk, tt, x, conv, convx, err;
+  DBuf lcat, rstk, tt, x, conv, convx;
   std::vector<long> lcat_off, K8, tt_off, x_off;
   std::vector<long> stk_off;
   // K layout per bra key: the operator classes (segments) side by side, and
@@ -1236,6 +1247,7 @@ struct TcState {
   // no piece of state s).
   std::vector<std::vector<std::array<long, 4>>> kblk;
   std::vector<ConvTask> xconv;
+  long long xtiles = 0;
   // Phase-1 units: the rows of one R' stack with bra local state so (piece
   // of dimension d at row boff of the bra sector) for channels w0 .. w1-1
   // whose pieces (so, .) agree; `in` = the ket local states of those pieces.
@@ -1253,8 +1265,8 @@ struct TcState {
   // (TC_CAPS[0..2]), built on first use; phase 2 keeps its K-split FP32 partials
   // and the segments of their fixed-order sum.
   struct Lists {
-    bool built = false;
-    DBuf t1, t2, ypart, segs, runs;
+    bool built[2] = {false, false};   // per phase
+    DBuf t1, t2, ypart, segs, runs[2];
     int n1 = 0, n2 = 0, nseg = 0;
     long long tiles1 = 0, tiles2 = 0, seg_tiles = 0;
   };
@@ -1377,7 +1389,6 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
   zalloc(S->rstk, ssz, es);
   zalloc(S->tt, tsz, es);
   zalloc(S->x, xsz, es);
-  zalloc(S->err, 4, 1);
   // FP64 -> low precision copies of the non-zero pieces of L' (A side of
   // phase 2), per run of channels with equal piece masks
   std::vector<ConvTask> cv;
@@ -1452,7 +1463,7 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
       if (d1 == 0) continue;
       ConvTask t;
       std::memset(&t, 0, sizeof(t));
-      t.src = P.xin.d() + P.off_k[ki] + (long)piece_off(lf.FLk, fl, s1) * rk;
+      t.src_off = P.off_k[ki] + (long)piece_off(lf.FLk, fl, s1) * rk;
       t.dst = (char*)S->x.p + (size_t)(S->x_off[ki] + rows_p(lf.FLk, fl, s1) * sp * pad8(rk)) * es;
       t.rows = d1;
       t.cols = rk;
@@ -1465,6 +1476,18 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
       S->xconv.push_back(t);
     }
   }
+  // uploaded once: its sources are offsets from the vector of a product
+  for (const auto& t : S->xconv) {
+    MPSLCC_REQUIRE(t.src_off >= 0 && t.src_off + (long long)(t.rows - 1) * t.src_ld + t.cols <= P.nk, ST_INTERNAL,
+                   "conversion outside the local vector");
+    check_conv_dst(c, t, es);
+  }
+  S->xtiles = plan_conv(S->xconv.data(), (int)S->xconv.size());
+  S->convx.alloc(&c, std::max<size_t>(S->xconv.size(), 1) * sizeof(ConvTask));
+  if (!S->xconv.empty())
+    cuda_check(cudaMemcpyAsync(S->convx.p, S->xconv.data(), S->xconv.size() * sizeof(ConvTask), cudaMemcpyHostToDevice,
+                               c.s()),
+               "vector conversion tasks");
   // algorithmic bytes of each variant, per BF16 (or TF32) piece read or
   // written: the non-zero pieces of the fused operators and the parts of the
   // vector and of T they multiply, each read once; T and sigma written once
@@ -1495,16 +1518,18 @@ void tc_prepare(Ctx& c, SigmaPlan& P, int prec) {
       double a = 0, kc = 0;
       for (const auto& sg : lf.seg[bi]) {
         const int fk = lf.kk[sg.kidx], c0 = S->cstartL[sg.cls];
-        for (int w = 0; w < sg.nw; ++w) {
+        for (int w = 0; w < sg.nw;) {
           const uint16_t m = S->mL[c0 + w];
-          int used = 0;
+          int w1 = w + 1, used = 0;
+          while (w1 < sg.nw && S->mL[c0 + w1] == m) ++w1;
           for (int b = 0; b < 16; ++b)
             if (m >> b & 1) {
-              a += (double)piece_dim(lf.FLb, fb, b >> 2) * piece_dim(lf.FLk, fk, b & 3);
+              a += (double)(w1 - w) * piece_dim(lf.FLb, fb, b >> 2) * piece_dim(lf.FLk, fk, b & 3);
               used |= 1 << (b & 3);
             }
           for (int sn = 0; sn < 4; ++sn)
-            if (used >> sn & 1) kc += piece_dim(lf.FLk, fk, sn);
+            if (used >> sn & 1) kc += (double)(w1 - w) * piece_dim(lf.FLk, fk, sn);
+          w = w1;
         }
       }
       S->bytes2[v] += (double)es * pcs * (a + rb * kc) + 4.0 * lb * rb;
@@ -1552,10 +1577,11 @@ long total_steps(const std::vector<KRun>& r) {
   return s;
 }
 
-// Task lists of sigma variant v with N tiles of at most TC_CAPS[ci] rows.
-void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
+// Task list of one phase (0, 1) of sigma variant v with N tiles of at most
+// TC_CAPS[ci] rows.
+void build_list(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci, int phase) {
   TcState::Lists& Ls = S->lists[v][ci];
-  if (Ls.built) return;
+  if (Ls.built[phase]) return;
   const int cap = TC_CAPS[ci];
   const int layout = S->layout;
   const int es = esize(layout);
@@ -1570,60 +1596,85 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
   const int kp = v == 1 ? MPSLCC_BF16 : layout;
   const int KT = kp == MPSLCC_TF32 ? 32 : 64;
   const int reps = v == 1 ? 6 : 1;
-  std::vector<TcTask> t1, t2;
-  std::vector<std::vector<KRun>> r1, r2;
+  std::vector<TcTask> tasks;
+  std::vector<std::vector<KRun>> runs;   // per task
+  auto upload = [&](DBuf& dt, int& n, long long& tiles) {
+    // the run tables in one device buffer
+    std::vector<int> tab;
+    std::vector<long> at(tasks.size());
+    for (size_t i = 0; i < tasks.size(); ++i) at[i] = append_runs(tab, runs[i], tasks[i].kchunk, tasks[i].ksplit);
+    Ls.runs[phase].alloc(&c, std::max<size_t>(tab.size(), 4) * sizeof(int));
+    if (!tab.empty())
+      cuda_check(cudaMemcpyAsync(Ls.runs[phase].p, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, c.s()),
+                 "K runs");
+    for (size_t i = 0; i < tasks.size(); ++i) {
+      tasks[i].kr = (const int*)Ls.runs[phase].p + at[i];
+      tasks[i].nkr = (int)runs[i].size();
+    }
+    n = (int)tasks.size();
+    tiles = plan_tc(tasks);
+    dt.alloc(&c, std::max<size_t>(tasks.size(), 1) * sizeof(TcTask));
+    if (!tasks.empty())
+      cuda_check(cudaMemcpyAsync(dt.p, tasks.data(), tasks.size() * sizeof(TcTask), cudaMemcpyHostToDevice, c.s()),
+                 "tc tasks");
+    Ls.built[phase] = true;
+  };
   // phase 1: T_w^T = R'_w psi^T, one task per unit (rows of one bra local
   // state for a run of channels of one class); K runs = the ket pieces the
   // unit's channels reach
-  const int mode1 = v == 1 ? 5 : (six ? 3 : (layout == MPSLCC_TF32 ? 2 : 1));
-  for (const auto& u : S->u1) {
-    const auto& st = rf.stk[u.si];
-    const int bi = st.bidx, ki = st.kidx;
-    const LeftFused::Seg* sg = lf.find_seg(bi, st.cls);
-    const size_t g = sg - lf.seg[bi].data();
-    const int fk = rf.kk[ki], rk = rf.FRk.d[fk];
-    const long pitch = sp * pad8(rk);
-    const int kk = v == 1 ? (int)pitch : rk;
-    std::vector<std::pair<long, long>> rg;
-    for (int j = 0; j < reps; ++j)
-      for (int sn = 0; sn < 4; ++sn) {
-        if (!(u.in >> sn & 1)) continue;
-        const long co = piece_off(rf.FRk, fk, sn) + (long)j * pad8(rk);
-        rg.push_back({co, co + piece_dim(rf.FRk, fk, sn)});
+  if (phase == 0) {
+    const int mode1 = v == 1 ? 5 : (six ? 3 : (layout == MPSLCC_TF32 ? 2 : 1));
+    for (const auto& u : S->u1) {
+      const auto& st = rf.stk[u.si];
+      const int bi = st.bidx, ki = st.kidx;
+      const LeftFused::Seg* sg = lf.find_seg(bi, st.cls);
+      const size_t g = sg - lf.seg[bi].data();
+      const int fk = rf.kk[ki], rk = rf.FRk.d[fk];
+      const long pitch = sp * pad8(rk);
+      const int kk = v == 1 ? (int)pitch : rk;
+      RunBuilder rb(KT);   // pieces ascend with the local state
+      for (int j = 0; j < reps; ++j)
+        for (int sn = 0; sn < 4; ++sn) {
+          if (!(u.in >> sn & 1)) continue;
+          const long co = piece_off(rf.FRk, fk, sn) + (long)j * pad8(rk);
+          rb.add(co, co + piece_dim(rf.FRk, fk, sn));
+        }
+      const int steps = (int)total_steps(rb.runs);
+      if (steps == 0) continue;   // the ket sector has none of the unit's pieces: T stays zero there
+      const long ldc = sp * S->K8[bi];
+      // split tasks: lo parts in block 2 of both operands (and of the output)
+      const long long so = v == 1 ? S->K8[bi] : 2 * S->K8[bi];
+      // the output columns (psi's padded rows) are scattered by local-state
+      // piece s1 to block s1 of the segment (piece-major K layout), channel w
+      // of the unit at stride padp(d1)
+      const int fl = lf.kk[ki];
+      const long n8 = rows_p(lf.FLk, fl, 4);
+      void* C = (char*)S->tt.p + (size_t)(S->tt_off[bi] + (long)u.boff * ldc) * es;
+      TcTask t = make_task(c, kp, (char*)S->rstk.p + (size_t)(S->stk_off[u.si] + u.row0 * pitch) * es, pitch,
+                           (char*)S->x.p + (size_t)S->x_off[ki] * es, pitch, (u.w1 - u.w0) * u.d, (int)n8, kk, C,
+                           (int)ldc, u.d, 0, mode1, 1, six ? so : 0, six ? 2 * pad8(rk) : 0, 1, 0, 0, 0, 0, cap, steps);
+      long long last = 0;
+      for (int s1 = 0; s1 < 4; ++s1) {
+        const int d1 = piece_dim(lf.FLk, fl, s1);
+        if (d1 == 0) continue;
+        MPSLCC_REQUIRE(S->kblk[bi][g][s1] >= 0 && t.npc < 4, ST_INTERNAL, "phase-1 column pieces");
+        t.pcs[t.npc] = (int)rows_p(lf.FLk, fl, s1);
+        t.pcw[t.npc] = (int)padp(d1);
+        t.pcb[t.npc] = S->kblk[bi][g][s1] + (long long)u.w0 * padp(d1);
+        last = std::max(last, (long long)(u.d - 1) * ldc + t.pcb[t.npc] + (long long)(u.w1 - u.w0) * padp(d1) - 1);
+        t.npc++;
       }
-    std::vector<KRun> runs = merge_runs(rg, KT);
-    const int steps = (int)total_steps(runs);
-    if (steps == 0) continue;   // the ket sector has none of the unit's pieces: T stays zero there
-    const long ldc = sp * S->K8[bi];
-    // split tasks: lo parts in block 2 of both operands (and of the output)
-    const long long so = v == 1 ? S->K8[bi] : 2 * S->K8[bi];
-    // the output columns (psi's padded rows) are scattered by local-state
-    // piece s1 to block s1 of the segment (piece-major K layout), channel w
-    // of the unit at stride padp(d1)
-    const int fl = lf.kk[ki];
-    const long n8 = rows_p(lf.FLk, fl, 4);
-    void* C = (char*)S->tt.p + (size_t)(S->tt_off[bi] + (long)u.boff * ldc) * es;
-    TcTask t = make_task(c, kp, (char*)S->rstk.p + (size_t)(S->stk_off[u.si] + u.row0 * pitch) * es, pitch,
-                         (char*)S->x.p + (size_t)S->x_off[ki] * es, pitch, (u.w1 - u.w0) * u.d, (int)n8, kk, C,
-                         (int)ldc, u.d, 0, mode1, 1, six ? so : 0, six ? 2 * pad8(rk) : 0, 1, 0, 0, 0, 0, cap, steps);
-    long long last = 0;
-    for (int s1 = 0; s1 < 4; ++s1) {
-      const int d1 = piece_dim(lf.FLk, fl, s1);
-      if (d1 == 0) continue;
-      MPSLCC_REQUIRE(S->kblk[bi][g][s1] >= 0 && t.npc < 4, ST_INTERNAL, "phase-1 column pieces");
-      t.pcs[t.npc] = (int)rows_p(lf.FLk, fl, s1);
-      t.pcw[t.npc] = (int)padp(d1);
-      t.pcb[t.npc] = S->kblk[bi][g][s1] + (long long)u.w0 * padp(d1);
-      last = std::max(last, (long long)(u.d - 1) * ldc + t.pcb[t.npc] + (long long)(u.w1 - u.w0) * padp(d1) - 1);
-      t.npc++;
+      t.pcs[t.npc] = (int)n8;
+      if (t.npc == 0) continue;
+      if (mode1 == 3) last += so;
+      if (mode1 == 5) last += 5 * so;
+      c.check_bytes(C, (last + 1) * (mode1 == 2 ? 4 : 2), "phase-1 piece output");
+      MPSLCC_REQUIRE(t.ksplit == 1, ST_INTERNAL, "phase-1 task split over K");
+      runs.push_back(std::move(rb.runs));
+      tasks.push_back(t);
     }
-    t.pcs[t.npc] = (int)n8;
-    if (t.npc == 0) continue;
-    if (mode1 == 3) last += so;
-    if (mode1 == 5) last += 5 * so;
-    c.check_bytes(C, (last + 1) * (mode1 == 2 ? 4 : 2), "phase-1 piece output");
-    r1.push_back(std::move(runs));
-    t1.push_back(t);
+    upload(Ls.t1, Ls.n1, Ls.tiles1);
+    return;
   }
   // phase 2: sigma = Lcat Tt^T per unit (rows of one bra local state of a
   // middle sector), over the K runs of the channel pieces those rows reach,
@@ -1633,8 +1684,9 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
   // Split j of a unit stores its FP32 partial at its own offset; one
   // reduction sums the partials in increasing j into the FP64 sigma, so the
   // result does not depend on the order the splits finish in.
+  std::vector<std::vector<KRun>> r2;
   for (const auto& u : S->u2) {
-    std::vector<std::pair<long, long>> rg;
+    RunBuilder rb(KT);   // blocks, classes, states and channels in the order of the K layout
     const int bi = u.bi;
     for (int j = 0; j < reps; ++j)
       for (size_t g = 0; g < lf.seg[bi].size(); ++g) {
@@ -1646,11 +1698,11 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
           for (int w = 0; w < sg.nw; ++w) {
             if (!((S->mL[c0 + w] >> (4 * u.so + sn)) & 1)) continue;
             const long co = (long)j * S->K8[bi] + S->kblk[bi][g][sn] + (long)w * padp(d);
-            rg.push_back({co, co + d});
+            rb.add(co, co + d);
           }
         }
       }
-    r2.push_back(merge_runs(rg, KT));
+    r2.push_back(std::move(rb.runs));
   }
   long long work = 0;
   for (size_t i = 0; i < S->u2.size(); ++i) {
@@ -1683,7 +1735,6 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
     segs.push_back(sg);   // nsplit = 0: no channel reaches these rows, sigma is zero there
   }
   Ls.ypart.alloc(&c, std::max<long>(poff, 4) * 4);
-  std::vector<int> r2i;
   for (size_t i = 0; i < S->u2.size(); ++i) {
     if (ksv[i] == 0) continue;
     const auto& u = S->u2[i];
@@ -1691,32 +1742,12 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
     const long pitch = sp * S->K8[u.bi];
     const int kk = v == 1 ? (int)pitch : (int)S->K8[u.bi];
     const SplitSeg& sg = segs[i];
-    t2.push_back(make_task(c, kp, (char*)S->lcat.p + (size_t)(S->lcat_off[u.bi] + (long)u.boff * pitch) * es, pitch,
+    tasks.push_back(make_task(c, kp, (char*)S->lcat.p + (size_t)(S->lcat_off[u.bi] + (long)u.boff * pitch) * es, pitch,
                            (char*)S->tt.p + (size_t)S->tt_off[u.bi] * es, pitch, u.d, rb, kk,
                            (float*)Ls.ypart.p + sg.part_off, sg.ldp, 1 << 30, 0, 2, ksv[i], 0,
                            (six && v == 0) ? 2 * S->K8[u.bi] : 0, 1, 0, 0, 0, sg.sstride, cap,
                            (int)total_steps(r2[i])));
-    r2i.push_back((int)i);
-  }
-  // run tables of both phases in one device buffer
-  std::vector<int> tab;
-  std::vector<long> at1(t1.size()), at2(t2.size());
-  for (size_t i = 0; i < t1.size(); ++i) {
-    MPSLCC_REQUIRE(t1[i].ksplit == 1, ST_INTERNAL, "phase-1 task split over K");
-    at1[i] = append_runs(tab, r1[i], t1[i].kchunk, t1[i].ksplit);
-  }
-  for (size_t i = 0; i < t2.size(); ++i) at2[i] = append_runs(tab, r2[r2i[i]], t2[i].kchunk, t2[i].ksplit);
-  Ls.runs.alloc(&c, std::max<size_t>(tab.size(), 4) * sizeof(int));
-  if (!tab.empty())
-    cuda_check(cudaMemcpyAsync(Ls.runs.p, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, c.s()),
-               "K runs");
-  for (size_t i = 0; i < t1.size(); ++i) {
-    t1[i].kr = (const int*)Ls.runs.p + at1[i];
-    t1[i].nkr = (int)r1[i].size();
-  }
-  for (size_t i = 0; i < t2.size(); ++i) {
-    t2[i].kr = (const int*)Ls.runs.p + at2[i];
-    t2[i].nkr = (int)r2[r2i[i]].size();
+    runs.push_back(std::move(r2[i]));
   }
   Ls.nseg = (int)segs.size();
   Ls.seg_tiles = plan_split_tiles(segs.data(), (int)segs.size());
@@ -1724,20 +1755,7 @@ void build_lists(Ctx& c, SigmaPlan& P, TcState* S, int v, int ci) {
   if (!segs.empty())
     cuda_check(cudaMemcpyAsync(Ls.segs.p, segs.data(), segs.size() * sizeof(SplitSeg), cudaMemcpyHostToDevice, c.s()),
                "split segments");
-  Ls.n1 = (int)t1.size();
-  Ls.n2 = (int)t2.size();
-  Ls.tiles1 = plan_tc(t1);
-  Ls.tiles2 = plan_tc(t2);
-  Ls.t1.alloc(&c, std::max<size_t>(t1.size(), 1) * sizeof(TcTask));
-  Ls.t2.alloc(&c, std::max<size_t>(t2.size(), 1) * sizeof(TcTask));
-  if (!t1.empty())
-    cuda_check(cudaMemcpyAsync(Ls.t1.p, t1.data(), t1.size() * sizeof(TcTask), cudaMemcpyHostToDevice, c.s()),
-               "tc tasks");
-  if (!t2.empty())
-    cuda_check(cudaMemcpyAsync(Ls.t2.p, t2.data(), t2.size() * sizeof(TcTask), cudaMemcpyHostToDevice, c.s()),
-               "tc tasks");
-  cuda_check(cudaStreamSynchronize(c.s()), "tc lists sync");
-  Ls.built = true;
+  upload(Ls.t2, Ls.n2, Ls.tiles2);
 }
 
 // Tile-shape autotuner of the sigma phases.  For every (operator family,
@@ -1786,26 +1804,25 @@ void tc_sigma(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
   TcState* S = (prec == MPSLCC_BF16X3 || prec == MPSLCC_BF16X6) ? P.tc6 : P.tc;
   const int v = prec == MPSLCC_BF16X6 ? 1 : 0;
   const int kp = v == 1 ? MPSLCC_BF16 : S->layout;
-  if (P.nk > 0)
-    cuda_check(cudaMemcpyAsync(P.xin.p, x, P.nk * sizeof(double), cudaMemcpyDeviceToDevice, c.s()), "sigma in");
-  std::vector<ConvTask> xc = S->xconv;
-  run_conv(c, S->layout, xc, S->convx);
+  launch_conv(S->layout, (const ConvTask*)S->convx.p, (int)S->xconv.size(), S->xtiles, c.s(), x);
+  cuda_check(cudaGetLastError(), "conv launch");
+  c.st.kernel_launches++;
   Ctx::TuneEntry& e1 = tune_entry(c, P, 1, prec, S->bytes1[v]);
   Ctx::TuneEntry& e2 = tune_entry(c, P, 2, prec, S->bytes2[v]);
   const int c1 = tune_choice(c, e1), c2 = tune_choice(c, e2);
-  build_lists(c, P, S, v, list_of(c1));
-  build_lists(c, P, S, v, list_of(c2));
+  build_list(c, P, S, v, list_of(c1), 0);
+  build_list(c, P, S, v, list_of(c2), 1);
   const TcState::Lists& L1 = S->lists[v][list_of(c1)];
   const TcState::Lists& L2 = S->lists[v][list_of(c2)];
   cudaEventRecord(c.ev_p0, c.s());
-  launch_tc(c, kp, (const TcTask*)L1.t1.p, L1.n1, L1.tiles1, (int*)S->err.p, TC_CAPS[c1], TC_CFG[c1]);
+  launch_tc(c, kp, (const TcTask*)L1.t1.p, L1.n1, L1.tiles1, tc_flag(c), TC_CAPS[c1], TC_CFG[c1]);
   cudaEventRecord(c.ev_p1, c.s());
-  launch_tc(c, kp, (const TcTask*)L2.t2.p, L2.n2, L2.tiles2, (int*)S->err.p, TC_CAPS[c2], TC_CFG[c2]);
+  launch_tc(c, kp, (const TcTask*)L2.t2.p, L2.n2, L2.tiles2, tc_flag(c), TC_CAPS[c2], TC_CFG[c2]);
   cudaEventRecord(c.ev_p2, c.s());
   launch_splitk_reduce_f32((const SplitSeg*)L2.segs.p, L2.nseg, L2.seg_tiles, (const float*)L2.ypart.p, y, c.s());
   cuda_check(cudaGetLastError(), "split-K reduction");
   c.st.kernel_launches++;
-  check_err(c, S->err);
+  check_err(c);
   float m1 = 0, m2 = 0;
   cudaEventElapsedTime(&m1, c.ev_p0, c.ev_p1);
   cudaEventElapsedTime(&m2, c.ev_p1, c.ev_p2);
@@ -1829,7 +1846,7 @@ void tc_selftest(Ctx& c, int prec, int m, int n, int k, const double* A, const d
   const int es = esize(prec);
   const int sp = prec == MPSLCC_BF16X3 ? 2 : 1;
   long k8 = pad8(k), kk = sp * k8;
-  DBuf dA, dB, lA, lB, out, err, conv;
+  DBuf dA, dB, lA, lB, out, conv;
   dA.alloc(&c, std::max<long>((long)m * k, 1) * 8);
   dB.alloc(&c, std::max<long>((long)n * k, 1) * 8);
   cuda_check(cudaMemcpyAsync(dA.p, A, (size_t)m * k * 8, cudaMemcpyHostToDevice, c.s()), "A");
@@ -1848,16 +1865,14 @@ void tc_selftest(Ctx& c, int prec, int m, int n, int k, const double* A, const d
   const int oes = mode == 1 ? 2 : 4;
   out.alloc(&c, (size_t)m * n * oes);
   cuda_check(cudaMemsetAsync(out.p, 0, (size_t)m * n * oes, c.s()), "z");
-  err.alloc(&c, 16);
-  cuda_check(cudaMemsetAsync(err.p, 0, 16, c.s()), "z");
   std::vector<TcTask> t{make_task(c, prec, lA.p, kk, lB.p, kk, m, n, (int)(sp == 2 ? k8 : kk), out.p, n, 1 << 30,
                                   0, mode, ksplit, 0, k8)};
   long long tiles = plan_tc(t);
   DBuf dt;
   dt.alloc(&c, sizeof(TcTask));
   cuda_check(cudaMemcpyAsync(dt.p, t.data(), sizeof(TcTask), cudaMemcpyHostToDevice, c.s()), "task");
-  launch_tc(c, prec, (const TcTask*)dt.p, 1, tiles, (int*)err.p);
-  check_err(c, err);
+  launch_tc(c, prec, (const TcTask*)dt.p, 1, tiles, tc_flag(c));
+  check_err(c);
   if (mode == 1) {
     std::vector<uint16_t> hb((size_t)m * n);
     cuda_check(cudaMemcpy(hb.data(), out.p, hb.size() * 2, cudaMemcpyDeviceToHost), "d2h");
@@ -2093,12 +2108,10 @@ void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
   c.tc_gemm_tasks.ensure(&c, tt.size() * sizeof(TcTask));
   cuda_check(cudaMemcpyAsync(c.tc_gemm_tasks.p, tt.data(), tt.size() * sizeof(TcTask), cudaMemcpyHostToDevice, c.s()),
              "tc gemm tasks");
-  c.tc_err.ensure(&c, 16);
-  cuda_check(cudaMemsetAsync(c.tc_err.p, 0, 16, c.s()), "tc err zero");
   const double th1 = c.opts.verbose >= 2 ? wall_seconds() : 0.0;
-  launch_tc(c, MPSLCC_BF16, (const TcTask*)c.tc_gemm_tasks.p, (int)tt.size(), tiles, (int*)c.tc_err.p);
+  launch_tc(c, MPSLCC_BF16, (const TcTask*)c.tc_gemm_tasks.p, (int)tt.size(), tiles, tc_flag(c));
   c.st.tc_gemm_flops += fl;
-  check_err(c, c.tc_err);
+  check_err(c);
   if (c.opts.verbose >= 2) {
     long conv_elems = 0;
     for (const auto& t : cv) conv_elems += (long)t.rows * t.cols * t.batch;
