@@ -31,6 +31,7 @@
 
 #include "engine.hpp"
 #include "kruns.hpp"
+#include "tcfold.hpp"
 #include "tcgen05.cuh"
 
 namespace mpslcc {
@@ -44,6 +45,7 @@ struct alignas(64) TcTask {
   long long bstride;    // output offset between row batches (elements)
   int rpb;              // rows per batch of the output remap
   int ldc;
+  int cst;              // mode 4: elements between output columns
   int m, n, k;
   int ksteps, kchunk, ksplit;
   int ntile;            // UMMA N (multiple of 16, <= 256)
@@ -274,13 +276,15 @@ __device__ __forceinline__ void store_row(const TcTask* T, long long roff, int c
   // the remaining paths index v only with unrolled constants, so that the
   // accumulator row stays in registers
   if (T->mode == 4) {
-    double* C = (double*)T->C + roff + c0;
+    const int cst = T->cst;
+    double* C = (double*)T->C + roff + (long long)c0 * cst;
     const double al = T->alpha, be = T->beta;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       if (j >= nv) break;
       const double x = al * (double)__uint_as_float(v[j]);
-      C[j] = be == 0.0 ? x : x + be * C[j];
+      *C = be == 0.0 ? x : x + be * *C;
+      C += cst;
     }
     return;
   }
@@ -1032,7 +1036,7 @@ int tc_ksplit_steps(int ksteps, int hint) {
 TcTask make_task(Ctx& c, int prec, const void* A, long lda, const void* B, long ldb, int m, int n, int k, void* C,
                  int ldc, int rpb, long long bstride, int mode, int ksplit_hint, long long soff = 0,
                  long lo_off = 0, int batch = 1, long long a_bs = 0, long long b_bs = 0, long long c_bs = 0,
-                 long long kstride = 0, int cap = 256, int steps = 0) {
+                 long long kstride = 0, int cap = 256, int steps = 0, int cst = 1) {
   // steps > 0: the task reads `steps` K steps through a run table set by the
   // caller (k is then the operands' K extent, not the summed length)
   TcTask t;
@@ -1059,6 +1063,7 @@ TcTask make_task(Ctx& c, int prec, const void* A, long lda, const void* B, long 
   }
   t.C = C;
   t.ldc = ldc;
+  t.cst = cst;
   t.rpb = rpb;
   t.bstride = bstride;
   t.m = m;
@@ -1078,8 +1083,9 @@ TcTask make_task(Ctx& c, int prec, const void* A, long lda, const void* B, long 
   // output range check
   const int es = (mode == 1 || mode == 3 || mode == 5) ? 2 : (mode == 4 ? 8 : 4);
   // the furthest row is the last one, or the last of the full row batches
-  long long last = (long long)((m - 1) / rpb) * bstride + (long long)((m - 1) % rpb) * ldc + (n - 1);
-  if (m >= rpb) last = std::max(last, (long long)(m / rpb - 1) * bstride + (long long)(rpb - 1) * ldc + (n - 1));
+  const long long lc = (long long)(n - 1) * cst;
+  long long last = (long long)((m - 1) / rpb) * bstride + (long long)((m - 1) % rpb) * ldc + lc;
+  if (m >= rpb) last = std::max(last, (long long)(m / rpb - 1) * bstride + (long long)(rpb - 1) * ldc + lc);
   if (mode == 3) last += soff;
   if (mode == 5) last += 5 * soff;
   last += (long long)(batch - 1) * t.cbatch;
@@ -2024,7 +2030,8 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
 // and multiplied by the plain BF16 kernel over K' = 6 K, with an FP64
 // alpha/beta epilogue (about 2^-24 relative).  A task's batch stays one
 // tensor-core task: batched operands are converted to contiguous
-// [batch][rows][6 K] stacks read through 3D tensor maps.
+// [batch][rows][6 K] stacks, read as one tall operand beside a shared one and
+// through 3D tensor maps where both are batched.
 void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
   if (tasks.empty()) return;
   for (const auto& t : tasks) MPSLCC_REQUIRE(!t.kr, ST_INTERNAL, "K-run task on the FP64 emulation path");
@@ -2093,13 +2100,32 @@ void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
   char* base = (char*)c.scratch_tc.p;
   for (auto& t : cv) t.dst = base + (uintptr_t)t.dst * 2;
   run_conv(c, MPSLCC_BF16, cv, c.tc_conv_tasks);
+  // Orientation per task (tcfold.hpp); the six blocks of each operand keep
+  // their pattern on either side, so every sum has the same terms in the same
+  // order.  N tiles of 64 on two CTAs per SM unless wide tasks would then
+  // reload their rows for a quarter more operand traffic than tiles of 256.
+  std::vector<TcFold> fold[2];
+  double cost[2] = {0, 0};
+  constexpr int caps[2] = {256, 64};
+  for (int w = 0; w < 2; ++w)
+    for (const auto& j : jobs) {
+      fold[w].push_back(tc_fold(j.m, j.n, j.nb, j.a3, j.b3, j.ldc, j.sC, caps[w]));
+      const TcFold& f = fold[w].back();
+      const int nt = std::min(caps[w], (f.cols + 15) / 16 * 16);
+      cost[w] += (double)f.batch * ((f.rows + 127) / 128) * ((f.cols + nt - 1) / nt) * (128 + nt) * j.k;
+    }
+  const int w = cost[1] <= 1.25 * cost[0] ? 1 : 0, cap = caps[w];
   std::vector<TcTask> tt;
   tt.reserve(jobs.size());
-  for (const auto& j : jobs) {
+  for (size_t i = 0; i < jobs.size(); ++i) {
+    const Job& j = jobs[i];
+    const TcFold& f = fold[w][i];
     const long kp = pad8(j.k);
-    const long long sa = (long long)j.m * 6 * kp, sb = (long long)j.n * 6 * kp;
-    TcTask t = make_task(c, MPSLCC_BF16, base + j.ao * 2, 6 * kp, base + j.bo * 2, 6 * kp, j.m, j.n, (int)(6 * kp),
-                         j.C, j.ldc, 1 << 30, 0, 4, 1, 0, 0, j.nb, j.a3 ? sa : 0, j.b3 ? sb : 0, j.sC);
+    const long long sa = j.a3 ? (long long)j.m * 6 * kp : 0, sb = j.b3 ? (long long)j.n * 6 * kp : 0;
+    const bool one = f.batch == 1;
+    TcTask t = make_task(c, MPSLCC_BF16, base + (f.swap ? j.bo : j.ao) * 2, 6 * kp, base + (f.swap ? j.ao : j.bo) * 2,
+                         6 * kp, f.rows, f.cols, (int)(6 * kp), j.C, f.ldr, f.rpb, f.bstride, 4, 1, 0, 0, f.batch,
+                         one ? 0 : (f.swap ? sb : sa), one ? 0 : (f.swap ? sa : sb), f.cbatch, 0, cap, 0, f.cst);
     t.alpha = j.alpha;
     t.beta = j.beta;
     tt.push_back(t);
@@ -2109,7 +2135,7 @@ void run_gemms_tc(Ctx& c, std::vector<GemmTask>& tasks) {
   cuda_check(cudaMemcpyAsync(c.tc_gemm_tasks.p, tt.data(), tt.size() * sizeof(TcTask), cudaMemcpyHostToDevice, c.s()),
              "tc gemm tasks");
   const double th1 = c.opts.verbose >= 2 ? wall_seconds() : 0.0;
-  launch_tc(c, MPSLCC_BF16, (const TcTask*)c.tc_gemm_tasks.p, (int)tt.size(), tiles, tc_flag(c));
+  launch_tc(c, MPSLCC_BF16, (const TcTask*)c.tc_gemm_tasks.p, (int)tt.size(), tiles, tc_flag(c), cap, w);
   c.st.tc_gemm_flops += fl;
   check_err(c);
   if (c.opts.verbose >= 2) {
