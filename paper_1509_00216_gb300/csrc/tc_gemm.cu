@@ -144,40 +144,48 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* map, uint
   else tma_load_2d(dst, map, bar, x, y);
 }
 
-// Tile coordinates of global tile `tile` within task T: batch entry, K split,
-// M tile and N tile.
-struct TileCoord { int b, ks, tmi, tni; };
-__device__ __forceinline__ TileCoord tile_coord(const TcTask* T, long long tile) {
-  const long long local = tile - T->tile0;
-  const long long tiles_mn = (long long)T->tm * T->tn;
-  const long long per_b = tiles_mn * T->ksplit;
-  TileCoord tc;
-  tc.b = (int)(local / per_b);
-  const long long lb = local - (long long)tc.b * per_b;
-  tc.ks = (int)(lb / tiles_mn);
-  const int r = (int)(lb - (long long)tc.ks * tiles_mn);
-  tc.tmi = r / T->tn;
-  tc.tni = r - tc.tmi * T->tn;
-  return tc;
-}
-
-// A CTA visits its tiles in increasing order, so the owning task index never
-// decreases: step forward from the previous one (usually zero or one step),
-// with a binary search for long jumps.
-__device__ __forceinline__ int next_tc(const TcTask* t, int n, long long tile, int prev) {
-  int i = prev;
-  for (int s = 0; s < 4; ++s) {
-    if (i + 1 >= n || t[i + 1].tile0 > tile) return i;
-    ++i;
-  }
-  int lo = i, hi = n - 1;
+// Where a tile lies: its task, batch entry, K split, first row and column,
+// first K step, K steps, and the N of its products.
+struct TileAt { int ti, b, ks, row0, col0, kt0, nk, ntile; };
+__device__ __forceinline__ TileAt tile_at(const TcTask* tasks, int n, long long tile, int lo) {
+  int hi = n - 1;
   while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (t[mid].tile0 <= tile) lo = mid;
+    const int mid = (lo + hi + 1) >> 1;
+    if (tasks[mid].tile0 <= tile) lo = mid;
     else hi = mid - 1;
   }
-  return lo;
+  const TcTask* T = &tasks[lo];
+  const long long local = tile - T->tile0;
+  const int tn = T->tn, kchunk = T->kchunk, ksteps = T->ksteps;
+  const long long tiles_mn = (long long)T->tm * tn;
+  const long long per_b = tiles_mn * T->ksplit;
+  TileAt t;
+  t.ti = lo;
+  t.ntile = T->ntile;
+  t.b = (int)(local / per_b);
+  const long long lb = local - (long long)t.b * per_b;
+  t.ks = (int)(lb / tiles_mn);
+  const int r = (int)(lb - (long long)t.ks * tiles_mn);
+  const int tmi = r / tn;
+  t.row0 = tmi * 128;
+  t.col0 = (r - tmi * tn) * t.ntile;
+  t.kt0 = t.ks * kchunk;
+  t.nk = min(ksteps, t.kt0 + kchunk) - t.kt0;
+  return t;
 }
+
+// A warp finds its CTA's tiles 32 at a time, one per lane: the search over the
+// tasks and the divisions are dependent loads and long chains, and tile by
+// tile they were most of the time of a launch of short tiles (a phase-1 launch
+// of 7487 tiles of 2 K steps: 150 us).  Lane q holds the q-th of the next 32
+// tiles; lanes past the end hold the last tile.
+__device__ __forceinline__ TileAt look_ahead(const TcTask* tasks, int n, long long tile, long long total, int lane,
+                                             int prev) {
+  const long long mine = tile + (long long)lane * gridDim.x;
+  return tile_at(tasks, n, mine < total ? mine : total - 1, prev);
+}
+
+__device__ __forceinline__ int pick(int v, int q) { return __shfl_sync(0xffffffffu, v, q); }
 
 // Writes one accumulator row segment (32 FP32 values of row `roff`,
 // columns c0 .. c0 + nv - 1) in the task's output mode.
@@ -555,38 +563,50 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
   fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0) {
-    if (lane == 0) {  // TMA producer
-      uint32_t it = 0;
-      int ti = 0, prefetched = -1;
-      for (long long tile = blockIdx.x; tile < total && !*s_abort; tile += gridDim.x) {
-        ti = next_tc(tasks, ntasks, tile, ti);
-        const TcTask* T = &tasks[ti];
-        if (prefetched < ti) {
-          // descriptors of this task and of the next one
-          if (prefetched < ti - 1 || prefetched < 0) prefetch_maps(T, SPLIT);
-          if (ti + 1 < ntasks) prefetch_maps(&tasks[ti + 1], SPLIT);
-          prefetched = ti + 1;
+  if (warp == 0) {   // TMA producer: all lanes look ahead, lane 0 issues
+    uint32_t it = 0;
+    int q = 0, prev = 0;
+    TileAt L;
+    // K runs of this lane's tile: the open run (first column rx, steps
+    // rs0 .. rs1 - 1) and the next one's entries
+    const int* Lkr = nullptr;
+    int Lnkr = 0, Lr = 0, Lrx = 0, Lrs0 = 0, Lrs1 = 0, Lnx = 0, Lns1 = 0;
+    for (long long tile = blockIdx.x; tile < total; tile += gridDim.x, q = (q + 1) & 31) {
+      if (q == 0) {
+        L = look_ahead(tasks, ntasks, tile, total, lane, prev);
+        prev = pick(L.ti, 31);
+        const TcTask* T = &tasks[L.ti];
+        if (lane < 3) prefetch_maps(T, SPLIT);
+        Lkr = T->kr;
+        Lr = Lrx = Lrs0 = Lnx = Lns1 = 0;
+        Lrs1 = 0x7fffffff;
+        if (Lkr) {
+          Lnkr = T->nkr;
+          Lr = __ldg(Lkr + 2 * (Lnkr + 1) + L.ks);
+          Lrx = __ldg(Lkr + 2 * Lr);
+          Lrs0 = __ldg(Lkr + 2 * Lr + 1);
+          Lrs1 = __ldg(Lkr + 2 * Lr + 3);
+          if (Lr + 1 < Lnkr) { Lnx = __ldg(Lkr + 2 * Lr + 2); Lns1 = __ldg(Lkr + 2 * Lr + 5); }
         }
-        const TileCoord tc = tile_coord(T, tile);
-        const int kt0 = tc.ks * T->kchunk;
-        const int nk = min(T->ksteps, kt0 + T->kchunk) - kt0;
-        const int row0 = tc.tmi * 128, col0 = tc.tni * T->ntile;
-        const uint32_t bbytes = (uint32_t)T->ntile * 128u;
-        // K runs: the open run (first column rx, steps rs0 .. rs1 - 1) and
-        // the next one's entries, loaded a run ahead
-        const int* kr = T->kr;
-        int r = 0, rx = 0, rs0 = 0, rs1 = 0x7fffffff, nx = 0, ns1 = 0;
-        if (kr) {
-          r = __ldg(kr + 2 * (T->nkr + 1) + tc.ks);
-          rx = __ldg(kr + 2 * r);
-          rs0 = __ldg(kr + 2 * r + 1);
-          rs1 = __ldg(kr + 2 * r + 3);
-          if (r + 1 < T->nkr) { nx = __ldg(kr + 2 * r + 2); ns1 = __ldg(kr + 2 * r + 5); }
-        }
-        for (int j = 0; j < nk; ++j, ++it) {
+      } else if (q + 2 < 32) {   // descriptors two tiles ahead (the last lanes repeat the last tile)
+        const int t1 = pick(L.ti, q + 1), t2 = pick(L.ti, q + 2);
+        if (lane == 0 && t2 != t1) prefetch_maps(&tasks[t2], SPLIT);
+      }
+      const TcTask* T = &tasks[pick(L.ti, q)];
+      const int row0 = pick(L.row0, q), col0 = pick(L.col0, q), tb = pick(L.b, q);
+      const int kt0 = pick(L.kt0, q), nk = pick(L.nk, q);
+      const uint32_t bbytes = (uint32_t)pick(L.ntile, q) * 128u;
+      int r = pick(Lr, q), rx = pick(Lrx, q), rs0 = pick(Lrs0, q), rs1 = pick(Lrs1, q), nx = pick(Lnx, q),
+          ns1 = pick(Lns1, q);
+      const int* kr = (const int*)__shfl_sync(0xffffffffu, (unsigned long long)Lkr, q);
+      const int nkr = pick(Lnkr, q);
+      int go = 1;
+      if (lane == 0) {
+        if (*s_abort) go = 0;
+        const int a3 = T->a3d, b3 = T->b3d;
+        for (int j = 0; j < nk && go; ++j, ++it) {
           const uint32_t s = it % NST, ph = (it / NST) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, err, 1, wait_ns)) { *s_abort = 1; break; }
+          if (!mbar_wait(&empty[s], ph ^ 1u, err, 1, wait_ns)) { *s_abort = 1; go = 0; break; }
           uint8_t* st = smem + s * SB;
           const int g = kt0 + j;
           int kx = g * KT;
@@ -596,19 +616,22 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
               rx = nx;
               rs0 = rs1;
               rs1 = ns1;
-              if (r + 1 < T->nkr) { nx = __ldg(kr + 2 * r + 2); ns1 = __ldg(kr + 2 * r + 5); }
+              if (r + 1 < nkr) { nx = __ldg(kr + 2 * r + 2); ns1 = __ldg(kr + 2 * r + 5); }
             }
             kx = rx + (g - rs0) * KT;
           }
           mbar_expect_tx(&full[s], (SPLIT ? 2u : 1u) * (A_BYTES + bbytes));
-          tma_load(st, &T->ma, &full[s], kx, row0, tc.b, T->a3d);
-          tma_load(st + A_BYTES, &T->mb, &full[s], kx, col0, tc.b, T->b3d);
+          tma_load(st, &T->ma, &full[s], kx, row0, tb, a3);
+          tma_load(st + A_BYTES, &T->mb, &full[s], kx, col0, tb, b3);
           if (SPLIT) {
-            tma_load(st + A_BYTES + BB, &T->ma2, &full[s], kx, row0, tc.b, T->a3d);
-            tma_load(st + 2 * A_BYTES + BB, &T->mb2, &full[s], kx, col0, tc.b, T->b3d);
+            tma_load(st + A_BYTES + BB, &T->ma2, &full[s], kx, row0, tb, a3);
+            tma_load(st + 2 * A_BYTES + BB, &T->mb2, &full[s], kx, col0, tb, b3);
           }
         }
       }
+      if (!pick(go, 0)) break;
+    }
+    if (lane == 0) {
       // Before the CTA exits, every TMA load this thread issued must have
       // landed, whichever warp stopped the loop and when: only the last NST
       // fills can still be in flight (each earlier stage was re-armed only
@@ -617,44 +640,52 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
       const uint32_t first = it > (uint32_t)NST ? it - (uint32_t)NST : 0u;
       for (uint32_t j = first; j < it; ++j) mbar_wait(&full[j % NST], (j / NST) & 1u, err, 5, DRAIN_NS);
     }
-  } else if (warp == 1) {
-    if (lane == 0) {  // MMA issuer
-      uint32_t it = 0, tcount = 0;
-      int ti = 0;
-      for (long long tile = blockIdx.x; tile < total && !*s_abort; tile += gridDim.x, ++tcount) {
-        ti = next_tc(tasks, ntasks, tile, ti);
-        const TcTask* T = &tasks[ti];
-        const TileCoord tc = tile_coord(T, tile);
-        const int kt0 = tc.ks * T->kchunk;
-        const int nk = min(T->ksteps, kt0 + T->kchunk) - kt0;
+    __syncwarp();
+  } else if (warp == 1) {   // MMA issuer: all lanes look ahead, lane 0 issues
+    uint32_t it = 0, tcount = 0;
+    int q = 0, prev = 0;
+    TileAt L;
+    for (long long tile = blockIdx.x; tile < total; tile += gridDim.x, ++tcount, q = (q + 1) & 31) {
+      if (q == 0) {
+        L = look_ahead(tasks, ntasks, tile, total, lane, prev);
+        prev = pick(L.ti, 31);
+      }
+      const int nk = pick(L.nk, q), ntile = pick(L.ntile, q);
+      int go = 1;
+      if (lane == 0) {
         const uint32_t buf = tcount & 1u;
         const uint32_t acc = tmem + buf * ACC_COLS;
-        if (!mbar_wait(&acc_empty[buf], ((tcount >> 1) & 1u) ^ 1u, err, 4, wait_ns)) { *s_abort = 1; break; }
-        fence_after();
-        const uint32_t id = idesc<PREC>(128, T->ntile);
-        bool ok = true;
-        for (int j = 0; j < nk; ++j, ++it) {
-          const uint32_t s = it % NST, ph = (it / NST) & 1u;
-          if (!mbar_wait(&full[s], ph, err, 2, wait_ns)) { ok = false; break; }
+        if (*s_abort) go = 0;
+        else if (!mbar_wait(&acc_empty[buf], ((tcount >> 1) & 1u) ^ 1u, err, 4, wait_ns)) { *s_abort = 1; go = 0; }
+        if (go) {
           fence_after();
-          uint8_t* st = smem + s * SB;
-          const uint64_t a = sdesc(st);
-          const uint64_t b = sdesc(st + A_BYTES);
+          const uint32_t id = idesc<PREC>(128, ntile);
+          for (int j = 0; j < nk; ++j, ++it) {
+            const uint32_t s = it % NST, ph = (it / NST) & 1u;
+            if (!mbar_wait(&full[s], ph, err, 2, wait_ns)) { go = 0; break; }
+            fence_after();
+            uint8_t* st = smem + s * SB;
+            const uint64_t a = sdesc(st);
+            const uint64_t b = sdesc(st + A_BYTES);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a + 2 * kk, b + 2 * kk, id, (j > 0 || kk > 0) ? 1u : 0u);
-          if (SPLIT) {
-            const uint64_t a2 = sdesc(st + A_BYTES + BB);
-            const uint64_t b2 = sdesc(st + 2 * A_BYTES + BB);
+            for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a + 2 * kk, b + 2 * kk, id, (j > 0 || kk > 0) ? 1u : 0u);
+            if (SPLIT) {
+              const uint64_t a2 = sdesc(st + A_BYTES + BB);
+              const uint64_t b2 = sdesc(st + 2 * A_BYTES + BB);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a + 2 * kk, b2 + 2 * kk, id, 1u);
+              for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a + 2 * kk, b2 + 2 * kk, id, 1u);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a2 + 2 * kk, b + 2 * kk, id, 1u);
+              for (int kk = 0; kk < 4; ++kk) umma<PREC>(acc, a2 + 2 * kk, b + 2 * kk, id, 1u);
+            }
+            umma_commit(&empty[s]);
           }
-          umma_commit(&empty[s]);
+          umma_commit(&acc_full[buf]);
+          if (!go) *s_abort = 1;
         }
-        umma_commit(&acc_full[buf]);
-        if (!ok) { *s_abort = 1; break; }
       }
+      if (!pick(go, 0)) break;
+    }
+    if (lane == 0) {
       // Every product this thread issued completes before tensor memory is
       // freed and the shared-memory stages they read are released, also when
       // an epilogue warp stopped early (on the normal path the epilogue has
@@ -662,6 +693,7 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
       umma_commit(drain);
       mbar_wait(drain, 0u, err, 6, DRAIN_NS);
     }
+    __syncwarp();
   } else {
     // epilogue: warp w drains tensor-memory lanes 32 (w % 4) .. + 31 (the
     // lanes its position in the warpgroup may access); with eight epilogue
@@ -671,30 +703,35 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
     const int half = (warp - 2) >> 2;
     uint8_t* stg = smem + RING_BYTES + 256 + (warp - 2) * STG_WARP;
     uint32_t tcount = 0;
-    int ti = 0;
-    for (long long tile = blockIdx.x; tile < total; tile += gridDim.x, ++tcount) {
-      ti = next_tc(tasks, ntasks, tile, ti);
-      const TcTask* T = &tasks[ti];
-      const TileCoord tc = tile_coord(T, tile);
-      const int row0 = tc.tmi * 128, col0 = tc.tni * T->ntile;
-      const int ntile = T->ntile;
+    int q = 0, prev = 0;
+    TileAt L;
+    for (long long tile = blockIdx.x; tile < total; tile += gridDim.x, ++tcount, q = (q + 1) & 31) {
+      if (q == 0) {
+        L = look_ahead(tasks, ntasks, tile, total, lane, prev);
+        prev = pick(L.ti, 31);
+      }
+      const TcTask* T = &tasks[pick(L.ti, q)];
+      const int row0 = pick(L.row0, q), col0 = pick(L.col0, q), ntile = pick(L.ntile, q);
+      const int tb = pick(L.b, q), tks = pick(L.ks, q);
       const uint32_t buf = tcount & 1u;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (tcount >> 1) & 1u, err, 3, wait_ns));
-      if (!ok || *s_abort) { *s_abort = 1; break; }
-      fence_after();
+      // the task's fields are fetched while its products run
       const int row = row0 + quarter * 32 + lane;
       const uint32_t taddr = tmem + buf * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
       const bool live = row < T->m;
       const bool pieces = T->npc > 0;
+      const int tn = T->n;
       long long roff = 0;
       if (live)
         roff = pieces ? (long long)(row % T->rpb) * T->ldc
-                      : (long long)tc.b * T->cbatch + (long long)tc.ks * T->kstride +
+                      : (long long)tb * T->cbatch + (long long)tks * T->kstride +
                             (long long)(row / T->rpb) * T->bstride + (long long)(row % T->rpb) * T->ldc;
       const int wch = live ? row / T->rpb : 0;
       const bool staged = pieces && T->mode != 2;
       PieceTile PT;
       if (staged) piece_tile(T, row0 + quarter * 32, lane, PT);
+      const bool ok = mbar_wait(&acc_full[buf], (tcount >> 1) & 1u, err, 3, wait_ns);
+      if (__any_sync(0xffffffffu, !ok || *s_abort)) { *s_abort = 1; break; }   // the warp as a whole
+      fence_after();
       for (int cb = 32 * half; cb < ntile; cb += 32 * NHALF) {
         uint32_t v[32];
         tmem_ld32(taddr + cb, v);
@@ -704,7 +741,7 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
         }
         if (!live) continue;
         const int c0 = col0 + cb;
-        const int nv = min(32, T->n - c0);
+        const int nv = min(32, tn - c0);
         if (nv <= 0) continue;
         if (pieces) store_row_pieces(T, roff, wch, c0, nv, v);
         else store_row(T, roff, c0, nv, v);
