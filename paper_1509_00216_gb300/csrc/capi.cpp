@@ -655,6 +655,7 @@ mpslcc_status mpslcc_get_stats(mpslcc_ctx* ctx, mpslcc_stats* out) {
   return guard(ctx, [&](Ctx& c) {
     MPSLCC_REQUIRE(out, ST_ARG, "null output");
     std::memset(out, 0, sizeof(*out));
+    settle_sigma(c);
     out->sigma_flops = c.st.sigma_flops;
     out->sigma_seconds = c.st.sigma_seconds;
     out->sigma_calls = c.st.sigma_calls;

@@ -204,14 +204,21 @@ void run_copies(Ctx& c, std::vector<CopyTask>& t) {
   c.st.kernel_launches++;
 }
 
-static unsigned int* dot_ticket(Ctx& c) {
+Reduction reduction(Ctx& c) {
   if (!c.red_ticket.p) {
-    c.red_ticket.alloc(&c, 256);
-    cuda_check(cudaMemsetAsync(c.red_ticket.p, 0, 256, c.s()), "dot ticket");
+    c.red_ticket.alloc(&c, MD_TICKETS * sizeof(unsigned int));
+    cuda_check(cudaMemsetAsync(c.red_ticket.p, 0, MD_TICKETS * sizeof(unsigned int), c.s()), "dot tickets");
   }
   c.red.ensure(&c, 4096 * sizeof(double));
   c.red_out.ensure(&c, 256 * sizeof(double));
-  return (unsigned int*)c.red_ticket.p;
+  return {c.red.d(), (unsigned int*)c.red_ticket.p, c.out_dev->red};
+}
+
+void wait_dots(Ctx& c, double* r1, double* r2) {
+  cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
+  check_f64(c);
+  *r1 = c.out->red[0];
+  if (r2) *r2 = c.out->red[1];
 }
 
 double dev_dot(Ctx& c, const double* x, const double* y, long n) {
@@ -224,20 +231,17 @@ void dev_dot2(Ctx& c, const double* x1, const double* y1, const double* x2, cons
               double* r2) {
   *r1 = *r2 = 0.0;
   if (n <= 0) return;
-  unsigned int* tk = dot_ticket(c);
-  launch_dot_fused(x1, y1, x2, y2, n, c.out_dev->red, c.red.d(), tk, c.s());
+  const Reduction R = reduction(c);
+  launch_dot_fused(x1, y1, x2, y2, n, R.out, R.part, R.ticket, c.s());
   c.st.kernel_launches++;
-  cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
-  check_f64(c);
-  *r1 = c.out->red[0];
-  if (x2) *r2 = c.out->red[1];
+  wait_dots(c, r1, x2 ? r2 : nullptr);
 }
 
 void dev_project(Ctx& c, const double* u, double* v, long n) {
   if (n <= 0) return;
-  unsigned int* tk = dot_ticket(c);
+  const Reduction R = reduction(c);
   double* a = c.red_out.d() + 8;   // consumed by the next launch on the stream
-  launch_dot_fused(u, v, nullptr, nullptr, n, a, c.red.d(), tk, c.s());
+  launch_dot_fused(u, v, nullptr, nullptr, n, a, R.part, R.ticket, c.s());
   launch_axpy_dev(n, a, -1.0, u, v, c.s());
   c.st.kernel_launches += 2;
 }
@@ -1177,6 +1181,15 @@ static void prepare_f64_sigma(Ctx& c, SigmaPlan& P) {
   upload_f64(p2, P.tasks2.p, c.s());
   cuda_check(cudaStreamSynchronize(c.s()), "sigma plan sync");
   P.f64_ready = true;
+}
+
+void settle_sigma(Ctx& c) {
+  if (!c.sigma_open) return;
+  c.sigma_open = false;
+  cuda_check(cudaEventSynchronize(c.ev1), "sigma sync");
+  float ms = 0;
+  cudaEventElapsedTime(&ms, c.ev0, c.ev1);
+  c.st.sigma_seconds += ms * 1e-3;
 }
 
 void sigma_apply(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {

@@ -273,6 +273,7 @@ struct Ctx {
   volatile HostOut* out = nullptr;
   HostOut* out_dev = nullptr;
   cudaMemPool_t pool = nullptr;   // of the stream-ordered allocations (no caller allocator)
+  bool sigma_open = false;   // ev0 .. ev1 bracket a local product whose time is not yet in the statistics
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_p0 = nullptr, ev_p1 = nullptr, ev_p2 = nullptr;
 
   // problem
@@ -382,6 +383,12 @@ void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t);
 void validate_gemm(const Ctx& c, const GemmTask& t);
 void validate_copy(const Ctx& c, const CopyTask& t);
 void run_copies(Ctx& c, std::vector<CopyTask>& t);
+// Adds the time of the last local product to the statistics.
+void settle_sigma(Ctx& c);
+// Scratch of a reduction whose results land in pinned host memory, and the
+// wait for them (throws what the products before it reported).
+Reduction reduction(Ctx& c);
+void wait_dots(Ctx& c, double* r1, double* r2);
 double dev_dot(Ctx& c, const double* x, const double* y, long n);
 // x1.y1 and x2.y2 in one pass (one launch, one host round trip)
 void dev_dot2(Ctx& c, const double* x1, const double* y1, const double* x2, const double* y2, long n, double* r1,

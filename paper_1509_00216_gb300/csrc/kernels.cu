@@ -95,25 +95,19 @@ __device__ __forceinline__ double block_sum(double v) {
   return v;
 }
 
-// Dots of one or two vector pairs in one launch.  Every block stores its
-// partial sums; the block that finishes last (a ticket counter) adds the
-// partials in block order, so the value does not depend on timing and equals
-// a reduction of the partials by one block per output.
-__global__ void dot_fused(const double* __restrict__ x1, const double* __restrict__ y1,
-                          const double* __restrict__ x2, const double* __restrict__ y2, long n,
-                          double* __restrict__ part, unsigned int* ticket, double* __restrict__ out) {
-  const bool two = x2 != nullptr;
-  double s1 = 0.0, s2 = 0.0;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    s1 = fma(x1[i], y1[i], s1);
-    if (two) s2 = fma(x2[i], y2[i], s2);
-  }
+// Ends a reduction over RED_BLOCKS blocks of RED_T threads.  Every block stores
+// its partial sums; the block that finishes last (a ticket counter) adds the
+// partials in block order, so the value does not depend on timing.  Short
+// vectors launch only the blocks that hold elements; the others' partials are
+// the zeros they would have stored.
+__device__ __forceinline__ void finish_dots(double s1, double s2, bool two, double* __restrict__ part,
+                                            unsigned int* ticket, double* __restrict__ out) {
   s1 = block_sum(s1);
   if (two) s2 = block_sum(s2);
   __shared__ unsigned int tk;
   if (threadIdx.x == 0) {
     part[blockIdx.x] = s1;
-    if (two) part[gridDim.x + blockIdx.x] = s2;
+    if (two) part[RED_BLOCKS + blockIdx.x] = s2;
     __threadfence();
     tk = atomicAdd(ticket, 1u);
   }
@@ -122,9 +116,9 @@ __global__ void dot_fused(const double* __restrict__ x1, const double* __restric
   __threadfence();
   const volatile double* vp = part;
   double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += RED_T) {
     a += vp[i];
-    if (two) b += vp[gridDim.x + i];
+    if (two) b += vp[RED_BLOCKS + i];
   }
   a = block_sum(a);
   if (two) b = block_sum(b);
@@ -132,6 +126,98 @@ __global__ void dot_fused(const double* __restrict__ x1, const double* __restric
     out[0] = a;
     if (two) out[1] = b;
     *ticket = 0u;
+  }
+}
+
+// The vector steps of the local solvers are bound by their launches and the
+// waits between them (2.4 to 11 us each at up to 2e5 elements, five launches
+// and two copies a CG iteration), so each is one pass that ends in the dots it
+// needs (a six-site program of 1300 local products: 128 -> 110 ms); element i goes to thread i mod (RED_BLOCKS RED_T) in
+// ascending order whatever the pass, so every dot keeps its value.
+#define RED_LOOP(i, n) \
+  for (long i = blockIdx.x * (long)RED_T + threadIdx.x; i < n; i += (long)RED_BLOCKS * RED_T)
+
+// Dots of one or two vector pairs.
+__global__ void dot_fused(const double* __restrict__ x1, const double* __restrict__ y1,
+                          const double* __restrict__ x2, const double* __restrict__ y2, long n,
+                          double* __restrict__ part, unsigned int* ticket, double* __restrict__ out) {
+  const bool two = x2 != nullptr;
+  double s1 = 0.0, s2 = 0.0;
+  RED_LOOP(i, n) {
+    s1 = fma(x1[i], y1[i], s1);
+    if (two) s2 = fma(x2[i], y2[i], s2);
+  }
+  finish_dots(s1, s2, two, part, ticket, out);
+}
+
+// y -= shift q, then p . y
+__global__ void shift_dot_kernel(long n, double shift, const double* __restrict__ q, double* __restrict__ y,
+                                 const double* __restrict__ p, double* __restrict__ part, unsigned int* ticket,
+                                 double* __restrict__ out) {
+  double s = 0.0;
+  RED_LOOP(i, n) {
+    const double v = fma(-shift, q[i], y[i]);
+    y[i] = v;
+    s = fma(p[i], v, s);
+  }
+  finish_dots(s, 0.0, false, part, ticket, out);
+}
+
+__device__ __forceinline__ double precond_den(double d, double shift, double fl, int absval) {
+  double den = d - shift;
+  if (absval) den = fmax(fabs(den), fl);
+  else if (fabs(den) < fl) den = (den < 0.0) ? -fl : fl;
+  return den;
+}
+
+// One CG update: x += alpha p, r -= alpha ap, z = r / max(|d - shift|, fl),
+// then r . z and r . r
+__global__ void cg_update_kernel(long n, double alpha, const double* __restrict__ p, const double* __restrict__ ap,
+                                 double* __restrict__ x, double* __restrict__ r, const double* __restrict__ d,
+                                 double shift, double fl, double* __restrict__ z, double* __restrict__ part,
+                                 unsigned int* ticket, double* __restrict__ out) {
+  double s1 = 0.0, s2 = 0.0;
+  RED_LOOP(i, n) {
+    x[i] = fma(alpha, p[i], x[i]);
+    const double ri = fma(-alpha, ap[i], r[i]);
+    const double zi = ri / precond_den(d[i], shift, fl, 1);
+    r[i] = ri;
+    z[i] = zi;
+    s1 = fma(ri, zi, s1);
+    s2 = fma(ri, ri, s2);
+  }
+  finish_dots(s1, s2, true, part, ticket, out);
+}
+
+struct LincombArgs { double c[LINCOMB_ARGS]; };
+
+// Ritz vector xs = sum_j c_j V_j and residual r = sum_j c_j AV_j - theta xs, then r . r
+__global__ void ritz_kernel(long n, int m, const double* __restrict__ V, const double* __restrict__ AV, long ld,
+                            const __grid_constant__ LincombArgs coef, double theta, double* __restrict__ xs,
+                            double* __restrict__ r, double* __restrict__ part, unsigned int* ticket,
+                            double* __restrict__ out) {
+  double s = 0.0;
+  RED_LOOP(i, n) {
+    double x = 0.0, a = 0.0;
+    for (int j = 0; j < m; ++j) {
+      x = fma(coef.c[j], V[j * ld + i], x);
+      a = fma(coef.c[j], AV[j * ld + i], a);
+    }
+    a = fma(-theta, x, a);
+    xs[i] = x;
+    r[i] = a;
+    s = fma(a, a, s);
+  }
+  finish_dots(s, 0.0, false, part, ticket, out);
+}
+
+// t -= sum_j c_j V_j with the coefficients on the device
+__global__ void gs_kernel(long n, int m, const double* __restrict__ V, long ld, const double* __restrict__ c,
+                          double* __restrict__ t) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int j = 0; j < m; ++j) s = fma(-c[j], V[j * ld + i], s);
+    t[i] += s;
   }
 }
 
@@ -143,29 +229,39 @@ __global__ void axpy_dev_kernel(long n, const double* __restrict__ a, double sgn
     y[i] = fma(cf, x[i], y[i]);
 }
 
-__global__ void multidot_partial(const double* __restrict__ V, long ld, const double* __restrict__ x,
-                                 long n, double* __restrict__ part) {
+// proj[j] = <V_j, x>: MD_BLOCKS blocks per vector, the last one of each vector
+// (a ticket per vector) adds its partials.
+constexpr int MD_BLOCKS = 64;
+__global__ void multidot_kernel(const double* __restrict__ V, long ld, const double* __restrict__ x, long n,
+                                double* __restrict__ part, unsigned int* ticket, double* __restrict__ out) {
   const double* v = V + blockIdx.y * ld;
   double s = 0.0;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    s = fma(v[i], x[i], s);
+  for (long i = blockIdx.x * (long)RED_T + threadIdx.x; i < n; i += (long)MD_BLOCKS * RED_T) s = fma(v[i], x[i], s);
   s = block_sum(s);
-  if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+  __shared__ unsigned int tk;
+  if (threadIdx.x == 0) {
+    part[blockIdx.y * MD_BLOCKS + blockIdx.x] = s;
+    __threadfence();
+    tk = atomicAdd(ticket + blockIdx.y, 1u);
+  }
+  __syncthreads();
+  if (tk != gridDim.x - 1) return;
+  __threadfence();
+  const volatile double* vp = part + blockIdx.y * MD_BLOCKS;
+  double a = threadIdx.x < gridDim.x ? 0.0 + vp[threadIdx.x] : 0.0;
+  a = block_sum(a);
+  if (threadIdx.x == 0) {
+    out[blockIdx.y] = a;
+    ticket[blockIdx.y] = 0u;
+  }
 }
 
-__global__ void reduce_partials(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) s += part[blockIdx.x * nb + i];
-  s = block_sum(s);
-  if (threadIdx.x == 0) out[blockIdx.x] = s;
-}
-
-__global__ void axpby_kernel(long n, double a, const double* __restrict__ x, double b, double* __restrict__ y,
+__global__ void axpby_kernel(long n, double a, const double* x, double b, double* y,
                              int mode) {
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     if (mode == 0) y[i] = fma(a, x[i], y[i]);
     else if (mode == 1) y[i] = a * x[i] + b * y[i];
-    else if (mode == 2) y[i] *= a;
+    else if (mode == 2) y[i] = a * x[i];
     else y[i] = a;
   }
 }
@@ -173,10 +269,7 @@ __global__ void axpby_kernel(long n, double a, const double* __restrict__ x, dou
 __global__ void precond_kernel(long n, const double* __restrict__ x, const double* __restrict__ d, double shift,
                                double fl, double* __restrict__ y, int absval) {
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    double den = d[i] - shift;
-    if (absval) den = fmax(fabs(den), fl);
-    else if (fabs(den) < fl) den = (den < 0.0) ? -fl : fl;
-    y[i] = x[i] / den;
+    y[i] = x[i] / precond_den(d[i], shift, fl, absval);
   }
 }
 
@@ -189,7 +282,6 @@ __global__ void lincomb_kernel(long n, int m, const double* __restrict__ V, long
   }
 }
 
-struct LincombArgs { double c[LINCOMB_ARGS]; };
 __global__ void lincomb_args_kernel(long n, int m, const double* __restrict__ V, long ld,
                                     const __grid_constant__ LincombArgs coef, double* __restrict__ out) {
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
@@ -247,6 +339,9 @@ __global__ void f32_to_f64_kernel(long n, const float* __restrict__ x, double* _
     y[i] = (double)x[i];
 }
 
+inline int red_grid(long n, int blocks) {
+  return (int)std::max(1L, std::min((n + RED_T - 1) / RED_T, (long)blocks));
+}
 inline int elem_grid(long n) {
   long g = (n + 255) / 256;
   return (int)std::max(1L, std::min(g, 152L * 16));
@@ -294,7 +389,29 @@ void launch_copy_f64(const CopyTask* d_tasks, int ntasks, long long total, cudaS
 
 void launch_dot_fused(const double* x1, const double* y1, const double* x2, const double* y2, long n, double* d_out,
                       double* d_part, unsigned int* d_ticket, cudaStream_t s) {
-  dot_fused<<<RED_BLOCKS, RED_T, 0, s>>>(x1, y1, x2, y2, n, d_part, d_ticket, d_out);
+  dot_fused<<<red_grid(n, RED_BLOCKS), RED_T, 0, s>>>(x1, y1, x2, y2, n, d_part, d_ticket, d_out);
+}
+
+void launch_shift_dot(long n, double shift, const double* q, double* y, const double* p, const Reduction& R,
+                      cudaStream_t s) {
+  shift_dot_kernel<<<red_grid(n, RED_BLOCKS), RED_T, 0, s>>>(n, shift, q, y, p, R.part, R.ticket, R.out);
+}
+
+void launch_cg_update(long n, double alpha, const double* p, const double* ap, double* x, double* r, const double* d,
+                      double shift, double fl, double* z, const Reduction& R, cudaStream_t s) {
+  cg_update_kernel<<<red_grid(n, RED_BLOCKS), RED_T, 0, s>>>(n, alpha, p, ap, x, r, d, shift, fl, z, R.part, R.ticket,
+                                                             R.out);
+}
+
+void launch_ritz(long n, int m, const double* V, const double* AV, long ld, const double* coef, double theta,
+                 double* xs, double* r, const Reduction& R, cudaStream_t s) {
+  LincombArgs a;
+  for (int j = 0; j < LINCOMB_ARGS; ++j) a.c[j] = j < m ? coef[j] : 0.0;
+  ritz_kernel<<<red_grid(n, RED_BLOCKS), RED_T, 0, s>>>(n, m, V, AV, ld, a, theta, xs, r, R.part, R.ticket, R.out);
+}
+
+void launch_gs(long n, int m, const double* V, long ld, const double* d_coef, double* t, cudaStream_t s) {
+  gs_kernel<<<elem_grid(n), 256, 0, s>>>(n, m, V, ld, d_coef, t);
 }
 
 void launch_axpy_dev(long n, const double* d_a, double sgn, const double* x, double* y, cudaStream_t s) {
@@ -302,11 +419,10 @@ void launch_axpy_dev(long n, const double* d_a, double sgn, const double* x, dou
 }
 
 void launch_multidot(long n, int m, const double* V, long ld, const double* x, double* d_out, double* d_part,
-                     cudaStream_t s) {
-  if (m <= 0) return;
-  const int nb = 64;
-  multidot_partial<<<dim3(nb, m), RED_T, 0, s>>>(V, ld, x, n, d_part);
-  reduce_partials<<<m, RED_T, 0, s>>>(d_part, nb, d_out);
+                     unsigned int* d_tickets, cudaStream_t s) {
+  for (int j = 0; j < m; j += MD_TICKETS)
+    multidot_kernel<<<dim3(red_grid(n, MD_BLOCKS), std::min(m - j, MD_TICKETS)), RED_T, 0, s>>>(
+        V + j * ld, ld, x, n, d_part + (long)j * MD_BLOCKS, d_tickets, d_out + j);
 }
 
 void launch_axpy(long n, double a, const double* x, double* y, cudaStream_t s) {
@@ -315,8 +431,8 @@ void launch_axpy(long n, double a, const double* x, double* y, cudaStream_t s) {
 void launch_axpby(long n, double a, const double* x, double b, double* y, cudaStream_t s) {
   axpby_kernel<<<elem_grid(n), 256, 0, s>>>(n, a, x, b, y, 1);
 }
-void launch_scale(long n, double a, double* x, cudaStream_t s) {
-  axpby_kernel<<<elem_grid(n), 256, 0, s>>>(n, a, nullptr, 0.0, x, 2);
+void launch_scale(long n, double a, const double* x, double* y, cudaStream_t s) {
+  axpby_kernel<<<elem_grid(n), 256, 0, s>>>(n, a, x, 0.0, y, 2);
 }
 void launch_fill(long n, double v, double* x, cudaStream_t s) {
   axpby_kernel<<<elem_grid(n), 256, 0, s>>>(n, v, nullptr, 0.0, x, 3);

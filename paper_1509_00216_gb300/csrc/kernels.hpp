@@ -91,12 +91,25 @@ void launch_copy_f64(const CopyTask* d_tasks, int ntasks, long long total_tiles,
 // x1.y1 (and x2.y2 when x2 is not null) in one launch into d_out[0] (and
 // d_out[1]); d_partial holds 2 x 512 doubles, d_ticket one zeroed counter
 // (left zeroed)
+struct Reduction { double* part; unsigned int* ticket; double* out; };
 void launch_dot_fused(const double* x1, const double* y1, const double* x2, const double* y2, long n, double* d_out,
                       double* d_partial, unsigned int* d_ticket, cudaStream_t s);
+// Vector steps of the local solvers, each ending in dots (into R.out):
+// y -= shift q; p.y
+void launch_shift_dot(long n, double shift, const double* q, double* y, const double* p, const Reduction& R,
+                      cudaStream_t s);
+// x += alpha p; r -= alpha ap; z = r / max(|d - shift|, fl); r.z, r.r
+void launch_cg_update(long n, double alpha, const double* p, const double* ap, double* x, double* r, const double* d,
+                      double shift, double fl, double* z, const Reduction& R, cudaStream_t s);
+// xs = sum_j coef[j] V_j; r = sum_j coef[j] AV_j - theta xs; r.r  (m <= LINCOMB_ARGS)
+void launch_ritz(long n, int m, const double* V, const double* AV, long ld, const double* coef, double theta,
+                 double* xs, double* r, const Reduction& R, cudaStream_t s);
+// t -= sum_j d_coef[j] V_j
+void launch_gs(long n, int m, const double* V, long ld, const double* d_coef, double* t, cudaStream_t s);
 void launch_axpy_dev(long n, const double* d_a, double sgn, const double* x, double* y, cudaStream_t s);  // y += sgn*(*d_a) x
 void launch_axpy(long n, double a, const double* x, double* y, cudaStream_t s);   // y += a x
 void launch_axpby(long n, double a, const double* x, double b, double* y, cudaStream_t s);  // y = a x + b y
-void launch_scale(long n, double a, double* x, cudaStream_t s);
+void launch_scale(long n, double a, const double* x, double* y, cudaStream_t s);   // y = a x (y may be x)
 void launch_fill(long n, double v, double* x, cudaStream_t s);
 // Diagonal preconditioner y = x / (d - shift), the denominator kept away from
 // zero by `floor_` (sign kept) or, with absval, replaced by max(|d-shift|, floor_).
@@ -108,9 +121,11 @@ void launch_lincomb(long n, int m, const double* V, long ld, const double* d_coe
 // The same with the coefficients (host, m <= LINCOMB_ARGS) as launch arguments.
 constexpr int LINCOMB_ARGS = 64;
 void launch_lincomb_args(long n, int m, const double* V, long ld, const double* coef, double* out, cudaStream_t s);
-// proj[j] = <V_j, x> for j < m (batched dots), written to d_out[0..m)
-void launch_multidot(long n, int m, const double* V, long ld, const double* x, double* d_out,
-                     double* d_partial, cudaStream_t s);
+// proj[j] = <V_j, x> for j < m (batched dots), written to d_out[0..m);
+// d_partial holds 64 m doubles, d_tickets MD_TICKETS zeroed counters (left zeroed)
+constexpr int MD_TICKETS = 512;
+void launch_multidot(long n, int m, const double* V, long ld, const double* x, double* d_out, double* d_partial,
+                     unsigned int* d_tickets, cudaStream_t s);
 
 // Fixed-order reduction of split-K partial products into an FP64 output
 // segment: out[out_off + r * n + c] = sum_{j < nsplit} part[part_off + j *

@@ -40,11 +40,12 @@ void copyv(Ctx& c, double* dst, const double* src, long n) {
 std::vector<double> multidot(Ctx& c, const double* V, long ld, int m, const double* x, long n) {
   std::vector<double> out(m);
   if (m == 0) return out;
+  const Reduction R = reduction(c);
   c.red.ensure(&c, std::max<size_t>(4096, (size_t)m * 64) * sizeof(double));
   const bool host = m <= 256;   // results straight to pinned host memory
   if (!host) c.red_out.ensure(&c, m * sizeof(double));
-  launch_multidot(n, m, V, ld, x, host ? c.out_dev->red : c.red_out.d(), c.red.d(), c.s());
-  c.st.kernel_launches += 2;
+  launch_multidot(n, m, V, ld, x, host ? R.out : c.red_out.d(), c.red.d(), R.ticket, c.s());
+  c.st.kernel_launches++;
   if (!host)
     cuda_check(cudaMemcpyAsync(out.data(), c.red_out.p, m * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "mdot");
   cuda_check(cudaStreamSynchronize(c.s()), "mdot sync");
@@ -52,6 +53,16 @@ std::vector<double> multidot(Ctx& c, const double* V, long ld, int m, const doub
   if (host)
     for (int j = 0; j < m; ++j) out[j] = c.out->red[j];
   return out;
+}
+
+// t -= sum_j <V_j, t> V_j, the overlaps staying on the device
+void orthogonalise(Ctx& c, const double* V, long ld, int m, double* t, long n) {
+  const Reduction R = reduction(c);
+  c.red.ensure(&c, std::max<size_t>(4096, (size_t)m * 64) * sizeof(double));
+  c.red_out.ensure(&c, std::max(256, m) * sizeof(double));
+  launch_multidot(n, m, V, ld, t, c.red_out.d(), c.red.d(), R.ticket, c.s());
+  launch_gs(n, m, V, ld, c.red_out.d(), t, c.s());
+  c.st.kernel_launches += 2;
 }
 
 // out = sum_j coef[j] V_j
@@ -106,14 +117,14 @@ void jacobi_eigh(int n, std::vector<double>& A, std::vector<double>& w, std::vec
   for (int i = 0; i < n; ++i) w[i] = A[i * n + i];
 }
 
+// Its time is read when the next one begins or the statistics are asked for:
+// the dots that follow a product wait for it anyway.
 void sigma_timed(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
+  settle_sigma(c);
   cudaEventRecord(c.ev0, c.s());
   sigma_apply(c, P, x, y, prec);
   cudaEventRecord(c.ev1, c.s());
-  cuda_check(cudaEventSynchronize(c.ev1), "sigma sync");
-  float ms = 0;
-  cudaEventElapsedTime(&ms, c.ev0, c.ev1);
-  c.st.sigma_seconds += ms * 1e-3;
+  c.sigma_open = true;
 }
 
 // Davidson for the lowest eigenpair of the local H_eff (reference, Eq. EH).
@@ -135,7 +146,7 @@ double davidson(Ctx& c, SigmaPlan& P, double* x, long n, const double* diag, dou
     nx = std::sqrt((double)n);
   }
   copyv(c, V, x, n);
-  launch_scale(n, 1.0 / nx, V, c.s());
+  launch_scale(n, 1.0 / nx, V, V, c.s());
   sigma_timed(c, P, V, AV, prec);
   int m = 1;
   std::vector<double> Hs(1, dev_dot(c, V, AV, n));
@@ -151,10 +162,18 @@ double davidson(Ctx& c, SigmaPlan& P, double* x, long n, const double* diag, dou
     theta = w[imin];
     y.assign(m, 0.0);
     for (int i = 0; i < m; ++i) y[i] = Ym[i * m + imin];
-    lincomb(c, V, n, m, y, xs.d(), n);
-    lincomb(c, AV, n, m, y, r.d(), n);
-    launch_axpy(n, -theta, xs.d(), r.d(), c.s());
-    double rn = vnorm(c, r);
+    double rn = 0;
+    if (m <= LINCOMB_ARGS) {
+      launch_ritz(n, m, V, AV, n, y.data(), theta, xs.d(), r.d(), reduction(c), c.s());
+      c.st.kernel_launches++;
+      wait_dots(c, &rn, nullptr);
+      rn = std::sqrt(std::max(0.0, rn));
+    } else {
+      lincomb(c, V, n, m, y, xs.d(), n);
+      lincomb(c, AV, n, m, y, r.d(), n);
+      launch_axpy(n, -theta, xs.d(), r.d(), c.s());
+      rn = vnorm(c, r);
+    }
     if (!std::isfinite(theta) || !std::isfinite(rn))
       throw Error(ST_NUMERIC, "non-finite Ritz value or residual in the Davidson solve");
     if (rn < tol || n == 1 || m >= n) {
@@ -162,19 +181,16 @@ double davidson(Ctx& c, SigmaPlan& P, double* x, long n, const double* diag, dou
       break;
     }
     launch_precond(n, r.d(), diag, theta, 1e-4, t.d(), 0, c.s());
-    for (int pass = 0; pass < 2; ++pass) {
-      std::vector<double> pr = multidot(c, V, n, m, t.d(), n);
-      for (auto& v : pr) v = -v;
-      lincomb(c, V, n, m, pr, r.d(), n);
-      launch_axpy(n, 1.0, r.d(), t.d(), c.s());
-    }
+    for (int pass = 0; pass < 2; ++pass) orthogonalise(c, V, n, m, t.d(), n);
     double tn = vnorm(c, t);
     if (tn < 1e-12) {
       *converged = rn < 1e3 * tol;
       break;
     }
-    launch_scale(n, 1.0 / tn, t.d(), c.s());
-    if (m == maxsub) {
+    if (m < maxsub) {
+      launch_scale(n, 1.0 / tn, t.d(), V + (long)m * n, c.s());
+    } else {
+      launch_scale(n, 1.0 / tn, t.d(), t.d(), c.s());
       // restart from the current Ritz vector
       copyv(c, V, xs.d(), n);
       lincomb(c, AV, n, m, y, r.d(), n);
@@ -185,9 +201,8 @@ double davidson(Ctx& c, SigmaPlan& P, double* x, long n, const double* diag, dou
       launch_axpy(n, -pr[0], V, t.d(), c.s());
       double tn2 = vnorm(c, t);
       if (tn2 < 1e-12) { *converged = true; break; }
-      launch_scale(n, 1.0 / tn2, t.d(), c.s());
+      launch_scale(n, 1.0 / tn2, t.d(), V + (long)m * n, c.s());
     }
-    copyv(c, V + (long)m * n, t.d(), n);
     sigma_timed(c, P, V + (long)m * n, AV + (long)m * n, prec);
     std::vector<double> col = multidot(c, V, n, m + 1, AV + (long)m * n, n);
     std::vector<double> H2((size_t)(m + 1) * (m + 1));
@@ -215,14 +230,27 @@ struct LinOp {
   double shift;
   const double* u;
   Vec q;
-  void apply(Ctx& c, const double* v, double* out, int prec) {
+  // out = A v, and v . out where asked for
+  void apply(Ctx& c, const double* v, double* out, int prec, double* vout = nullptr) {
     long n = P->nb;
+    if (!u) {
+      sigma_timed(c, *P, v, out, prec);
+      if (!vout) {
+        launch_axpy(n, -shift, v, out, c.s());
+        return;
+      }
+      launch_shift_dot(n, shift, v, out, v, reduction(c), c.s());
+      c.st.kernel_launches++;
+      wait_dots(c, vout, nullptr);
+      return;
+    }
     q.alloc(c, n);
     copyv(c, q.d(), v, n);
     project(c, u, q.d(), n);
     sigma_timed(c, *P, q.d(), out, prec);
     launch_axpy(n, -shift, q.d(), out, c.s());
     project(c, u, out, n);
+    if (vout) *vout = dev_dot(c, v, out, n);
   }
 };
 
@@ -262,19 +290,23 @@ double solve_linear(Ctx& c, LinOp& A, const double* b, double* x, const double* 
   int it = 0;
   *indefinite = false;
   while (rn > thr && it < maxit) {
-    A.apply(c, p.d(), Ap.d(), prec);
-    double pAp = dev_dot(c, p.d(), Ap.d(), n);
+    double pAp = 0;
+    A.apply(c, p.d(), Ap.d(), prec, &pAp);
     if (!std::isfinite(pAp)) throw Error(ST_NUMERIC, "non-finite curvature <p|A|p> in the local CG solve");
     if (!(pAp > 0)) {
       *indefinite = true;
       break;
     }
     double alpha = rz / pAp;
-    launch_axpy(n, alpha, p.d(), x, c.s());
-    launch_axpy(n, -alpha, Ap.d(), r.d(), c.s());
-    precond(r.d(), z.d());
     double rz2 = 0;
-    dev_dot2(c, r.d(), z.d(), r.d(), r.d(), n, &rz2, &rr);
+    launch_cg_update(n, alpha, p.d(), Ap.d(), x, r.d(), diag, A.shift, 1e-2, z.d(), reduction(c), c.s());
+    c.st.kernel_launches++;
+    if (A.u) {   // the projected z has dots of its own
+      project(c, A.u, z.d(), n);
+      dev_dot2(c, r.d(), z.d(), r.d(), r.d(), n, &rz2, &rr);
+    } else {
+      wait_dots(c, &rz2, &rr);
+    }
     launch_axpby(n, 1.0, z.d(), rz2 / rz, p.d(), c.s());
     rz = rz2;
     rn = std::sqrt(std::max(0.0, rr));
@@ -293,11 +325,11 @@ double solve_linear(Ctx& c, LinOp& A, const double* b, double* x, const double* 
     launch_fill(n, 0.0, w0.d(), c.s());
     launch_fill(n, 0.0, w1.d(), c.s());
     double gam0 = 1, gam1 = 1, sig0 = 0, sig1 = 0, betaold = 0;
-    if (beta > 0) launch_scale(n, 1.0 / beta, v1.d(), c.s());
+    if (beta > 0) launch_scale(n, 1.0 / beta, v1.d(), v1.d(), c.s());
     rn = beta;
     while (rn > thr && it < maxit && beta > 1e-300) {
-      A.apply(c, v1.d(), av.d(), prec);
-      double alpha = dev_dot(c, v1.d(), av.d(), n);
+      double alpha = 0;
+      A.apply(c, v1.d(), av.d(), prec, &alpha);
       if (!std::isfinite(alpha)) throw Error(ST_NUMERIC, "non-finite Lanczos coefficient in the local MINRES solve");
       launch_axpy(n, -alpha, v1.d(), av.d(), c.s());
       launch_axpy(n, -beta, v0.d(), av.d(), c.s());
@@ -315,7 +347,7 @@ double solve_linear(Ctx& c, LinOp& A, const double* b, double* x, const double* 
       copyv(c, w2.d(), v1.d(), n);
       launch_axpy(n, -r3, w0.d(), w2.d(), c.s());
       launch_axpy(n, -r2, w1.d(), w2.d(), c.s());
-      launch_scale(n, 1.0 / r1, w2.d(), c.s());
+      launch_scale(n, 1.0 / r1, w2.d(), w2.d(), c.s());
       launch_axpy(n, gam1 * eta, w2.d(), x, c.s());
       eta = -sig1 * eta;
       rn = std::fabs(eta);
@@ -324,7 +356,7 @@ double solve_linear(Ctx& c, LinOp& A, const double* b, double* x, const double* 
       std::swap(v0.b, v1.b);
       if (beta > 0) {
         copyv(c, v1.d(), av.d(), n);
-        launch_scale(n, 1.0 / beta, v1.d(), c.s());
+        launch_scale(n, 1.0 / beta, v1.d(), v1.d(), c.s());
       }
       ++it;
     }
@@ -982,7 +1014,7 @@ double lcc_local(Ctx& c, MPS& target, SigmaPlan& P11, SigmaPlan& P10, MPS& tket,
   double vn = std::sqrt(std::max(0.0, dev_dot(c, ub.d(), ub.d(), n)));
   const double* u = nullptr;
   if (vn > 1e-10 && vn * vn >= (1.0 - deficit) * n00) {
-    launch_scale(n, 1.0 / vn, ub.d(), c.s());
+    launch_scale(n, 1.0 / vn, ub.d(), ub.d(), c.s());
     u = ub.d();
   }
   project(c, u, bb.d(), n);
@@ -1305,6 +1337,7 @@ double lcc_sweeps(Ctx& c, int M1, int n_sweeps, int order) {
   cudaEventCreate(&t0);
   cudaEventCreate(&t1);
   for (int sw = 0; sw < n_sweeps; ++sw) {
+    settle_sigma(c);
     double s_sig0 = c.st.sigma_seconds, f_sig0 = c.st.sigma_flops;
     long long n_sig0 = c.st.sigma_calls, n_k0 = c.st.kernel_launches;
     cudaEventRecord(t0, c.s());
@@ -1321,6 +1354,7 @@ double lcc_sweeps(Ctx& c, int M1, int n_sweeps, int order) {
     float ms = 0;
     cudaEventElapsedTime(&ms, t0, t1);
     c.st.last_sweep_seconds = ms * 1e-3;
+    settle_sigma(c);
     c.st.last_sweep_sigma_seconds = c.st.sigma_seconds - s_sig0;
     c.st.last_sweep_sigma_flops = c.st.sigma_flops - f_sig0;
     c.st.last_sweep_sigma_calls = c.st.sigma_calls - n_sig0;
