@@ -726,7 +726,10 @@ mpslcc_status mpslcc_tc_gemm_noalloc(int device, void* stream, int prec, int m, 
 size_t mpslcc_tc_gemm_noalloc_scratch_bytes(void) { return tc_gemm_noalloc_max_bytes(); }
 
 mpslcc_status mpslcc_reset_stats(mpslcc_ctx* ctx) {
-  return guard(ctx, [&](Ctx& c) { c.st = Stats(); });
+  return guard(ctx, [&](Ctx& c) {
+    settle_sigma(c);
+    c.st = Stats();
+  });
 }
 
 }  // extern "C"
