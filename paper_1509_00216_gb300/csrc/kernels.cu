@@ -1,6 +1,7 @@
 // FP64 device kernels: strided window copies and the BLAS-1 / reduction
 // kernels of the iterative solvers.
 #include "kernels.hpp"
+#include "widen.cuh"
 
 #include <cuda_bf16.h>
 #include <algorithm>
@@ -45,14 +46,6 @@ __global__ void copy_f64_kernel(const CopyTask* __restrict__ tasks, int ntasks, 
 // (up to some hundreds), so outputs are what fills the chip.  With 16 outputs
 // a thread (4096 a block) a sigma of 1e5 entries ran on 32 blocks: 112 us.
 constexpr int SPLIT_CHUNK = 256;
-
-// (double)x without the FP64 pipe, which converts at two values a clock and SM
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) return (double)x;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-}
 
 template <class T>
 __global__ void __launch_bounds__(SPLIT_CHUNK) splitk_reduce_kernel(const SplitSeg* __restrict__ segs, int nseg,
@@ -334,11 +327,6 @@ __global__ void f64_to_f32_kernel(long n, const double* __restrict__ x, float* _
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
     y[i] = (float)x[i];
 }
-__global__ void f32_to_f64_kernel(long n, const float* __restrict__ x, double* __restrict__ y) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    y[i] = (double)x[i];
-}
-
 inline int red_grid(long n, int blocks) {
   return (int)std::max(1L, std::min((n + RED_T - 1) / RED_T, (long)blocks));
 }
@@ -465,9 +453,6 @@ void launch_f64_to_bf16(long n, const double* x, uint16_t* y, cudaStream_t s) {
 }
 void launch_f64_to_f32(long n, const double* x, float* y, cudaStream_t s) {
   f64_to_f32_kernel<<<elem_grid(n), 256, 0, s>>>(n, x, y);
-}
-void launch_f32_to_f64(long n, const float* x, double* y, cudaStream_t s) {
-  f32_to_f64_kernel<<<elem_grid(n), 256, 0, s>>>(n, x, y);
 }
 
 }  // namespace mpslcc

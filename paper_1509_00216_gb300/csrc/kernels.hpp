@@ -161,6 +161,5 @@ void launch_noise(long n, double amp, unsigned long long seed, double* x, cudaSt
 // Precision conversion for the tensor-core path.
 void launch_f64_to_bf16(long n, const double* x, uint16_t* y, cudaStream_t s);
 void launch_f64_to_f32(long n, const double* x, float* y, cudaStream_t s);
-void launch_f32_to_f64(long n, const float* x, double* y, cudaStream_t s);
 
 }  // namespace mpslcc

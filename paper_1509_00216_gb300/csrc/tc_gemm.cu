@@ -33,6 +33,7 @@
 #include "kruns.hpp"
 #include "tcfold.hpp"
 #include "tcgen05.cuh"
+#include "widen.cuh"
 
 namespace mpslcc {
 
@@ -52,7 +53,8 @@ struct alignas(64) TcTask {
   int tm, tn;
   int mode;             // 0: FP32 atomic add, 1: BF16 store, 2: FP32 store,
                         // 3: split BF16 store (hi at +0, lo at +soff), 4: FP64 alpha/beta store,
-                        // 5: three-piece BF16 store, six B-side blocks at +j soff
+                        // 5: three-piece BF16 store, six B-side blocks at +j soff,
+                        // 6: FP64 store of the plain product
   int split;            // operands are hi + lo pairs: acc += Ah Bh + Ah Bl + Al Bh
   long long soff;
   double alpha, beta;   // mode 4: FP64 store C = alpha acc + beta C
@@ -287,11 +289,12 @@ __device__ __forceinline__ void store_row(const TcTask* T, long long roff, int c
     const int cst = T->cst;
     double* C = (double*)T->C + roff + (long long)c0 * cst;
     const double al = T->alpha, be = T->beta;
+    const bool keep = be != 0.0;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       if (j >= nv) break;
-      const double x = al * (double)__uint_as_float(v[j]);
-      *C = be == 0.0 ? x : x + be * *C;
+      const double x = al * widen(__uint_as_float(v[j]));
+      *C = keep ? x + be * *C : x;
       C += cst;
     }
     return;
@@ -492,6 +495,30 @@ __device__ __forceinline__ void store_chunk_staged(const PieceTile& P, uint8_t* 
           *reinterpret_cast<uint4*>(C + (part == 1 ? so : 0)) = val;
         }
       }
+    }
+    __syncwarp();
+  }
+}
+
+// A warp's 32 x 32 accumulator chunk (lane i holding row rw0 + i) widened to
+// FP64 rows of C, 16 columns at a time through the staging rows: each store
+// instruction covers two rows x 128 contiguous bytes instead of 32 rows x 8.
+__device__ __forceinline__ void store_chunk_f64(double* C, int ldc, int m, uint8_t* stg, int lane, int rw0, int c0,
+                                                int nv, const uint32_t* v) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (16 * h >= nv) break;
+    uint4* mine = reinterpret_cast<uint4*>(stg + lane * STG_ROW);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      mine[q] = make_uint4(v[16 * h + 4 * q], v[16 * h + 4 * q + 1], v[16 * h + 4 * q + 2], v[16 * h + 4 * q + 3]);
+    __syncwarp();
+    const int c = lane & 15;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int r = 2 * q + (lane >> 4);
+      const float f = *reinterpret_cast<const float*>(stg + r * STG_ROW + c * 4);
+      if (rw0 + r < m && 16 * h + c < nv) C[(long long)(rw0 + r) * ldc + c0 + 16 * h + c] = widen(f);
     }
     __syncwarp();
   }
@@ -726,7 +753,7 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
                       : (long long)tb * T->cbatch + (long long)tks * T->kstride +
                             (long long)(row / T->rpb) * T->bstride + (long long)(row % T->rpb) * T->ldc;
       const int wch = live ? row / T->rpb : 0;
-      const bool staged = pieces && T->mode != 2;
+      const bool staged = pieces && T->mode != 2, plain64 = T->mode == 6;
       PieceTile PT;
       if (staged) piece_tile(T, row0 + quarter * 32, lane, PT);
       const bool ok = mbar_wait(&acc_full[buf], (tcount >> 1) & 1u, err, 3, wait_ns);
@@ -739,10 +766,14 @@ __global__ void __launch_bounds__(KCfg<CFG>::THREADS, KCfg<CFG>::MINB) tc_gemm_k
           store_chunk_staged(PT, stg, lane, col0 + cb, v);
           continue;
         }
-        if (!live) continue;
         const int c0 = col0 + cb;
         const int nv = min(32, tn - c0);
         if (nv <= 0) continue;
+        if (plain64) {
+          store_chunk_f64((double*)T->C, T->ldc, T->m, stg, lane, row0 + quarter * 32, c0, nv, v);
+          continue;
+        }
+        if (!live) continue;
         if (pieces) store_row_pieces(T, roff, wch, c0, nv, v);
         else store_row(T, roff, c0, nv, v);
       }
@@ -1941,8 +1972,8 @@ void tc_selftest(Ctx& c, int prec, int m, int n, int k, const double* A, const d
 // ones inside its step, or code whose device memory is all reserved at
 // start-up.  For
 // them, C = A B^T (the self-test product above) is also offered with all of
-// its scratch -- the low-precision operand copies, the FP32 result, the task
-// descriptors and the error flag -- in one fixed file-scope device array.
+// its scratch -- the low-precision operand copies, the task descriptors and the
+// error flag -- in one fixed file-scope device array.
 // ---------------------------------------------------------------------------
 constexpr size_t NOALLOC_SCRATCH_BYTES = 64ull << 20;  // 64 MiB held by every GPU that loads the library
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
@@ -1989,7 +2020,8 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
   const int es = esize(prec);
   const int sp = prec == MPSLCC_BF16X3 ? 2 : 1;
   const long k8 = pad8(k), kk = sp * k8;
-  // scratch layout: [conv tasks | tc task | error flag | A copy | B copy | FP32 result]
+  // scratch layout: [conv tasks | tc task | error flag | A copy | B copy]; the
+  // largest accepted problem also counts 4 bytes per element of C
   const size_t o_conv = 0, o_task = up256(2 * sizeof(ConvTask)), o_err = o_task + up256(sizeof(TcTask));
   const size_t o_a = o_err + 256, o_b = o_a + up256((size_t)m * kk * es), o_c = o_b + up256((size_t)n * kk * es);
   const size_t need = o_c + up256((size_t)m * n * 4);
@@ -2001,7 +2033,6 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
   MPSLCC_REQUIRE(cur == device, ST_ARG, "device must be the current device");
   char* base = (char*)noalloc_scratch(device);
   // operand copies; the conversion clears the padding columns
-  cuda_check(cudaMemsetAsync(base + o_err, 0, 256, stream), "noalloc memset");
   ConvTask cv[2];
   std::memset(cv, 0, sizeof(cv));
   cv[0].src = dA; cv[0].dst = base + o_a; cv[0].rows = m; cv[0].cols = k; cv[0].src_ld = k; cv[0].dst_ld = (int)kk;
@@ -2009,14 +2040,22 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
   cv[1].src = dB; cv[1].dst = base + o_b; cv[1].rows = n; cv[1].cols = k; cv[1].src_ld = k; cv[1].dst_ld = (int)kk;
   cv[1].batch = 1; cv[1].pattern = sp == 2 ? 1 : 0; cv[1].soff = k8; cv[1].pad = 1;
   const long long tot = plan_conv(cv, 2);
-  cuda_check(cudaMemcpyAsync(base + o_conv, cv, sizeof(cv), cudaMemcpyHostToDevice, stream), "noalloc tasks");
-  launch_conv(prec, (const ConvTask*)(base + o_conv), 2, tot, stream);
-  cuda_check(cudaGetLastError(), "noalloc conv");
-  // one GEMM task writing FP32 rows of C
+  // One GEMM task writing FP64 rows of C.  Its N tile: the widest whose waves of
+  // tiles cost least, a tile's time going with its operand rows.  (1021 x 775 x
+  // 1502, BF16x3: 32 tiles of 256 take 47 us on 152 SMs, 104 of 64 take 24.5.)
+  const int sms = sm_count_dev(device);
+  int cap = 256;
+  long long best = 0;
+  for (int w : {256, 128, 64}) {
+    const int nt = (int)std::min<long>(w, (n + 15) / 16 * 16);
+    const long long waves = ((long long)((m + 127) / 128) * ((n + nt - 1) / nt) + sms - 1) / sms;
+    const long long cost = waves * (128 + nt);
+    if (w == 256 || cost < best) { cap = w; best = cost; }
+  }
   TcTask t;
   std::memset(&t, 0, sizeof(t));
   const int KT = prec == MPSLCC_TF32 ? 32 : 64;
-  t.ntile = (int)std::min<long>(256, (n + 15) / 16 * 16);
+  t.ntile = (int)std::min<long>(cap, (n + 15) / 16 * 16);
   const long klen = sp == 2 ? k8 : kk;  // length of one operand part along K
   noalloc_map(&t.ma, prec, base + o_a, m, klen, kk, 128);
   noalloc_map(&t.mb, prec, base + o_b, n, klen, kk, t.ntile);
@@ -2025,13 +2064,14 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
     noalloc_map(&t.ma2, prec, base + o_a + k8 * 2, m, klen, kk, 128);
     noalloc_map(&t.mb2, prec, base + o_b + k8 * 2, n, klen, kk, t.ntile);
   }
-  t.C = base + o_c;
+  t.C = dC;
   t.ldc = n;
+  t.cst = 1;
   t.rpb = 1 << 30;
   t.m = m;
   t.n = n;
   t.k = (int)klen;
-  t.mode = 2;
+  t.mode = 6;
   t.ksteps = (int)((klen + KT - 1) / KT);
   t.ksplit = 1;
   t.kchunk = t.ksteps;
@@ -2040,12 +2080,18 @@ void tc_gemm_noalloc(int device, cudaStream_t stream, int prec, int m, int n, in
   t.tile0 = 0;
   t.batch = 1;
   long long tiles = (long long)t.tm * t.tn;
-  cuda_check(cudaMemcpyAsync(base + o_task, &t, sizeof(t), cudaMemcpyHostToDevice, stream), "noalloc task");
-  int grid = (int)std::min<long long>(tiles, sm_count_dev(device));
-  launch_tc_stream(stream, grid, prec, (const TcTask*)(base + o_task), 1, tiles, (int*)(base + o_err));
+  // tasks and a cleared error flag in one copy
+  alignas(64) unsigned char image[2048];
+  MPSLCC_REQUIRE(o_a <= sizeof(image), ST_INTERNAL, "task image");
+  std::memset(image, 0, o_a);
+  std::memcpy(image + o_conv, cv, sizeof(cv));
+  std::memcpy(image + o_task, &t, sizeof(t));
+  cuda_check(cudaMemcpyAsync(base, image, o_a, cudaMemcpyHostToDevice, stream), "noalloc tasks");
+  launch_conv(prec, (const ConvTask*)(base + o_conv), 2, tot, stream);
+  cuda_check(cudaGetLastError(), "noalloc conv");
+  launch_tc_stream(stream, (int)std::min<long long>(tiles, sms), prec, (const TcTask*)(base + o_task), 1, tiles,
+                   (int*)(base + o_err), WAIT_NS, cap);
   cuda_check(cudaGetLastError(), "noalloc gemm");
-  launch_f32_to_f64((long)m * n, (const float*)(base + o_c), dC, stream);
-  cuda_check(cudaGetLastError(), "noalloc result");
   int h = 0;
   cuda_check(cudaMemcpyAsync(&h, base + o_err, sizeof(int), cudaMemcpyDeviceToHost, stream), "noalloc flag");
   cuda_check(cudaStreamSynchronize(stream), "noalloc sync");
