@@ -106,8 +106,9 @@ def peaks():
     return dict(hbm=6800.0, bf16=1900.0, bf16_sust=1700.0, src="fallback")
 
 
-# FP64 pipe of GB300 (nominal, no FP64 tensor path): 1.25 TFLOP/s
-FP64_PEAK_TFLOPS = 1.25
+# An FP64 product is 36 products of 8-bit digit planes on the FP16 tensor pipe,
+# whose dense rate is that of BF16.
+FP64_DIGIT_PRODUCTS = 36
 
 
 class Clocks:
@@ -467,9 +468,10 @@ def gpu_arm(args, rank, world, local_rank):
     pk = peaks()
     kern = sweep_sigma_s
     if prec == 0:
-        # FP64 DFMA path: ALU-bound against the FP64 pipe
-        roof = {"bound": "alu", "achieved": flops / kern / 1e12 if kern else None, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "kernel": "gemm_f64_kernel (sigma phases)"}
+        # FP64 products as digit products on the tensor cores
+        roof = {"bound": "tensor", "achieved": flops / kern / 1e12 if kern else None,
+                "peak": pk["bf16"] / FP64_DIGIT_PRODUCTS, "unit": "TFLOP/s",
+                "kernel": "gemm_f64_tc_kernel (sigma phases)"}
     else:
         # tensor-core sigma GEMMs run far below the BF16 ridge (about 100
         # algorithmic flop per byte against ~280): they are bounded by HBM
@@ -522,7 +524,7 @@ def gpu_arm(args, rank, world, local_rank):
         with open(args.save_state, "wb") as f:
             pickle.dump({"phi0": ctx.export_mps(0), "phi1": ctx.export_mps(1)}, f, protocol=4)
     if args.fp64_sweep and prec != 0:
-        # one whole sweep on the plain FP64 path (DFMA GEMMs) and one in mixed
+        # one whole sweep on the FP64 path and one in mixed
         # precision, both from the timed sweeps' final states, outside the
         # timed region; times and the energies of the resulting states
         p0, p1 = ctx.export_mps(0), ctx.export_mps(1)

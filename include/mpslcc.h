@@ -57,7 +57,9 @@ typedef enum {
                             solver (breakdown); see the sweep calls        */
 } mpslcc_status;
 
-/* FP64 DFMA; TF32 or BF16 tensor-core operands (FP32 accumulation); BF16X3:
+/* FP64 (products on the tensor cores as exact integer digit products, small
+   ones on the FP64 pipe; at least as accurate as a chain of FP64 fused
+   multiply-adds); TF32 or BF16 tensor-core operands (FP32 accumulation); BF16X3:
    operands split into BF16 hi + lo parts, hi*hi + hi*lo + lo*hi accumulated
    in FP32 (about 2^-17 relative accuracy); BF16X6: three BF16 parts h, m, l,
    the six products hh hm mh mm hl lh accumulated in FP32 (about 2^-24, the
@@ -104,7 +106,8 @@ typedef struct {
   double wait_timeout_s; /* bound on every device-side wait of the tensor-core
                             kernels, seconds (0 = 2 s, at most 60 s); a wait
                             that runs out makes the call return
-                            MPSLCC_E_TIMEOUT and leaves the context usable  */
+                            MPSLCC_E_TIMEOUT and leaves the context usable.
+                            FP64 products wait at most 2 s whatever it says  */
   int tc_environments;   /* 1: the environments and fused operators that
                             mpslcc_apply_heff builds run on the tensor cores
                             as inside mixed-precision sweeps (three-piece

@@ -18,7 +18,7 @@
 //
 // Measured against the 64 x 64 FP64-pipe tiles that did all of this before
 // (3-band model, middle position, M1 = 500): sigma phases 27.0 + 28.8 ms ->
-// 2.5 + 3.4 ms, error against 64-bit contraction 2.4e-15 -> 1.0e-15; all
+// 2.4 + 2.8 ms, error against 64-bit contraction 2.4e-15 -> 1.0e-15; all
 // products of the energies at M1 = 400, 790 ms -> 49 ms.  A tile's time is its
 // chain (loads, cutting, products, drain, conversion, stores), of which the
 // integer pipe carries most; the tensor pipe is busy a tenth of it.
