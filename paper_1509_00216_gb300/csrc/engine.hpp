@@ -378,7 +378,7 @@ void run_f64(Ctx& c, const F64Launch& l, const void* d);
 // Throws ST_TIMEOUT if an FP64 product of the (synchronised) stream gave up.
 void check_f64(Ctx& c);
 int sm_count_dev(int device);
-// FP64 DFMA kernel or split-BF16 tensor cores, by c.gemm_prec
+// FP64 products or split-BF16 tensor cores, by c.gemm_prec
 void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t);
 void validate_gemm(const Ctx& c, const GemmTask& t);
 void validate_copy(const Ctx& c, const CopyTask& t);
