@@ -58,8 +58,8 @@ typedef enum {
 } mpslcc_status;
 
 /* FP64 (products on the tensor cores as exact integer digit products, small
-   ones on the FP64 pipe; at least as accurate as a chain of FP64 fused
-   multiply-adds); TF32 or BF16 tensor-core operands (FP32 accumulation); BF16X3:
+   ones on the FP64 pipe; the error of every sum of n terms x y is within the
+   bound of a chain of FP64 fused multiply-adds, about n 2^-53 sum |x y|); TF32 or BF16 tensor-core operands (FP32 accumulation); BF16X3:
    operands split into BF16 hi + lo parts, hi*hi + hi*lo + lo*hi accumulated
    in FP32 (about 2^-17 relative accuracy); BF16X6: three BF16 parts h, m, l,
    the six products hh hm mh mm hl lh accumulated in FP32 (about 2^-24, the

@@ -10,18 +10,25 @@
 // 128 products of 2^14).  The 36 plane pairs whose weight is at least 2^-56 of
 // the largest are formed; pairs of equal weight share one accumulator, the
 // accumulators are combined in integers and rounded to FP64 once per 1024 K
-// values.  Against a chain of FP64 multiply-adds, whose error grows with K,
-// what is lost is the rounding of an operand to 2^-62 of its row's largest
-// value and the pairs left out (2^-60 of a product of two such values).
+// values.  What is lost is the cut of an operand (below 2^-61 of its row's
+// largest value) and the pairs left out (at most 2^-57.2 of the product of the
+// two rows' largest values per term, typically 2^-60).  Both go with the rows'
+// largest values, not with the terms: where the large values of two rows meet
+// the small ones of the other, an output's error would pass that of a chain of
+// FP64 multiply-adds.  So every output is checked against a lower bound of sum
+// |x y| (sum_magnitudes), and those that might pass the chain's bound, n 2^-53
+// sum |x y|, are summed in FP64 instead.  (Operands graded over 2^40 in opposite
+// directions were off by 1e-8 of sum |x y| before this check.)
 //
 // Tasks of few multiply-adds run on the FP64 pipe (gemm_f64_pipe_kernel).
 //
 // Measured against the 64 x 64 FP64-pipe tiles that did all of this before
 // (3-band model, middle position, M1 = 500): sigma phases 27.0 + 28.8 ms ->
-// 2.4 + 2.8 ms, error against 64-bit contraction 2.4e-15 -> 1.0e-15; all
-// products of the energies at M1 = 400, 790 ms -> 49 ms.  A tile's time is its
-// chain (loads, cutting, products, drain, conversion, stores), of which the
-// integer pipe carries most; the tensor pipe is busy a tenth of it.
+// 2.8 + 3.0 ms (2.4 + 2.8 without the check), error against 64-bit contraction
+// 2.4e-15 -> 1.0e-15; all products of the energies at M1 = 400, 790 ms -> 55 ms.
+// A tile's time is its chain (loads, cutting, products, check, drain, conversion,
+// stores), of which the integer pipe carries most; the tensor pipe is busy a
+// tenth of it.
 #include <algorithm>
 #include <atomic>
 #include <vector>
@@ -40,6 +47,8 @@ constexpr int KS = 32;                 // K values per step (64 bytes of FP16)
 constexpr int CHUNK = 4;               // steps between two drains: 128 K values
 constexpr int PLANES = 8;
 constexpr int MAX_DEV = 128;
+constexpr uint32_t ENOUGH = 1156, ENOUGH_B = 255;   // see sum_magnitudes
+constexpr int ZERO_ROW = 63;           // exponent in the scale of a row of zeros (others: 64 and more)
 
 // Two shapes.  TN = 64, one CTA of 16 warps per SM: two step buffers, so that
 // digits are cut while the previous step multiplies; 8 x 64 accumulator columns
@@ -55,14 +64,28 @@ template <int TN_> struct F64Cfg {
   static constexpr int OPER = PLANES * (XPLANE + YPLANE);      // 192 or 80 KB
   static constexpr int XU = 16 / WARPS;                        // loader units of X per warp
   static constexpr int YU0 = WARPS - TN / 8;                   // first warp that loads Y
+  // Leading magnitudes, a byte each: MW steps, 16-byte groups of a row swizzled.
+  // (Four steps at TN = 32 would take the chip from 196 to 228 KB of shared
+  // memory per SM, and the loads' share of L1 from 60 to 28 KB: 9.7 instead of
+  // 8.7 ms for a sigma of the 3-band model at M1 = 500.)
+  static constexpr int MW = TN == 64 ? 4 : 2, MROW = KS * MW;
+  static constexpr int MAGS = (TM + TN) * MROW;
+  static constexpr int ALIGN = 8 * ROW;                        // of the planes: a swizzle atom
 };
+template <class F> __device__ __forceinline__ int mag_at(int row, int group) {
+  return row * F::MROW + ((group ^ (F::MW == 4 ? row & 7 : row >> 1 & 3)) << 4);
+}
 struct F64Slot {
   F64Task t;
   int b, ks, ix, iy;
 };
-template <class F> constexpr int f64_smem() {
-  return F::OPER + 1024 + KB * 4 + (TM + F::TN) * 8 + 64 + 2 * (int)sizeof(F64Slot) + (TM + F::TN) * 8;
+template <bool MULTI> constexpr int TAB = MULTI ? KB : KS * CHUNK;   // K values of a block
+template <class F, bool MULTI> constexpr int f64_smem() {
+  return F::OPER + F::ALIGN + F::MAGS + TAB<MULTI> * 4 + (TM + F::TN) * 4 + 64 + 2 * (int)sizeof(F64Slot) +
+         (TM + F::TN) * 8;
 }
+// see F64Cfg
+static_assert(2 * (f64_smem<F64Cfg<32>, true>() + 1024) <= 196 * 1024, "two CTAs in 196 KB");
 
 struct F64Tile { int b, ks, ix, iy; };
 __device__ __forceinline__ F64Tile tile_of(const F64Task& T, long long tile) {
@@ -197,12 +220,14 @@ __device__ __forceinline__ uint32_t unit_max(const double (&v)[8], uint32_t m) {
 
 // v as an integer of 62 bits relative to the row exponent (cut towards zero:
 // 2^-61 of the row's largest value at most), offset by 128 in every digit:
-// byte i of the result is digit i plus 128.
-__device__ __forceinline__ unsigned long long digits(double v, int emax) {
+// byte i of the result is digit i plus 128.  The top byte of `mag` gets the
+// integer's magnitude over 2^54, cut.
+__device__ __forceinline__ unsigned long long digits(double v, int emax, uint32_t& mag) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-  const int d = min(emax - (int)((hi >> 20) & 0x7ffu), 63);   // 63 clears zeros too: emax >= 64
+  const int d = min(emax - (int)((hi >> 20) & 0x7ffu), 63);   // 63 clears zeros too: emax >= 63
   unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
   m = (m << 9) >> d;
+  mag = (uint32_t)(m >> 32) << 2;
   const long long s = (long long)((int)hi >> 31);
   return (m ^ (unsigned long long)s) + (0x8080808080808080ull - (unsigned long long)s);
 }
@@ -217,22 +242,27 @@ __device__ __forceinline__ int scale_exp(int scale) { return (scale >> 1) - ((sc
 // the FP16 exponent of 1024 is 1024 + digit + 128; one subtraction leaves it.
 // (Bound by the integer pipe: two byte permutations per pair of digits, where
 // BF16's shorter significand needed four operations.)
-template <int NBUF>
+template <class F>
 __device__ __forceinline__ void store_unit(const Unit& u, double (&v)[8], int scale, uint8_t* planes, int plane,
-                                           int half) {
+                                           int half, uint8_t* mags, int mrow, int step) {
   const int emax = scale >> 1;
   if (scale & 1) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] *= 0x1p512;
   }
-  uint32_t t0[8], t1[8];
+  uint32_t t0[8], t1[8], mg[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const unsigned long long t = digits(v[j], emax);
+    const unsigned long long t = digits(v[j], emax, mg[j]);
     t0[j] = (uint32_t)t;
     t1[j] = (uint32_t)(t >> 32);
   }
-  uint8_t* dst = NBUF == 2 ? planes + u.row * 128 + (((half * 4 + u.q) ^ (u.row & 7)) << 4)
+  auto tops = [](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0073), __byte_perm(c, d, 0x0073), 0x5410);
+  };
+  *reinterpret_cast<uint2*>(mags + mag_at<F>(mrow + u.row, 2 * (step & (F::MW - 1)) + (u.q >> 1)) + (u.q & 1) * 8) =
+      make_uint2(tops(mg[0], mg[1], mg[2], mg[3]), tops(mg[4], mg[5], mg[6], mg[7]));
+  uint8_t* dst = F::NBUF == 2 ? planes + u.row * 128 + (((half * 4 + u.q) ^ (u.row & 7)) << 4)
                            : planes + u.row * 64 + ((u.q ^ ((u.row >> 1) & 3)) << 4);
 #pragma unroll
   for (int p = 0; p < PLANES; p += 2) {
@@ -250,6 +280,119 @@ __device__ __forceinline__ void store_unit(const Unit& u, double (&v)[8], int sc
     }
     *reinterpret_cast<uint4*>(dst + p * plane) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
     *reinterpret_cast<uint4*>(dst + (p + 1) * plane) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
+  }
+}
+
+// Whether a digit product may stand.  With |X|, |Y| < 2^62 a term loses less
+// than 2 x 2^62 to the cut of its operands and 7.03 x 2^62 to the plane pairs
+// left out, in units of X Y, so the error of an output is below that of a chain
+// of n FP64 multiply-adds, n 2^-53 sum |x y|, if sum |X Y| >= 9.03 x 2^115.  The
+// leading eight bits of the operands bound that sum from below: sum (|X| >>
+// 54)(|Y| >> 54) >= 1156 = 9.03 x 2^7 will do.  Where x and y have their large
+// values at different k it may fail, and the output is summed again in FP64
+// (sum_again).  A thread adds up its row's outputs of 16 columns, four at a time,
+// over `steps` of a window and stops with its warp once all have enough (mostly
+// after 32 values); `sums` holds a byte per output, its sum / 16 so far or
+// ENOUGH_B.
+template <class F>
+__device__ __forceinline__ void sum_magnitudes(const uint8_t* mags, int row, int col0, int steps, uint32_t (&sums)[4]) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    if (!__any_sync(0xffffffffu, sums[g] != ~0u)) continue;
+    uint32_t acc[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint32_t b = sums[g] >> (8 * c) & 255u;
+      acc[c] = b == ENOUGH_B ? ENOUGH : b << 4;
+    }
+#pragma unroll 1
+    for (int st = 0; st < steps; ++st) {
+#pragma unroll
+      for (int w = 2 * st; w < 2 * st + 2; ++w) {
+        const uint4 a = *reinterpret_cast<const uint4*>(mags + mag_at<F>(row, w));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {   // rows TM + col0 + ...: a multiple of 16
+          const uint4 b = *reinterpret_cast<const uint4*>(mags + (TM + col0) * F::MROW + mag_at<F>(4 * g + c, w));
+          acc[c] = __dp4a(a.w, b.w, __dp4a(a.z, b.z, __dp4a(a.y, b.y, __dp4a(a.x, b.x, acc[c]))));
+        }
+      }
+      if (__all_sync(0xffffffffu, min(min(acc[0], acc[1]), min(acc[2], acc[3])) >= ENOUGH)) break;
+    }
+    sums[g] = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sums[g] |= (acc[c] >= ENOUGH ? ENOUGH_B : acc[c] >> 4) << (8 * c);
+  }
+}
+
+// Sums the n outputs of a tile in `list` (row << 6 | column), or its first n where
+// there is no list, in ascending K, from operand rows staged in shared memory:
+// at up to the two multiply-adds a clock that the FP64 pipe gives.
+template <int TN>
+__device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, int n, uint8_t* smem, const int* tab,
+                                       const long long* coff, const long long* roff, int kb, int len,
+                                       int mode) {
+  constexpr int THREADS = F64Cfg<TN>::THREADS, U = 4, LD = KS + 1;
+  const F64Task& T = S.t;
+  const int tid = threadIdx.x, x0 = S.ix * TM, y0 = S.iy * TN;
+  const int nx = min(TM, T.mx - x0), ny = min(TN, T.my - y0);
+  double* xs = (double*)smem;
+  double* ys = xs + TM * LD;
+  long long* xo = (long long*)(ys + TN * LD);
+  long long* yo = xo + TM;
+  static_assert((TM + TN) * (LD + 1) * 8 <= F64Cfg<TN>::OPER, "staging");
+  const double* X = T.x + (long long)S.b * T.xub;
+  const double* Y = T.y + (long long)S.b * T.yub;
+  double* C = T.c + (long long)S.b * T.cub + (long long)S.ks * T.sK;
+  if (tid < nx) xo[tid] = row_off(x0 + tid, T.nx, T.xrs, T.xbs);
+  if (tid >= THREADS - ny) yo[tid - (THREADS - ny)] = row_off(y0 + tid - (THREADS - ny), T.ny, T.yrs, T.ybs);
+  for (int base = 0; base < n; base += U * THREADS) {
+    int at[U];
+    double acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = base + u * THREADS + tid;
+      at[u] = e >= n ? -1 : (list ? list[e] : e / ny << 6 | e % ny);
+      acc[u] = 0.0;
+    }
+    for (int kk = 0; kk < len; kk += KS) {
+      const int nk = min(KS, len - kk);
+      __syncthreads();
+      constexpr int NX = TM * KS / THREADS, NY = TN * KS / THREADS;
+      double vx[NX], vy[NY];
+#pragma unroll
+      for (int i = 0; i < NX; ++i) {
+        const int e = tid + i * THREADS, r = T.xks == 1 ? e / KS : e % TM, q = T.xks == 1 ? e % KS : e / TM;
+        vx[i] = r < nx && q < nk ? __ldg(X + xo[r] + (long long)(T.kr ? tab[kk + q] : kb + kk + q) * T.xks) : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < NY; ++i) {
+        const int e = tid + i * THREADS, r = T.yks == 1 ? e / KS : e % TN, q = T.yks == 1 ? e % KS : e / TN;
+        vy[i] = r < ny && q < nk ? __ldg(Y + yo[r] + (long long)(T.kr ? tab[kk + q] : kb + kk + q) * T.yks) : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < NX; ++i) {
+        const int e = tid + i * THREADS;
+        xs[T.xks == 1 ? e / KS * LD + e % KS : e % TM * LD + e / TM] = vx[i];
+      }
+#pragma unroll
+      for (int i = 0; i < NY; ++i) {
+        const int e = tid + i * THREADS;
+        ys[T.yks == 1 ? e / KS * LD + e % KS : e % TN * LD + e / TN] = vy[i];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (at[u] < 0) continue;
+        const double* px = xs + (at[u] >> 6) * LD;
+        const double* py = ys + (at[u] & 63) * LD;
+        double a = acc[u];
+        for (int q = 0; q < nk; ++q) a = fma(px[q], py[q], a);
+        acc[u] = a;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (at[u] >= 0) put(T, mode, C + roff[at[u] >> 6] + coff[at[u] & 63], acc[u]);
   }
 }
 
@@ -294,8 +437,8 @@ __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
 // With MULTI = false every task sums at most one chunk (128 K values): the
 // accumulators go straight to the output, and the registers can hold two steps'
 // values.  With MULTI = true the chunks' sums stay in 64 registers a thread and
-// a step's values are loaded when they are cut; both kinds in one kernel
-// spilled registers to L2 in the cutting loop.
+// a step's values are loaded when they are cut (more than 128 registers all the
+// same: some 650 bytes a thread are spilled, 500 at TN = 64 with MULTI = false).
 template <int TN, bool MULTI>
 __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
     gemm_f64_tc_kernel(const F64Task* __restrict__ tasks, int ntasks, long long total, int* err,
@@ -304,16 +447,21 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
   constexpr int THREADS = F::THREADS, XU = F::XU, NBUF = F::NBUF;
   constexpr bool PAIR = !MULTI && XU == 1;            // registers hold two steps' values
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + F::ALIGN - 1) & ~(uintptr_t)(F::ALIGN - 1));
   uint8_t* yplanes = smem + PLANES * F::XPLANE;
-  int* tab = (int*)(smem + F::OPER);                  // operand column of each K value of the block
-  uint32_t* rmax = (uint32_t*)(tab + KB);             // largest high word per row: X, then Y
-  int* rscale = (int*)(rmax + TM + TN);               // the rows' scales
+  uint8_t* mags = smem + F::OPER;                     // leading magnitudes of a chunk; then outputs to sum again
+  int* tab = (int*)(mags + F::MAGS);                  // operand column of each K value of the block
+  uint32_t* rmax = (uint32_t*)(tab + TAB<MULTI>);     // largest high word per row: X, then Y
+  int* rscale = (int*)rmax;                           // then the rows' scales in its place
   uint64_t* bar = (uint64_t*)(rscale + TM + TN);      // [2] products of a buffer done, [1] drain
   volatile uint32_t* tslot = (volatile uint32_t*)(bar + 3);
+  int* nagain = (int*)(bar + 4);                      // outputs to sum again
   F64Slot* slots = (F64Slot*)(bar + 8);               // this tile's task and the next one's
   long long* coff = (long long*)(slots + 2);          // output offset of each column
   long long* roff = coff + TN;                        // and of each row
+  uint16_t* list = (uint16_t*)mags;                   // outputs to sum again (after a block's products)
+  uint16_t* skip = list + TM * TN;                    // and per thread which of its own
+  static_assert(TM * TN * 2 + THREADS * 2 <= F::MAGS, "list");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     mbar_init(&bar[0], 1);
@@ -372,6 +520,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
       const int len = max(0, min(KB, k1 - kb));
       const int nst = (len + KS - 1) / KS;
       if (tid < TM + TN) rmax[tid] = 0;
+      if (tid == 0) *nagain = 0;
       if (T.kr)
         for (int i = tid; i < len; i += THREADS) tab[i] = k_col(T, kb + i);
       __syncthreads();
@@ -418,7 +567,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         int e = (int)(h >> 20), tiny = 0;
         if (e < 64) {
           tiny = h != 0;
-          e = tiny ? (int)((uint32_t)__double2hiint(__hiloint2double((int)h + 1, 0) * 0x1p512) >> 20) : 64;
+          e = tiny ? (int)((uint32_t)__double2hiint(__hiloint2double((int)h + 1, 0) * 0x1p512) >> 20) : ZERO_ROW;
         }
         rscale[tid] = e << 1 | tiny;
       }
@@ -447,6 +596,13 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         }
       };
       if (!plain) {
+        // outputs to be checked: those of non-zero rows
+        uint32_t sums[4] = {~0u, ~0u, ~0u, ~0u};
+        if (mine && orow < nx && rscale[orow] != ZERO_ROW << 1) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            if (colq * 16 + c < ny && rscale[TM + colq * 16 + c] != ZERO_ROW << 1) sums[c >> 2] ^= ENOUGH_B << (8 * (c & 3));
+        }
         auto step = [&](int s, Vals& v) -> bool {
           const uint32_t h = NBUF == 2 ? it & 1u : 0u, use = NBUF == 2 ? it >> 1 : it;   // buffer, its use count
           if (!PAIR && nst > 1) load(s, v);
@@ -455,8 +611,8 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
           if (ok) {
 #pragma unroll
             for (int u = 0; u < XU; ++u)
-              if (ux[u].ok) store_unit<NBUF>(ux[u], v.x[u], rscale[ux[u].row], smem, F::XPLANE, h);
-            if (uy.ok) store_unit<NBUF>(uy, v.y, rscale[TM + uy.row], yplanes, F::YPLANE, h);
+              if (ux[u].ok) store_unit<F>(ux[u], v.x[u], rscale[ux[u].row], smem, F::XPLANE, h, mags, 0, s);
+            if (uy.ok) store_unit<F>(uy, v.y, rscale[TM + uy.row], yplanes, F::YPLANE, h, mags, TM, s);
           }
           if (PAIR && s + 2 < nst) load(s + 2, v);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -489,16 +645,20 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
             ti = fetch_slot(&slots[cur ^ 1], tasks, ntasks, tile + gridDim.x, ti);
             fetched = true;
           }
-          if (s + 1 == nst || (MULTI && (s & (CHUNK - 1)) == CHUNK - 1)) {
+          // a window of several: checked while the products run
+          const bool window = F::MW < CHUNK && (s + 1 == nst || (s & (F::MW - 1)) == F::MW - 1);
+          if (window) sum_magnitudes<F>(mags, orow, colq * 16, (s & (F::MW - 1)) + 1, sums);
+          if (MULTI && (s + 1 == nst || (s & (CHUNK - 1)) == CHUNK - 1)) {
             // all products up to this step are done
             if (!mbar_wait(&bar[h], use & 1u, err, 12, wait_ns)) abort = true;
             fence_after();
-            if (MULTI && mine) {
+            if (mine) {
 #pragma unroll
               for (int cb = 0; cb < 16; cb += 2) drain2(cb, ahi + (MULTI ? cb : 0), alo + (MULTI ? cb : 0));
             }
-            if (MULTI) fence_before();
+            fence_before();
           }
+          if (window && s + 1 < nst) __syncthreads();   // the next step overwrites the magnitudes
           ++it;
           return true;
         };
@@ -511,11 +671,27 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
             if (s + 1 < nst && !step(s + 1, v1)) { abort = true; break; }
           }
         }
+        // one window: checked where no step's values hold registers
+        static_assert(F::MW < CHUNK || !MULTI, "windows");
+        if (F::MW == CHUNK) sum_magnitudes<F>(mags, orow, colq * 16, nst, sums);
+        if (!MULTI && nst > 0 && !abort) {   // the last step's products
+          const uint32_t use = it - 1;
+          if (!mbar_wait(&bar[NBUF == 2 ? use & 1u : 0], (NBUF == 2 ? use >> 1 : use) & 1u, err, 12, wait_ns)) abort = true;
+          fence_after();
+        }
+        uint32_t open = 0;   // outputs to sum again
+#pragma unroll
+        for (int c = 0; c < 16; ++c) open |= ((sums[c >> 2] >> (8 * (c & 3)) & 255u) != ENOUGH_B ? 1u : 0u) << c;
+        int at = 0;
+        if (open) at = atomicAdd(nagain, __popc(open));
+        abort = __syncthreads_or(abort);
+        for (uint32_t o = open; o; o &= o - 1) list[at++] = (uint16_t)(orow << 6 | (colq * 16 + __ffs(o) - 1));
         // A warp holds 32 rows (one a lane) of 16 columns.  Where rows are
         // contiguous in memory it stores them column by column; else it turns
         // its piece in shared memory (its own part: the products are done) and
         // stores two rows of 16 columns at a time, instead of 32 rows of one.
-        if (mine) {
+        if (mine && !abort) {
+          const bool some = __any_sync(0xffffffffu, open != 0);
           const int exr = scale_exp(rscale[orow]);
           const bool lanes = T.cxs == 1;
           double* r = C + (orow < nx ? roff[orow] : 0);
@@ -535,34 +711,53 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
               const int col = colq * 16 + cb + j;
               const double x = to_f64(hi[j], lo[j], exr + scale_exp(rscale[TM + col]));
               if (!lanes) st[lane * 17 + cb + j] = x;
-              else if (col < ny && orow < nx) put(T, pm, r + coff[col], x);
+              else if (col < ny && orow < nx && !(open >> (cb + j) & 1)) put(T, pm, r + coff[col], x);
             }
           }
           if (!lanes) {
+            if (some) skip[tid] = (uint16_t)open;
             __syncwarp();
             const int col = colq * 16 + (lane & 15);
             double* c = C + (col < ny ? coff[col] : 0);
 #pragma unroll 4
             for (int i = lane >> 4; i < 32; i += 2) {
               const int row = quarter * 32 + i;
-              if (row < nx && col < ny) put(T, pm, c + roff[row], st[i * 17 + (lane & 15)]);
+              if (row < nx && col < ny && !(some && (skip[warp * 32 + i] >> (lane & 15) & 1)))
+                put(T, pm, c + roff[row], st[i * 17 + (lane & 15)]);
             }
           }
         }
         if (!MULTI) fence_before();
-      } else {
+      }
+      // The outputs listed, or all of a tile with a row that is not finite, as
+      // plain FP64 sums.  At TN = 64 some hundred a tile are common (sums of
+      // operators with coefficients, 12 % of the outputs at M1 = 1500): staged, 52000
+      // clocks for 1330 outputs of K = 48, 110000 read directly.  At TN = 32 they
+      // are few (56 of 4096 in 4 % of the tiles of the energies), and the call would
+      // cost the loops before it registers: eight lanes an output read it directly,
+      // 12000 clocks, 24000 staged.
+      const int nsum = plain ? nx * ny : (abort ? 0 : *nagain);
+      if (nsum > 0 && TN == 64) {
+        __syncthreads();   // the list, and the turned pieces are read
+        sum_again<TN>(slots[cur], plain ? nullptr : list, nsum, smem, tab, coff, roff, kb, len, pm);
+      } else if (nsum > 0) {
         const double* X = T.x + (long long)slots[cur].b * T.xub;
         const double* Y = T.y + (long long)slots[cur].b * T.yub;
-        for (int e = tid; e < nx * ny; e += THREADS) {
-          const int i = e / ny, j = e - i * ny;
+        __syncthreads();   // the list
+        for (int e0 = warp * 4; e0 < nsum; e0 += THREADS / 8) {
+          const int e = min(e0 + (lane >> 3), nsum - 1);
+          const int i = plain ? e / ny : list[e] >> 6, j = plain ? e - i * ny : list[e] & 63;
           const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
           const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
           double s = 0.0;
-          for (int k = 0; k < len; ++k) {
+#pragma unroll 4
+          for (int k = lane & 7; k < len; k += 8) {
             const int col = T.kr ? tab[k] : kb + k;
-            s = fma(px[(long long)col * T.xks], py[(long long)col * T.yks], s);
+            s = fma(__ldg(px + (long long)col * T.xks), __ldg(py + (long long)col * T.yks), s);
           }
-          put(T, pm, C + roff[i] + coff[j], s);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          if ((lane & 7) == 0 && e0 + (lane >> 3) < nsum) put(T, pm, C + roff[i] + coff[j], s);
         }
       }
       if (warp == 1 && next && !fetched && kb + KB >= k1) {
@@ -571,7 +766,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
       }
       abort = __syncthreads_or(abort);
       kb += KB;
-    } while (kb < k1 && !abort);
+    } while (MULTI && kb < k1 && !abort);   // a short sum is one block
   }
   if (abort && tid == 0) {
     // products already issued read shared and tensor memory: wait for them
@@ -910,12 +1105,12 @@ static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, 
   MPSLCC_REQUIRE(device >= 0 && device < MAX_DEV, ST_ARG, "device ordinal out of range");
   if (!attr[device].load(std::memory_order_acquire)) {
     cuda_check(cudaFuncSetAttribute(gemm_f64_tc_kernel<TN, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    f64_smem<F>()),
+                                    f64_smem<F, MULTI>()),
                "smem attr");
     attr[device].store(true, std::memory_order_release);
   }
   const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, sms) * F::CTAS);
-  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F>(), s>>>(d, n, tiles, err, WAIT_NS);
+  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F, MULTI>(), s>>>(d, n, tiles, err, WAIT_NS);
 }
 
 int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s) {
