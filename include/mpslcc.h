@@ -106,8 +106,7 @@ typedef struct {
   double wait_timeout_s; /* bound on every device-side wait of the tensor-core
                             kernels, seconds (0 = 2 s, at most 60 s); a wait
                             that runs out makes the call return
-                            MPSLCC_E_TIMEOUT and leaves the context usable.
-                            FP64 products wait at most 2 s whatever it says  */
+                            MPSLCC_E_TIMEOUT and leaves the context usable   */
   int tc_environments;   /* 1: the environments and fused operators that
                             mpslcc_apply_heff builds run on the tensor cores
                             as inside mixed-precision sweeps (three-piece

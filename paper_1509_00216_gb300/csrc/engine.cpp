@@ -173,7 +173,7 @@ void run_gemms(Ctx& c, std::vector<GemmTask>& t) {
 
 void run_f64(Ctx& c, const F64Launch& l, const void* d) {
   const int sms = std::max(1, sm_count_dev(c.device) - std::max(0, c.tc_sm_reserve));
-  const int n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s());
+  const int n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s(), wait_bound_ns(c));
   cuda_check(cudaGetLastError(), "gemm_f64 launch");
   c.st.gemm_launches += n;
   c.st.kernel_launches += n;

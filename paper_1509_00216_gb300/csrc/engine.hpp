@@ -378,6 +378,8 @@ void run_f64(Ctx& c, const F64Launch& l, const void* d);
 // Throws ST_TIMEOUT if an FP64 product of the (synchronised) stream gave up.
 void check_f64(Ctx& c);
 int sm_count_dev(int device);
+// Bound on each mbarrier wait of a context's tensor-core launches.
+unsigned long long wait_bound_ns(const Ctx& c);
 // FP64 products or split-BF16 tensor cores, by c.gemm_prec
 void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t);
 void validate_gemm(const Ctx& c, const GemmTask& t);

@@ -606,8 +606,8 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         auto step = [&](int s, Vals& v) -> bool {
           const uint32_t h = NBUF == 2 ? it & 1u : 0u, use = NBUF == 2 ? it >> 1 : it;   // buffer, its use count
           if (!PAIR && nst > 1) load(s, v);
-          bool ok = true;
-          if (use >= 1) ok = mbar_wait(&bar[h], (use - 1) & 1u, err, 11, wait_ns);
+          bool ok = !abort;   // a wait of the last chunk ran out: no more of them
+          if (ok && use >= 1) ok = mbar_wait(&bar[h], (use - 1) & 1u, err, 11, wait_ns);
           if (ok) {
 #pragma unroll
             for (int u = 0; u < XU; ++u)
@@ -1099,7 +1099,8 @@ void upload_f64(const F64Plan& p, void* d, cudaStream_t s) {
 }
 
 template <int TN, bool MULTI>
-static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, int sms, int* err, cudaStream_t s) {
+static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, int sms, int* err, cudaStream_t s,
+                          unsigned long long wait_ns) {
   using F = F64Cfg<TN>;
   static std::atomic<bool> attr[MAX_DEV];
   MPSLCC_REQUIRE(device >= 0 && device < MAX_DEV, ST_ARG, "device ordinal out of range");
@@ -1110,10 +1111,11 @@ static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, 
     attr[device].store(true, std::memory_order_release);
   }
   const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, sms) * F::CTAS);
-  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F, MULTI>(), s>>>(d, n, tiles, err, WAIT_NS);
+  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F, MULTI>(), s>>>(d, n, tiles, err, wait_ns);
 }
 
-int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s) {
+int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s,
+               unsigned long long wait_ns) {
   int launches = 0;
   const F64Task* t = (const F64Task*)d;
   for (int i = 0; i < F64_LISTS; ++i) {
@@ -1123,9 +1125,9 @@ int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err,
     if (n == 0) continue;
     if (i == F64_PIPE)
       gemm_f64_pipe_kernel<<<(int)std::min<long long>(tiles, 152LL * 8), 256, 0, s>>>(t, n, tiles);
-    else if (i == F64_SHORT && l.tn == 32) launch_f64_tc<32, false>(t, n, tiles, device, sms, err, s);
-    else if (i == F64_SHORT) launch_f64_tc<64, false>(t, n, tiles, device, sms, err, s);
-    else launch_f64_tc<32, true>(t, n, tiles, device, sms, err, s);
+    else if (i == F64_SHORT && l.tn == 32) launch_f64_tc<32, false>(t, n, tiles, device, sms, err, s, wait_ns);
+    else if (i == F64_SHORT) launch_f64_tc<64, false>(t, n, tiles, device, sms, err, s, wait_ns);
+    else launch_f64_tc<32, true>(t, n, tiles, device, sms, err, s, wait_ns);
     t += n;
     ++launches;
   }

@@ -79,8 +79,10 @@ void plan_f64(const GemmTask* g, int n, F64Plan& p);
 size_t f64_plan_bytes(const F64Plan& p);
 void upload_f64(const F64Plan& p, void* d, cudaStream_t s);
 // Runs the lists uploaded at d; returns the number of launches.  The
-// tensor-core kernel takes at most `sms` SMs and records an expired wait in *err.
-int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s);
+// tensor-core kernel takes at most `sms` SMs and records a wait of more than
+// wait_ns in *err.
+int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s,
+               unsigned long long wait_ns = 2000000000ull);
 
 // Fill tile bookkeeping; returns total number of tiles.
 long long plan_copy_tiles(CopyTask* t, int n);

@@ -1084,6 +1084,12 @@ int sm_count_dev(int device) {
   return n;
 }
 
+unsigned long long wait_bound_ns(const Ctx& c) {
+  const double s = c.opts.wait_timeout_s;
+  if (!(s > 0.0)) return WAIT_NS;
+  return (unsigned long long)(std::min(s, 60.0) * 1e9);
+}
+
 namespace {
 
 int sm_count(Ctx& c) { return sm_count_dev(c.device); }
@@ -1207,13 +1213,6 @@ void launch_tc_stream(cudaStream_t st, int grid, int prec, const TcTask* d_tasks
                       int* err, unsigned long long wait_ns = WAIT_NS, int cap = 256, int cfg = 0) {
   if (cfg == 1) launch_cfg<1>(st, grid, prec, d_tasks, ntasks, total, err, wait_ns, cap);
   else launch_cfg<0>(st, grid, prec, d_tasks, ntasks, total, err, wait_ns, cap);
-}
-
-// bound on each mbarrier wait of a context's tensor-core launches
-unsigned long long wait_bound_ns(const Ctx& c) {
-  const double s = c.opts.wait_timeout_s;
-  if (!(s > 0.0)) return WAIT_NS;
-  return (unsigned long long)(std::min(s, 60.0) * 1e9);
 }
 
 void launch_tc(Ctx& c, int prec, const TcTask* d_tasks, int ntasks, long long total, int* err, int cap = 256,

@@ -43,18 +43,39 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// bounded wait; on expiry sets *err and returns false
+// The same without the suspension.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 __device__ __forceinline__ unsigned long long gtimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
 
+// Bounded wait; on expiry sets *err and returns false.  try_wait suspends the
+// thread for longer than the few microseconds that one step's products take, so
+// bounds of that order poll instead.
 __device__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code, unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
+  constexpr unsigned long long SHORT_NS = 10000;
+  auto try_wait = [&]() {
+    return limit_ns < SHORT_NS ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity);
+  };
+  if (try_wait()) return true;
   const unsigned long long t0 = gtimer();
   for (;;) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (try_wait()) return true;
     if (gtimer() - t0 > limit_ns) break;
     __nanosleep(32);
   }
