@@ -24,26 +24,51 @@ void reset_families(Ctx& c) {
   c.series_valid = false;
 }
 
+// Waits for products that no step of the call has waited for (the last
+// environments of a sweep, say) and throws if one gave up.
+void finish_products(Ctx& c) {
+  if (!c.products_open) return;
+  cuda_check(cudaStreamSynchronize(c.s()), "end of call");
+  check_products(c);
+}
+
 template <class F>
 mpslcc_status guard(mpslcc_ctx* ctx, F&& f) {
   if (!ctx) return MPSLCC_E_ARG;
+  Ctx& c = ctx->c;
+  mpslcc_status st = MPSLCC_OK;
+  bool spoiled = false;   // a product gave up: environments made from it may have been kept
+  std::string err;
   try {
-    f(ctx->c);
-    ctx->c.err.clear();
-    return MPSLCC_OK;
-  } catch (const Error& e) {
-    ctx->c.err = e.what();
-    if (!ctx->c.host_only) cudaGetLastError();
-    // an expired wait may be found after the environments it spoiled were kept
-    if (e.status == ST_TIMEOUT) reset_families(ctx->c);
-    return (mpslcc_status)e.status;
-  } catch (const std::bad_alloc&) {
-    ctx->c.err = "host allocation failed";
-    return MPSLCC_E_NOMEM;
-  } catch (const std::exception& e) {
-    ctx->c.err = e.what();
-    return MPSLCC_E_INTERNAL;
+    try {
+      f(c);
+      finish_products(c);
+    } catch (const Error& e) {
+      err = e.what();
+      if (!c.host_only) cudaGetLastError();
+      st = (mpslcc_status)e.status;
+      spoiled = e.status == ST_TIMEOUT;
+    } catch (const std::bad_alloc&) {
+      err = "host allocation failed";
+      st = MPSLCC_E_NOMEM;
+    } catch (const std::exception& e) {
+      err = e.what();
+      st = MPSLCC_E_INTERNAL;
+    }
+    if (st != MPSLCC_OK) {   // the call's own failure is the one reported
+      try {
+        finish_products(c);
+      } catch (const Error& e) {
+        cudaGetLastError();
+        spoiled = true;
+      }
+    }
+    if (spoiled) reset_families(c);
+    c.err = err;
+  } catch (const std::exception&) {
+    if (st == MPSLCC_OK) st = MPSLCC_E_INTERNAL;
   }
+  return st;
 }
 
 void need_device(Ctx& c) { MPSLCC_REQUIRE(!c.host_only, ST_STATE, "host-only context cannot run kernels"); }

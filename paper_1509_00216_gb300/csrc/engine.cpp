@@ -175,15 +175,21 @@ void run_f64(Ctx& c, const F64Launch& l, const void* d) {
   const int sms = std::max(1, sm_count_dev(c.device) - std::max(0, c.tc_sm_reserve));
   const int n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s(), wait_bound_ns(c));
   cuda_check(cudaGetLastError(), "gemm_f64 launch");
+  if (n > 0) c.products_open = true;
   c.st.gemm_launches += n;
   c.st.kernel_launches += n;
 }
 
-void check_f64(Ctx& c) {
-  const int h = c.out ? c.out->flag[0] : 0;
-  if (!h) return;
-  c.out->flag[0] = 0;
-  throw Error(ST_TIMEOUT, "FP64 product gave up waiting on an mbarrier (code " + std::to_string(h) + ")");
+// Both flags: a call may launch FP64 products (its environments) and end with
+// others, and a result must not leave it if either kind gave up.
+void check_products(Ctx& c) {
+  if (!c.out) return;
+  const int f64 = c.out->flag[0], tc = c.out->flag[1];
+  c.out->flag[0] = c.out->flag[1] = 0;
+  c.products_open = false;
+  if (f64) throw Error(ST_TIMEOUT, "FP64 product gave up waiting on an mbarrier (code " + std::to_string(f64) + ")");
+  if (tc)
+    throw Error(ST_TIMEOUT, "tensor-core kernel gave up waiting on an mbarrier (code " + std::to_string(tc) + ")");
 }
 
 void run_gemm_tasks(Ctx& c, std::vector<GemmTask>& t) {
@@ -216,7 +222,7 @@ Reduction reduction(Ctx& c) {
 
 void wait_dots(Ctx& c, double* r1, double* r2) {
   cuda_check(cudaStreamSynchronize(c.s()), "dot sync");
-  check_f64(c);
+  check_products(c);
   *r1 = c.out->red[0];
   if (r2) *r2 = c.out->red[1];
 }
@@ -1211,7 +1217,7 @@ void sigma_apply(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
   c.st.sigma_calls++;
   c.st.sigma_flops += P.flops;
   cuda_check(cudaEventSynchronize(c.ev_p2), "sigma phase sync");
-  check_f64(c);
+  check_products(c);
   float m1 = 0, m2 = 0;
   cudaEventElapsedTime(&m1, c.ev_p0, c.ev_p1);
   cudaEventElapsedTime(&m2, c.ev_p1, c.ev_p2);

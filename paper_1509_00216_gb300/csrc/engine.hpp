@@ -273,6 +273,7 @@ struct Ctx {
   volatile HostOut* out = nullptr;
   HostOut* out_dev = nullptr;
   cudaMemPool_t pool = nullptr;   // of the stream-ordered allocations (no caller allocator)
+  bool products_open = false;   // products launched since check_products last looked
   bool sigma_open = false;   // ev0 .. ev1 bracket a local product whose time is not yet in the statistics
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_p0 = nullptr, ev_p1 = nullptr, ev_p2 = nullptr;
 
@@ -375,8 +376,9 @@ void upload_boxes(Ctx& c, int which);
 void run_gemms(Ctx& c, std::vector<GemmTask>& t);
 void run_gemms_tc(Ctx& c, std::vector<GemmTask>& t);
 void run_f64(Ctx& c, const F64Launch& l, const void* d);
-// Throws ST_TIMEOUT if an FP64 product of the (synchronised) stream gave up.
-void check_f64(Ctx& c);
+// Throws ST_TIMEOUT if a product of the (synchronised) stream, FP64 or other, gave
+// up, and clears what it reported.
+void check_products(Ctx& c);
 int sm_count_dev(int device);
 // Bound on each mbarrier wait of a context's tensor-core launches.
 unsigned long long wait_bound_ns(const Ctx& c);

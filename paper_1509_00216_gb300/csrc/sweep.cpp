@@ -49,7 +49,7 @@ std::vector<double> multidot(Ctx& c, const double* V, long ld, int m, const doub
   if (!host)
     cuda_check(cudaMemcpyAsync(out.data(), c.red_out.p, m * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "mdot");
   cuda_check(cudaStreamSynchronize(c.s()), "mdot sync");
-  check_f64(c);
+  check_products(c);
   if (host)
     for (int j = 0; j < m; ++j) out[j] = c.out->red[j];
   return out;
@@ -516,7 +516,7 @@ double truncate(Ctx& c, MPS& m, int l, const double* psi, int M, bool moving_rig
   cuda_check(cudaMemcpyAsync(hw.data(), w.p, wtot * sizeof(double), cudaMemcpyDeviceToHost, c.s()), "eig d2h");
   cuda_check(cudaMemcpyAsync(hinfo.data(), info.p, ns * sizeof(int), cudaMemcpyDeviceToHost, c.s()), "eig info d2h");
   cuda_check(cudaStreamSynchronize(c.s()), "eig sync");
-  check_f64(c);
+  check_products(c);
   for (int i = 0; i < ns; ++i)
     MPSLCC_REQUIRE(hinfo[i] == 0, ST_CUDA,
                    "cusolverDnDsyevd did not converge for a density-matrix sector of dimension " +
@@ -597,7 +597,7 @@ double truncate(Ctx& c, MPS& m, int l, const double* psi, int M, bool moving_rig
   }
   run_gemm_tasks(c, ct);
   cuda_check(cudaStreamSynchronize(c.s()), "truncation sync");
-  check_f64(c);
+  check_products(c);
   // the new bond and both site tensors are committed together, after every
   // step that can fail, so a failed truncation leaves the MPS as it was
   m.bond[l + 1] = nb;

@@ -1223,6 +1223,7 @@ void launch_tc(Ctx& c, int prec, const TcTask* d_tasks, int ntasks, long long to
   int grid = (int)std::min<long long>(total, (long long)sms * per_sm);
   launch_tc_stream(c.s(), grid, prec, d_tasks, ntasks, total, err, wait_bound_ns(c), cap, cfg);
   cuda_check(cudaGetLastError(), "tc_gemm launch");
+  c.products_open = true;
   c.st.kernel_launches++;
   c.st.gemm_launches++;
 }
@@ -1285,14 +1286,10 @@ void run_conv(Ctx& c, int prec, std::vector<ConvTask>& t, DBuf& dtasks) {
 
 int* tc_flag(Ctx& c) { return &c.out_dev->flag[1]; }
 
-// Waits for the stream; throws if a tensor-core product gave up.
+// Waits for the stream; throws if a product gave up.
 void check_err(Ctx& c) {
   cuda_check(cudaStreamSynchronize(c.s()), "tc sync");
-  const int h = c.out->flag[1];
-  if (h) {
-    c.out->flag[1] = 0;
-    throw Error(ST_TIMEOUT, "tensor-core kernel gave up waiting on an mbarrier (code " + std::to_string(h) + ")");
-  }
+  check_products(c);
 }
 
 }  // namespace
