@@ -1007,7 +1007,7 @@ static F64Task make_task(const GemmTask& g, const F64Dims& d, const F64Form& f) 
   t.kr = g.kr;
   t.nkr = g.nkr;
   t.alpha = g.alpha;
-  t.beta = g.beta;
+  t.beta = d.ksplit > 1 ? 0.0 : g.beta;   // partial sums: what lies there is not C
   t.ksplit = d.ksplit;
   MPSLCC_REQUIRE(t.ksplit == 1 || g.sK > 0, ST_INTERNAL, "FP64 task split over K without partial offsets");
   t.sK = t.ksplit > 1 ? g.sK : 0;

@@ -115,6 +115,17 @@ struct Fill {
 int main(int argc, char** argv) {
   const bool run = argc > 1 && std::strcmp(argv[1], "run") == 0;
   bool good = true;
+  for (int ks : {1, 4}) {   // the parts of a split sum never add what lies at C
+    Case c = {"", 300, 200, 2500, GEMM_TB, 1, NORMAL, LONG, false, 1, 0.5};
+    GemmTask g = task(c, nullptr, nullptr, nullptr, nullptr, 0, 0);
+    g.ksplit = ks;
+    g.sK = g.sC;
+    F64Plan p;
+    plan_f64(&g, 1, p);
+    for (const auto& l : p.t)
+      for (const auto& t : l)
+        if (t.beta != (ks == 1 ? 0.5 : 0.0)) { printf("%d splits: beta %g\n", ks, t.beta); good = false; }
+  }
   for (const Case& c : CASES) {
     int nkr = 0, kv = c.k;
     std::vector<int> kr;
