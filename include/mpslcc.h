@@ -96,7 +96,10 @@ typedef struct {
   unsigned long long seed;   /* initial-guess MPS seed                       */
   int verbose;
   /* Optional device allocator (e.g. a framework's caching allocator).  NULL
-     means cudaMallocAsync / cudaFreeAsync on the context stream. */
+     means stream-ordered allocation on the context stream from a memory pool
+     of the context's own.  The pool keeps up to 4 GiB of what was freed for
+     later calls; it gives that back when an allocation of any context of the
+     process on the device fails, and when the context is destroyed. */
   void* (*alloc)(size_t bytes, void* user);
   void (*free)(void* ptr, size_t bytes, void* user);
   void* alloc_user;

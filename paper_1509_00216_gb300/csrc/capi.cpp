@@ -170,19 +170,7 @@ mpslcc_status mpslcc_create(mpslcc_ctx** out, const mpslcc_opts* opts) {
     std::memset(out, 0, sizeof(*out));
     c.out = out;
     cuda_check(cudaHostGetDevicePointer((void**)&c.out_dev, out, 0), "host results address");
-    if (!c.opts.alloc) {
-      // The context's own pool.  It keeps up to 4 GiB between synchronisations
-      // (the device's default pool keeps nothing: every buffer of every step was
-      // mapped anew) and is given back with the context.
-      cudaMemPoolProps props;
-      std::memset(&props, 0, sizeof(props));
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = c.device;
-      cuda_check(cudaMemPoolCreate(&c.pool, &props), "memory pool");
-      unsigned long long keep = 4ull << 30;
-      cuda_check(cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &keep), "memory pool threshold");
-    }
+    if (!c.opts.alloc) create_pool(c);
     for (cudaEvent_t* e : {&c.ev0, &c.ev1, &c.ev_p0, &c.ev_p1, &c.ev_p2}) cuda_check(cudaEventCreate(e), "event");
   });
   if (st != MPSLCC_OK) {
@@ -225,7 +213,7 @@ mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
       cudaStreamDestroy(c.stream);
       c.stream = nullptr;   // a buffer released after this point is freed synchronously
     }
-    if (c.pool) cudaMemPoolDestroy(c.pool);   // goes away with its last buffer
+    destroy_pool(c);
   }
   delete ctx;
   return MPSLCC_OK;

@@ -17,6 +17,7 @@
 #include <cstring>
 #include <ctime>
 #include <functional>
+#include <mutex>
 
 namespace mpslcc {
 
@@ -40,6 +41,47 @@ void cuda_check(cudaError_t e, const char* what) {
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// The pools of all contexts of the process: what one keeps idle is given back when
+// an allocation of another fails.
+namespace {
+std::mutex pools_mutex;
+std::vector<std::pair<int, cudaMemPool_t>> pools;   // device, pool
+}  // namespace
+
+void create_pool(Ctx& c) {
+  // It keeps up to 4 GiB between synchronisations (the device's default pool
+  // keeps nothing: every buffer of every step was mapped anew).  What mapping costs:
+  // a sigma at M1 = 1500, whose buffers pass the 4 GiB, takes 127 ms, and 26 ms with
+  // a caller's allocator that keeps them all.
+  cudaMemPoolProps props;
+  std::memset(&props, 0, sizeof(props));
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = c.device;
+  cuda_check(cudaMemPoolCreate(&c.pool, &props), "memory pool");
+  unsigned long long keep = 4ull << 30;
+  cuda_check(cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &keep), "memory pool threshold");
+  std::lock_guard<std::mutex> lock(pools_mutex);
+  pools.push_back({c.device, c.pool});
+}
+
+void destroy_pool(Ctx& c) {
+  if (!c.pool) return;
+  {
+    std::lock_guard<std::mutex> lock(pools_mutex);
+    pools.erase(std::remove(pools.begin(), pools.end(), std::make_pair(c.device, c.pool)), pools.end());
+  }
+  cudaMemPoolDestroy(c.pool);   // goes away with its last buffer
+  c.pool = nullptr;
+}
+
+static void trim_pools(int device) {
+  cudaDeviceSynchronize();   // frees that are still ordered on some stream
+  std::lock_guard<std::mutex> lock(pools_mutex);
+  for (const auto& p : pools)
+    if (p.first == device) cudaMemPoolTrimTo(p.second, 0);
+}
+
 void DBuf::alloc(Ctx* ctx, size_t nbytes) {
   c = ctx;
   bytes = nbytes;
@@ -51,10 +93,9 @@ void DBuf::alloc(Ctx* ctx, size_t nbytes) {
   } else {
     cudaError_t e = ctx->pool ? cudaMallocFromPoolAsync(&p, nbytes, ctx->pool, ctx->stream)
                               : cudaMallocAsync(&p, nbytes, ctx->stream);
-    if (e != cudaSuccess && ctx->pool) {   // give back what the pool keeps, and try once more
+    if (e != cudaSuccess && ctx->pool) {   // give back what the pools keep, and try once more
       cudaGetLastError();
-      cudaStreamSynchronize(ctx->stream);
-      cudaMemPoolTrimTo(ctx->pool, 0);
+      trim_pools(ctx->device);
       e = cudaMallocFromPoolAsync(&p, nbytes, ctx->pool, ctx->stream);
     }
     if (e != cudaSuccess) {

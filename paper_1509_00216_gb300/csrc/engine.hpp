@@ -372,6 +372,9 @@ struct Ctx {
 };
 
 // ---- engine entry points (engine.cpp / sweep.cpp) ----
+// The context's own pool of device memory.
+void create_pool(Ctx& c);
+void destroy_pool(Ctx& c);
 void upload_boxes(Ctx& c, int which);
 void run_gemms(Ctx& c, std::vector<GemmTask>& t);
 void run_gemms_tc(Ctx& c, std::vector<GemmTask>& t);
