@@ -96,6 +96,40 @@ void build_partition_mpos(Ctx& c) {
   }
 }
 
+// Gives back what a context holds on the device (all of it, or what creation made
+// before it failed).
+void release_device(Ctx& c) {
+  cudaSetDevice(c.device);
+  // every member that owns device memory is released here, while the
+  // stream its frees are ordered on still exists
+  reset_families(c);
+  c.phi0 = MPS();
+  c.phi1 = MPS();
+  c.phin.clear();
+  c.ofam.clear();
+  for (auto& b : c.boxes) b.release();
+  for (DBuf* b : {&c.red, &c.red_out, &c.red_ticket, &c.gtask, &c.ctask, &c.eig_work, &c.eig_w, &c.eig_info, &c.scratch_a,
+                  &c.scratch_b, &c.scratch_tc, &c.tc_conv_tasks, &c.tc_gemm_tasks})
+    b->release();
+  for (int s = 0; s < Ctx::NEIG; ++s) c.eig_ws[s].release();
+  cudaStreamSynchronize(c.stream);
+  for (int s = 0; s < Ctx::NEIG; ++s) {
+    if (c.eig_solver[s]) cusolverDnDestroy(c.eig_solver[s]);
+    if (c.eig_stream[s]) cudaStreamDestroy(c.eig_stream[s]);
+    if (c.eig_ev[s]) cudaEventDestroy(c.eig_ev[s]);
+  }
+  if (c.eig_fork) cudaEventDestroy(c.eig_fork);
+  if (c.out) cudaFreeHost((void*)c.out);
+  if (c.solver) cusolverDnDestroy(c.solver);
+  for (cudaEvent_t e : {c.ev0, c.ev1, c.ev_p0, c.ev_p1, c.ev_p2})
+    if (e) cudaEventDestroy(e);
+  if (c.own_stream && c.stream) {
+    cudaStreamDestroy(c.stream);
+    c.stream = nullptr;   // a buffer released after this point is freed synchronously
+  }
+  destroy_pool(c);
+}
+
 Family& family_for(Ctx& c, int op) {
   MPS* bra = nullptr;
   MPS* ket = nullptr;
@@ -174,6 +208,7 @@ mpslcc_status mpslcc_create(mpslcc_ctx** out, const mpslcc_opts* opts) {
     for (cudaEvent_t* e : {&c.ev0, &c.ev1, &c.ev_p0, &c.ev_p1, &c.ev_p2}) cuda_check(cudaEventCreate(e), "event");
   });
   if (st != MPSLCC_OK) {
+    if (ctx->c.stream) release_device(ctx->c);   // the first thing made
     delete ctx;
     return st;
   }
@@ -183,38 +218,7 @@ mpslcc_status mpslcc_create(mpslcc_ctx** out, const mpslcc_opts* opts) {
 
 mpslcc_status mpslcc_destroy(mpslcc_ctx* ctx) {
   if (!ctx) return MPSLCC_E_ARG;
-  Ctx& c = ctx->c;
-  if (!c.host_only) {
-    cudaSetDevice(c.device);
-    // every member that owns device memory is released here, while the
-    // stream its frees are ordered on still exists
-    reset_families(c);
-    c.phi0 = MPS();
-    c.phi1 = MPS();
-    c.phin.clear();
-    c.ofam.clear();
-    for (auto& b : c.boxes) b.release();
-    for (DBuf* b : {&c.red, &c.red_out, &c.red_ticket, &c.gtask, &c.ctask, &c.eig_work, &c.eig_w, &c.eig_info, &c.scratch_a,
-                    &c.scratch_b, &c.scratch_tc, &c.tc_conv_tasks, &c.tc_gemm_tasks})
-      b->release();
-    for (int s = 0; s < Ctx::NEIG; ++s) c.eig_ws[s].release();
-    cudaStreamSynchronize(c.stream);
-    for (int s = 0; s < Ctx::NEIG; ++s) {
-      if (c.eig_solver[s]) cusolverDnDestroy(c.eig_solver[s]);
-      if (c.eig_stream[s]) cudaStreamDestroy(c.eig_stream[s]);
-      if (c.eig_ev[s]) cudaEventDestroy(c.eig_ev[s]);
-    }
-    if (c.eig_fork) cudaEventDestroy(c.eig_fork);
-    if (c.out) cudaFreeHost((void*)c.out);
-    if (c.solver) cusolverDnDestroy(c.solver);
-    for (cudaEvent_t e : {c.ev0, c.ev1, c.ev_p0, c.ev_p1, c.ev_p2})
-      if (e) cudaEventDestroy(e);
-    if (c.own_stream && c.stream) {
-      cudaStreamDestroy(c.stream);
-      c.stream = nullptr;   // a buffer released after this point is freed synchronously
-    }
-    destroy_pool(c);
-  }
+  if (!ctx->c.host_only) release_device(ctx->c);
   delete ctx;
   return MPSLCC_OK;
 }

@@ -147,9 +147,26 @@ static bool idle_memory() {
   return nothing_left("idle memory") && ok;
 }
 
+// a context whose creation fails half way leaves nothing behind
+static bool failed_create() {
+  for (int n = 0;; ++n) {
+    created = 0;
+    fail_at = n;
+    mpslcc_ctx* c = nullptr;
+    const mpslcc_status st = mpslcc_create(&c, nullptr);
+    fail_at = -1;
+    if (st == MPSLCC_OK) {
+      mpslcc_destroy(c);
+      return n > 5 && nothing_left("destroyed");
+    }
+    if (c || !nothing_left(("creation step " + std::to_string(n)).c_str())) return false;
+  }
+}
+
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "idle_memory") return idle_memory() ? 0 : 1;
+  if (what == "failed_create") return failed_create() ? 0 : 1;
   printf("no such case\n");
   return 2;
 }
