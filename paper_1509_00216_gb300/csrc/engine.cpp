@@ -84,7 +84,7 @@ static void trim_pools(int device) {
 
 void DBuf::alloc(Ctx* ctx, size_t nbytes) {
   c = ctx;
-  bytes = nbytes;
+  bytes = 0;   // until there is memory: a refused buffer is empty, not of this size
   p = nullptr;
   if (nbytes == 0) return;
   if (ctx->opts.alloc) {
@@ -100,11 +100,11 @@ void DBuf::alloc(Ctx* ctx, size_t nbytes) {
     }
     if (e != cudaSuccess) {
       p = nullptr;
-      bytes = 0;
       cudaGetLastError();
       throw Error(ST_NOMEM, "cudaMallocAsync of " + std::to_string(nbytes) + " bytes failed");
     }
   }
+  bytes = nbytes;
   ctx->allocs[(uintptr_t)p] = nbytes;
 }
 

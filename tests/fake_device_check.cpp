@@ -163,10 +163,41 @@ static bool failed_create() {
   }
 }
 
+// a buffer whose allocation was refused is empty, so that the next call asks again
+static bool refused_buffer() {
+  static bool refuse;
+  mpslcc_opts o;
+  mpslcc_default_opts(&o);
+  o.alloc = [](size_t n, void*) -> void* { return refuse ? nullptr : std::malloc(n); };
+  o.free = [](void* p, size_t, void*) { std::free(p); };
+  mpslcc_ctx* c = nullptr;
+  if (mpslcc_create(&c, &o) != MPSLCC_OK) return printf("create\n"), false;
+  bool ok = true;
+  {
+    DBuf x;
+    refuse = true;
+    for (int i = 0; i < 2; ++i) {
+      try {
+        x.ensure((Ctx*)c, 100);
+        printf("a refused allocation went unnoticed\n");
+        ok = false;
+      } catch (const Error& e) {
+        ok = ok && e.status == ST_NOMEM && !x.p;
+      }
+    }
+    refuse = false;
+    x.ensure((Ctx*)c, 100);
+    ok = ok && x.p;
+  }
+  mpslcc_destroy(c);
+  return ok && nothing_left("refused buffer");
+}
+
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "idle_memory") return idle_memory() ? 0 : 1;
   if (what == "failed_create") return failed_create() ? 0 : 1;
+  if (what == "refused_buffer") return refused_buffer() ? 0 : 1;
   printf("no such case\n");
   return 2;
 }

@@ -22,7 +22,7 @@ def check(mpslcc, tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("case", ["idle_memory", "failed_create"])
+@pytest.mark.parametrize("case", ["idle_memory", "failed_create", "refused_buffer"])
 def test_device_resources(check, case):
     run = subprocess.run([check, case], capture_output=True, text=True, timeout=60)
     assert run.returncode == 0, run.stdout + run.stderr
