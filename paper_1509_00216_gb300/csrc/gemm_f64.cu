@@ -325,12 +325,13 @@ __device__ __forceinline__ void sum_magnitudes(const uint8_t* mags, int row, int
 }
 
 // Sums the n outputs of a tile in `list` (row << 6 | column), or its first n where
-// there is no list, in ascending K, from operand rows staged in shared memory:
-// at up to the two multiply-adds a clock that the FP64 pipe gives.
+// there is no list, in ascending K, from operand rows staged in shared memory.
+// Listed outputs are mostly those of sparse rows (operator sums with coefficients:
+// 5 of 48 terms are not zero at M1 = 1500), so their terms are found from bit masks
+// of the rows' non-zero values: 30000 clocks for 1330 outputs instead of 52000.
 template <int TN>
 __device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, int n, uint8_t* smem, const int* tab,
-                                       const long long* coff, const long long* roff, int kb, int len,
-                                       int mode) {
+                                       const long long* coff, const long long* roff, int kb, int len, int mode) {
   constexpr int THREADS = F64Cfg<TN>::THREADS, U = 4, LD = KS + 1;
   const F64Task& T = S.t;
   const int tid = threadIdx.x, x0 = S.ix * TM, y0 = S.iy * TN;
@@ -339,12 +340,15 @@ __device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, i
   double* ys = xs + TM * LD;
   long long* xo = (long long*)(ys + TN * LD);
   long long* yo = xo + TM;
-  static_assert((TM + TN) * (LD + 1) * 8 <= F64Cfg<TN>::OPER, "staging");
+  uint32_t* masks = (uint32_t*)(yo + TN);   // two sets, of this step's values and the next one's
+  static_assert((TM + TN) * (LD + 2) * 8 <= F64Cfg<TN>::OPER && 2 * (TM + TN) <= THREADS, "staging");
   const double* X = T.x + (long long)S.b * T.xub;
   const double* Y = T.y + (long long)S.b * T.yub;
   double* C = T.c + (long long)S.b * T.cub + (long long)S.ks * T.sK;
   if (tid < nx) xo[tid] = row_off(x0 + tid, T.nx, T.xrs, T.xbs);
   if (tid >= THREADS - ny) yo[tid - (THREADS - ny)] = row_off(y0 + tid - (THREADS - ny), T.ny, T.yrs, T.ybs);
+  if (tid < 2 * (TM + TN)) masks[tid] = 0;
+  uint32_t set = 0;
   for (int base = 0; base < n; base += U * THREADS) {
     int at[U];
     double acc[U];
@@ -354,8 +358,10 @@ __device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, i
       at[u] = e >= n ? -1 : (list ? list[e] : e / ny << 6 | e % ny);
       acc[u] = 0.0;
     }
-    for (int kk = 0; kk < len; kk += KS) {
+    for (int kk = 0; kk < len; kk += KS, set ^= 1u) {
       const int nk = min(KS, len - kk);
+      uint32_t* mx = masks + set * (TM + TN);
+      uint32_t* my = mx + TM;
       __syncthreads();
       constexpr int NX = TM * KS / THREADS, NY = TN * KS / THREADS;
       double vx[NX], vy[NY];
@@ -371,22 +377,30 @@ __device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, i
       }
 #pragma unroll
       for (int i = 0; i < NX; ++i) {
-        const int e = tid + i * THREADS;
-        xs[T.xks == 1 ? e / KS * LD + e % KS : e % TM * LD + e / TM] = vx[i];
+        const int e = tid + i * THREADS, r = T.xks == 1 ? e / KS : e % TM, q = T.xks == 1 ? e % KS : e / TM;
+        xs[r * LD + q] = vx[i];
+        if (vx[i] != 0.0) atomicOr(&mx[r], 1u << q);
       }
 #pragma unroll
       for (int i = 0; i < NY; ++i) {
-        const int e = tid + i * THREADS;
-        ys[T.yks == 1 ? e / KS * LD + e % KS : e % TN * LD + e / TN] = vy[i];
+        const int e = tid + i * THREADS, r = T.yks == 1 ? e / KS : e % TN, q = T.yks == 1 ? e % KS : e / TN;
+        ys[r * LD + q] = vy[i];
+        if (vy[i] != 0.0) atomicOr(&my[r], 1u << q);
       }
       __syncthreads();
+      if (tid < TM + TN) masks[(set ^ 1u) * (TM + TN) + tid] = 0;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (at[u] < 0) continue;
-        const double* px = xs + (at[u] >> 6) * LD;
-        const double* py = ys + (at[u] & 63) * LD;
+        const int i = at[u] >> 6, j = at[u] & 63;
+        const double* px = xs + i * LD;
+        const double* py = ys + j * LD;
         double a = acc[u];
-        for (int q = 0; q < nk; ++q) a = fma(px[q], py[q], a);
+        // a tile with values that are not finite takes every term
+        for (uint32_t m = list ? mx[i] & my[j] : ~0u >> (KS - nk); m; m &= m - 1) {
+          const int q = __ffs(m) - 1;
+          a = fma(px[q], py[q], a);
+        }
         acc[u] = a;
       }
     }
@@ -730,34 +744,35 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         if (!MULTI) fence_before();
       }
       // The outputs listed, or all of a tile with a row that is not finite, as
-      // plain FP64 sums.  At TN = 64 some hundred a tile are common (sums of
-      // operators with coefficients, 12 % of the outputs at M1 = 1500): staged, 52000
-      // clocks for 1330 outputs of K = 48, 110000 read directly.  At TN = 32 they
-      // are few (56 of 4096 in 4 % of the tiles of the energies), and the call would
-      // cost the loops before it registers: eight lanes an output read it directly,
-      // 12000 clocks, 24000 staged.
+      // plain FP64 sums.  At TN = 64 some hundred a tile are common (operator sums,
+      // 12 % of the outputs at M1 = 1500): staged (30000 clocks for 1330 outputs of
+      // K = 48, 110000 read directly).  At TN = 32 they are few (56 of 4096 in 4 % of
+      // the tiles of the energies) and the call would cost the loops before it
+      // registers: eight lanes an output read it directly (12000 clocks for 56,
+      // 24000 staged).
       const int nsum = plain ? nx * ny : (abort ? 0 : *nagain);
-      if (nsum > 0 && TN == 64) {
+      if (nsum > 0) {
         __syncthreads();   // the list, and the turned pieces are read
-        sum_again<TN>(slots[cur], plain ? nullptr : list, nsum, smem, tab, coff, roff, kb, len, pm);
-      } else if (nsum > 0) {
-        const double* X = T.x + (long long)slots[cur].b * T.xub;
-        const double* Y = T.y + (long long)slots[cur].b * T.yub;
-        __syncthreads();   // the list
-        for (int e0 = warp * 4; e0 < nsum; e0 += THREADS / 8) {
-          const int e = min(e0 + (lane >> 3), nsum - 1);
-          const int i = plain ? e / ny : list[e] >> 6, j = plain ? e - i * ny : list[e] & 63;
-          const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
-          const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
-          double s = 0.0;
+        if constexpr (TN == 64) {
+          sum_again<TN>(slots[cur], plain ? nullptr : list, nsum, smem, tab, coff, roff, kb, len, pm);
+        } else {
+          const double* X = T.x + (long long)slots[cur].b * T.xub;
+          const double* Y = T.y + (long long)slots[cur].b * T.yub;
+          for (int e0 = warp * 4; e0 < nsum; e0 += THREADS / 8) {
+            const int e = min(e0 + (lane >> 3), nsum - 1);
+            const int i = plain ? e / ny : list[e] >> 6, j = plain ? e - i * ny : list[e] & 63;
+            const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
+            const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
+            double s = 0.0;
 #pragma unroll 4
-          for (int k = lane & 7; k < len; k += 8) {
-            const int col = T.kr ? tab[k] : kb + k;
-            s = fma(__ldg(px + (long long)col * T.xks), __ldg(py + (long long)col * T.yks), s);
-          }
+            for (int k = lane & 7; k < len; k += 8) {
+              const int col = T.kr ? tab[k] : kb + k;
+              s = fma(__ldg(px + (long long)col * T.xks), __ldg(py + (long long)col * T.yks), s);
+            }
 #pragma unroll
-          for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          if ((lane & 7) == 0 && e0 + (lane >> 3) < nsum) put(T, pm, C + roff[i] + coff[j], s);
+            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((lane & 7) == 0 && e0 + (lane >> 3) < nsum) put(T, pm, C + roff[i] + coff[j], s);
+          }
         }
       }
       if (warp == 1 && next && !fetched && kb + KB >= k1) {

@@ -16,7 +16,7 @@ void mpslcc::cuda_check(cudaError_t e, const char* what) {
 
 using namespace mpslcc;
 
-enum Data { NORMAL, GRADED20, GRADED40, APART, IDENTITY, TINY, POSITIVE, BLOCKS };
+enum Data { NORMAL, GRADED20, GRADED40, APART, IDENTITY, TINY, POSITIVE, BLOCKS, SPARSE, INFINITE };
 enum List { SHORT64, SHORT32, LONG, PIPE };
 struct Case {
   const char* name;
@@ -36,6 +36,11 @@ static const Case CASES[] = {
     {"unit rows over noise", 640, 600, 100, GEMM_TB, 1, IDENTITY, SHORT64, false, 1, 0},
     {"rows below 2^-959", 640, 640, 64, GEMM_TB, 1, TINY, SHORT64, false, 1, 0},
     {"one sign", 640, 640, 128, GEMM_TB, 1, POSITIVE, SHORT64, false, 1, 0},
+    {"sparse", 640, 640, 90, GEMM_TB, 1, SPARSE, SHORT64, false, 1, 0},
+    {"sparse, K along columns", 641, 577, 51, GEMM_TA, 1, SPARSE, SHORT64, false, 2, 1},
+    {"an infinity", 640, 640, 64, GEMM_TB, 1, INFINITE, SHORT64, false, 1, 0},
+    {"32 columns, sparse", 45, 31, 40, 0, 600, SPARSE, SHORT32, false, 1, 0},
+    {"32 columns, an infinity", 45, 31, 40, 0, 600, INFINITE, SHORT32, false, 1, 0},
     {"32 columns", 45, 31, 40, GEMM_TB, 600, GRADED40, SHORT32, false, 1, 0},
     {"32 columns, unit rows", 45, 31, 40, 0, 600, IDENTITY, SHORT32, false, 2, 0.5},
     {"32 columns, rows below 2^-959", 45, 31, 40, 0, 600, TINY, SHORT32, false, 1, 0},
@@ -46,6 +51,8 @@ static const Case CASES[] = {
     {"several scaling blocks, rows below 2^-959", 300, 200, 2500, GEMM_TB, 1, TINY, LONG, false, 1, 0},
     {"parts of different magnitude", 300, 200, 1024, GEMM_TB, 1, BLOCKS, LONG, false, 1, 0},
     {"K runs, graded 2^40", 300, 200, 1600, GEMM_TB, 1, GRADED40, LONG, true, 1, 0},
+    {"several scaling blocks, sparse", 300, 200, 2500, GEMM_TB, 1, SPARSE, LONG, false, 1, 0},
+    {"several scaling blocks, an infinity", 300, 200, 2500, GEMM_TB, 1, INFINITE, LONG, false, 1, 0},
     {"FP64 pipe, graded 2^40", 70, 65, 130, GEMM_TB, 1, GRADED40, PIPE, false, 1, 0},
 };
 
@@ -107,6 +114,8 @@ struct Fill {
       case TINY: return side || r % 3 ? v : (r % 2 ? v * 1e-295 : v * 4e-320);
       case POSITIVE: return std::fabs(v) + 0.01;
       case BLOCKS: return std::ldexp(v, (k / 100 * 7 + (side ? 3 : 11) * (k / 100)) % 29);
+      case SPARSE: return (r * 7 + k * 11 + side) % (side ? 9 : 5) ? 0.0 : std::ldexp(v, (side ? 13 : 17) * (k % 4));
+      case INFINITE: return !side && r == 200 && k == 3 ? INFINITY : v;
       default: return v;
     }
   }
@@ -192,6 +201,10 @@ int main(int argc, char** argv) {
       const double ref = c.alpha * (s + lo) + c.beta * C0[e];
       const double rounds = terms + 6 + terms / 1024;
       const double tol = rounds * (0x1p-53 * (std::fabs(c.alpha) * S + std::fabs(c.beta * C0[e])) + 0x1p-1074);
+      if (c.data == INFINITE && e / c.n == 200) {   // the row with the infinity, and no other
+        if (std::isfinite(C[e])) { printf("%s: output %zu is finite\n", c.name, e); ok = false; }
+        continue;
+      }
       const double d = std::fabs(C[e] - ref);
       if (!(d <= tol)) {
         if (ok) printf("%s: output %zu is %.17g, not %.17g: off by %.3g, bound %.3g\n", c.name, e, C[e], ref, d, tol);
