@@ -324,6 +324,9 @@ def fp64_compare(mp, mx, c, M0, M1, prec, local_rank, window, torch):
     out = {"positions": list(range(first, first + window)), "direction": "left to right"}
 
     def run(ctx, label):
+        # The sweeps can leave PyTorch's cache as large as the device, and kernels
+        # that load at their first use (the fill below) need memory outside of it.
+        torch.cuda.empty_cache()
         ctx.load_mps(0, p0)
         ctx.dmrg_reference(M0, 0)
         ctx.load_mps(1, p1)
