@@ -108,7 +108,7 @@ void release_device(Ctx& c) {
   c.phin.clear();
   c.ofam.clear();
   for (auto& b : c.boxes) b.release();
-  for (DBuf* b : {&c.red, &c.red_out, &c.red_ticket, &c.gtask, &c.ctask, &c.eig_work, &c.eig_w, &c.eig_info, &c.scratch_a,
+  for (DBuf* b : {&c.f64_doubt, &c.red, &c.red_out, &c.red_ticket, &c.gtask, &c.ctask, &c.eig_work, &c.eig_w, &c.eig_info, &c.scratch_a,
                   &c.scratch_b, &c.scratch_tc, &c.tc_conv_tasks, &c.tc_gemm_tasks})
     b->release();
   for (int s = 0; s < Ctx::NEIG; ++s) c.eig_ws[s].release();

@@ -214,8 +214,27 @@ void run_gemms(Ctx& c, std::vector<GemmTask>& t) {
 
 void run_f64(Ctx& c, const F64Launch& l, const void* d) {
   const int sms = std::max(1, sm_count_dev(c.device) - std::max(0, c.tc_sm_reserve));
-  const int n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s(), wait_bound_ns(c));
-  cuda_check(cudaGetLastError(), "gemm_f64 launch");
+  const size_t want = f64_scratch_bytes(l);
+  if (want > c.f64_doubt.bytes && (c.f64_refused == 0 || want < c.f64_refused)) {
+    try {
+      c.f64_doubt.ensure(&c, want);
+      cuda_check(cudaMemsetAsync(c.f64_doubt.p, 0, 256, c.s()), "clear");
+      c.f64_turn = 0;
+    } catch (const Error& e) {   // not needed for the result
+      if (e.status != ST_NOMEM) throw;
+      c.f64_refused = want;
+    }
+  }
+  F64Scratch scratch{c.f64_doubt.p, c.f64_doubt.bytes, c.f64_turn};
+  int n = 0;
+  try {
+    n = launch_f64(l, d, c.device, sms, &c.out_dev->flag[0], c.s(), wait_bound_ns(c), &scratch);
+    cuda_check(cudaGetLastError(), "gemm_f64 launch");
+  } catch (const Error&) {   // its counts may not be those that the next launch expects
+    c.f64_doubt.release();
+    throw;
+  }
+  c.f64_turn = scratch.turn;
   if (n > 0) c.products_open = true;
   c.st.gemm_launches += n;
   c.st.kernel_launches += n;

@@ -339,6 +339,9 @@ struct Ctx {
   cudaEvent_t eig_ev[NEIG] = {}, eig_fork = nullptr;
   DBuf eig_ws[NEIG];
   DBuf scratch_a, scratch_b;
+  DBuf f64_doubt;              // see F64Scratch
+  unsigned f64_turn = 0;
+  size_t f64_refused = 0;      // a size that could not be had
   DBuf scratch_tc, tc_conv_tasks, tc_gemm_tasks;
   // precision of the per-site FP64 GEMM tasks (fusion, renormalisation,
   // truncation): MPSLCC_FP64, or MPSLCC_BF16X3 inside mixed-precision sweeps

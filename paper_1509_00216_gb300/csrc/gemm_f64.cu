@@ -17,8 +17,12 @@
 // the small ones of the other, an output's error would pass that of a chain of
 // FP64 multiply-adds.  So every output is checked against a lower bound of sum
 // |x y| (sum_magnitudes), and those that might pass the chain's bound, n 2^-53
-// sum |x y|, are summed in FP64 instead.  (Operands graded over 2^40 in opposite
-// directions were off by 1e-8 of sum |x y| before this check.)
+// sum |x y|, are summed in FP64 instead (gemm_f64_again_kernel).  Without the check
+// operands graded over 2^40 in opposite directions are off by 1e-8 of sum |x y|.
+// Few outputs of states with even spectra are in doubt (0 to 13 %), but most of
+// those of large converged states, whose rows are graded by their Schmidt values:
+// there the FP64 pipe bounds the product as it did before (a window of four
+// positions at M1 = 2000: 24 s; 6.5 s unchecked; 40 to 45 s on the FP64 pipe alone).
 //
 // Tasks of few multiply-adds run on the FP64 pipe (gemm_f64_pipe_kernel).
 //
@@ -33,6 +37,7 @@
 #include <atomic>
 #include <vector>
 #include <cstring>
+#include <type_traits>
 
 #include "engine.hpp"
 #include "tcgen05.cuh"
@@ -75,6 +80,23 @@ template <int TN_> struct F64Cfg {
 template <class F> __device__ __forceinline__ int mag_at(int row, int group) {
   return row * F::MROW + ((group ^ (F::MW == 4 ? row & 7 : row >> 1 & 3)) << 4);
 }
+// Tiles with outputs in doubt (see the head of the file), and for each of a tile's
+// blocks of 1024 K values a bit per output, 16 columns of a row a word.
+struct F64Doubt {
+  int* count;
+  long long* rec;
+  uint16_t* mask;
+  int cap, blocks;
+};
+constexpr size_t F64_SCRATCH_HEAD = 256;   // two counts
+inline size_t f64_record_bytes(int tn, int blocks) { return sizeof(long long) + (size_t)blocks * TM * tn / 8; }
+// Tiles of one launch where there are more: 64 MB of records, and no less than some
+// milliseconds of products.
+inline long long f64_launch_tiles(int tn, int blocks) {
+  return (long long)((64u << 20) / f64_record_bytes(tn, blocks));
+}
+constexpr int F64_MAX_BLOCKS = 32;         // outputs in doubt of longer sums are summed in place
+
 struct F64Slot {
   F64Task t;
   int b, ks, ix, iy;
@@ -164,6 +186,8 @@ enum { PUT_SCALE = 1, PUT_BETA = 2, PUT_ADD = 4 };
 __device__ __forceinline__ int put_mode(const F64Task& T, bool first) {
   return (T.alpha != 1.0 ? PUT_SCALE : 0) | (!first ? PUT_ADD : (T.beta != 0.0 ? PUT_BETA : 0));
 }
+// of a sum that joins what lies there
+__device__ __forceinline__ int sum_mode(const F64Task& T) { return (T.alpha != 1.0 ? PUT_SCALE : 0) | PUT_ADD; }
 __device__ __forceinline__ void put(const F64Task& T, int mode, double* c, double v) {
   if (mode) {
     if (mode & PUT_SCALE) v *= T.alpha;
@@ -290,9 +314,9 @@ __device__ __forceinline__ void store_unit(const Unit& u, double (&v)[8], int sc
 // leading eight bits of the operands bound that sum from below: sum (|X| >>
 // 54)(|Y| >> 54) >= 1156 = 9.03 x 2^7 will do.  Where x and y have their large
 // values at different k it may fail, and the output is summed again in FP64
-// (sum_again).  A thread adds up its row's outputs of 16 columns, four at a time,
-// over `steps` of a window and stops with its warp once all have enough (mostly
-// after 32 values); `sums` holds a byte per output, its sum / 16 so far or
+// (gemm_f64_again_kernel).  A thread adds up its row's outputs of 16 columns, four
+// at a time, over `steps` of a window and stops with its warp once all have enough
+// (mostly after 32 values); `sums` holds a byte per output, its sum / 16 so far or
 // ENOUGH_B.
 template <class F>
 __device__ __forceinline__ void sum_magnitudes(const uint8_t* mags, int row, int col0, int steps, uint32_t (&sums)[4]) {
@@ -321,92 +345,6 @@ __device__ __forceinline__ void sum_magnitudes(const uint8_t* mags, int row, int
     sums[g] = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) sums[g] |= (acc[c] >= ENOUGH ? ENOUGH_B : acc[c] >> 4) << (8 * c);
-  }
-}
-
-// Sums the n outputs of a tile in `list` (row << 6 | column), or its first n where
-// there is no list, in ascending K, from operand rows staged in shared memory.
-// Listed outputs are mostly those of sparse rows (operator sums with coefficients:
-// 5 of 48 terms are not zero at M1 = 1500), so their terms are found from bit masks
-// of the rows' non-zero values: 30000 clocks for 1330 outputs instead of 52000.
-template <int TN>
-__device__ __noinline__ void sum_again(const F64Slot& S, const uint16_t* list, int n, uint8_t* smem, const int* tab,
-                                       const long long* coff, const long long* roff, int kb, int len, int mode) {
-  constexpr int THREADS = F64Cfg<TN>::THREADS, U = 4, LD = KS + 1;
-  const F64Task& T = S.t;
-  const int tid = threadIdx.x, x0 = S.ix * TM, y0 = S.iy * TN;
-  const int nx = min(TM, T.mx - x0), ny = min(TN, T.my - y0);
-  double* xs = (double*)smem;
-  double* ys = xs + TM * LD;
-  long long* xo = (long long*)(ys + TN * LD);
-  long long* yo = xo + TM;
-  uint32_t* masks = (uint32_t*)(yo + TN);   // two sets, of this step's values and the next one's
-  static_assert((TM + TN) * (LD + 2) * 8 <= F64Cfg<TN>::OPER && 2 * (TM + TN) <= THREADS, "staging");
-  const double* X = T.x + (long long)S.b * T.xub;
-  const double* Y = T.y + (long long)S.b * T.yub;
-  double* C = T.c + (long long)S.b * T.cub + (long long)S.ks * T.sK;
-  if (tid < nx) xo[tid] = row_off(x0 + tid, T.nx, T.xrs, T.xbs);
-  if (tid >= THREADS - ny) yo[tid - (THREADS - ny)] = row_off(y0 + tid - (THREADS - ny), T.ny, T.yrs, T.ybs);
-  if (tid < 2 * (TM + TN)) masks[tid] = 0;
-  uint32_t set = 0;
-  for (int base = 0; base < n; base += U * THREADS) {
-    int at[U];
-    double acc[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = base + u * THREADS + tid;
-      at[u] = e >= n ? -1 : (list ? list[e] : e / ny << 6 | e % ny);
-      acc[u] = 0.0;
-    }
-    for (int kk = 0; kk < len; kk += KS, set ^= 1u) {
-      const int nk = min(KS, len - kk);
-      uint32_t* mx = masks + set * (TM + TN);
-      uint32_t* my = mx + TM;
-      __syncthreads();
-      constexpr int NX = TM * KS / THREADS, NY = TN * KS / THREADS;
-      double vx[NX], vy[NY];
-#pragma unroll
-      for (int i = 0; i < NX; ++i) {
-        const int e = tid + i * THREADS, r = T.xks == 1 ? e / KS : e % TM, q = T.xks == 1 ? e % KS : e / TM;
-        vx[i] = r < nx && q < nk ? __ldg(X + xo[r] + (long long)(T.kr ? tab[kk + q] : kb + kk + q) * T.xks) : 0.0;
-      }
-#pragma unroll
-      for (int i = 0; i < NY; ++i) {
-        const int e = tid + i * THREADS, r = T.yks == 1 ? e / KS : e % TN, q = T.yks == 1 ? e % KS : e / TN;
-        vy[i] = r < ny && q < nk ? __ldg(Y + yo[r] + (long long)(T.kr ? tab[kk + q] : kb + kk + q) * T.yks) : 0.0;
-      }
-#pragma unroll
-      for (int i = 0; i < NX; ++i) {
-        const int e = tid + i * THREADS, r = T.xks == 1 ? e / KS : e % TM, q = T.xks == 1 ? e % KS : e / TM;
-        xs[r * LD + q] = vx[i];
-        if (vx[i] != 0.0) atomicOr(&mx[r], 1u << q);
-      }
-#pragma unroll
-      for (int i = 0; i < NY; ++i) {
-        const int e = tid + i * THREADS, r = T.yks == 1 ? e / KS : e % TN, q = T.yks == 1 ? e % KS : e / TN;
-        ys[r * LD + q] = vy[i];
-        if (vy[i] != 0.0) atomicOr(&my[r], 1u << q);
-      }
-      __syncthreads();
-      if (tid < TM + TN) masks[(set ^ 1u) * (TM + TN) + tid] = 0;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (at[u] < 0) continue;
-        const int i = at[u] >> 6, j = at[u] & 63;
-        const double* px = xs + i * LD;
-        const double* py = ys + j * LD;
-        double a = acc[u];
-        // a tile with values that are not finite takes every term
-        for (uint32_t m = list ? mx[i] & my[j] : ~0u >> (KS - nk); m; m &= m - 1) {
-          const int q = __ffs(m) - 1;
-          a = fma(px[q], py[q], a);
-        }
-        acc[u] = a;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (at[u] >= 0) put(T, mode, C + roff[at[u] >> 6] + coff[at[u] & 63], acc[u]);
   }
 }
 
@@ -455,27 +393,26 @@ __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
 // same: some 650 bytes a thread are spilled, 500 at TN = 64 with MULTI = false).
 template <int TN, bool MULTI>
 __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
-    gemm_f64_tc_kernel(const F64Task* __restrict__ tasks, int ntasks, long long total, int* err,
-                       unsigned long long wait_ns) {
+    gemm_f64_tc_kernel(const F64Task* __restrict__ tasks, int ntasks, long long tile0, long long total, int* err,
+                       unsigned long long wait_ns, F64Doubt w) {   // tiles tile0 .. total - 1
   using F = F64Cfg<TN>;
   constexpr int THREADS = F::THREADS, XU = F::XU, NBUF = F::NBUF;
   constexpr bool PAIR = !MULTI && XU == 1;            // registers hold two steps' values
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + F::ALIGN - 1) & ~(uintptr_t)(F::ALIGN - 1));
   uint8_t* yplanes = smem + PLANES * F::XPLANE;
-  uint8_t* mags = smem + F::OPER;                     // leading magnitudes of a chunk; then outputs to sum again
+  uint8_t* mags = smem + F::OPER;                     // leading magnitudes of a window; then outputs to sum here
   int* tab = (int*)(mags + F::MAGS);                  // operand column of each K value of the block
   uint32_t* rmax = (uint32_t*)(tab + TAB<MULTI>);     // largest high word per row: X, then Y
   int* rscale = (int*)rmax;                           // then the rows' scales in its place
   uint64_t* bar = (uint64_t*)(rscale + TM + TN);      // [2] products of a buffer done, [1] drain
   volatile uint32_t* tslot = (volatile uint32_t*)(bar + 3);
-  int* nagain = (int*)(bar + 4);                      // outputs to sum again
+  int* nagain = (int*)(bar + 4);                      // a block's outputs in doubt; a tile's record
   F64Slot* slots = (F64Slot*)(bar + 8);               // this tile's task and the next one's
   long long* coff = (long long*)(slots + 2);          // output offset of each column
   long long* roff = coff + TN;                        // and of each row
-  uint16_t* list = (uint16_t*)mags;                   // outputs to sum again (after a block's products)
-  uint16_t* skip = list + TM * TN;                    // and per thread which of its own
-  static_assert(TM * TN * 2 + THREADS * 2 <= F::MAGS, "list");
+  uint16_t* list = (uint16_t*)mags;                   // outputs to sum here (after a block's products)
+  static_assert(TM * TN * 2 <= F::MAGS, "list");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     mbar_init(&bar[0], 1);
@@ -491,7 +428,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   int ti = 0;                                         // warp 1: task of the last slot filled
-  if (warp == 1 && blockIdx.x < total) ti = fetch_slot(&slots[0], tasks, ntasks, blockIdx.x, 0);
+  if (warp == 1 && tile0 + blockIdx.x < total) ti = fetch_slot(&slots[0], tasks, ntasks, tile0 + blockIdx.x, 0);
   fence_before();
   __syncthreads();
   fence_after();
@@ -503,7 +440,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
   bool abort = false;
   int cur = 0;
 
-  for (long long tile = blockIdx.x; tile < total && !abort; tile += gridDim.x, cur ^= 1) {
+  for (long long tile = tile0 + blockIdx.x; tile < total && !abort; tile += gridDim.x, cur ^= 1) {
     const F64Task& T = slots[cur].t;
     const int x0 = slots[cur].ix * TM, y0 = slots[cur].iy * TN;
     const int nx = min(TM, T.mx - x0), ny = min(TN, T.my - y0);
@@ -528,7 +465,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
     if (tid < ny) coff[tid] = row_off(y0 + tid, T.ny, T.cys, T.cyb);
     if (tid >= THREADS - nx) roff[tid - (THREADS - nx)] = row_off(x0 + tid - (THREADS - nx), T.nx, T.cxs, T.cxb);
     const bool mine = quarter * 32 < nx && colq * 16 < ny;
-
+    int rec = -1;                                     // the tile's record of outputs in doubt
     int kb = k0;
     do {
       const int len = max(0, min(KB, k1 - kb));
@@ -586,6 +523,7 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         rscale[tid] = e << 1 | tiny;
       }
       const bool plain = __syncthreads_or(bad);
+      int nsum = plain ? nx * ny : 0;   // outputs to sum here
       const int pm = put_mode(T, kb == k0);
       double* C = T.c + (long long)slots[cur].b * T.cub + (long long)slots[cur].ks * T.sK;
       long long ahi[MULTI ? 16 : 1], alo[MULTI ? 16 : 1];   // sums of accumulators 0 .. 3 and 4 .. 7
@@ -690,7 +628,8 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         if (F::MW == CHUNK) sum_magnitudes<F>(mags, orow, colq * 16, nst, sums);
         if (!MULTI && nst > 0 && !abort) {   // the last step's products
           const uint32_t use = it - 1;
-          if (!mbar_wait(&bar[NBUF == 2 ? use & 1u : 0], (NBUF == 2 ? use >> 1 : use) & 1u, err, 12, wait_ns)) abort = true;
+          const uint32_t parity = (NBUF == 2 ? use >> 1 : use) & 1u;
+          if (!mbar_wait(&bar[NBUF == 2 ? use & 1u : 0], parity, err, 12, wait_ns)) abort = true;
           fence_after();
         }
         uint32_t open = 0;   // outputs to sum again
@@ -699,13 +638,40 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
         int at = 0;
         if (open) at = atomicAdd(nagain, __popc(open));
         abort = __syncthreads_or(abort);
-        for (uint32_t o = open; o; o &= o - 1) list[at++] = (uint16_t)(orow << 6 | (colq * 16 + __ffs(o) - 1));
+        // Outputs in doubt are left to the second kernel, or summed below where there
+        // is no room for their record.
+        nsum = abort ? 0 : *nagain;
+        if (nsum > 0 && w.cap > 0) {
+          if (rec < 0) {   // the tile's first
+            __syncthreads();
+            if (tid == 0) *nagain = atomicAdd(w.count, 1);
+            __syncthreads();
+            rec = *nagain;
+            __syncthreads();
+            if (rec < w.cap) {
+              if (tid == 0) w.rec[rec] = tile;
+              for (int b = 0; MULTI && b < w.blocks; ++b)
+                w.mask[((long long)rec * w.blocks + b) * THREADS + orow * (TN / 16) + colq] = 0;
+            } else {
+              if (tid == 0) *nagain = 0;
+              __syncthreads();
+              at = open ? atomicAdd(nagain, __popc(open)) : 0;
+            }
+          }
+          if (rec < w.cap) {
+            const int b = MULTI ? (kb - k0) / KB : 0;
+            w.mask[((long long)rec * w.blocks + b) * THREADS + orow * (TN / 16) + colq] = (uint16_t)open;
+            nsum = 0;
+          }
+        }
+        if (nsum > 0)
+          for (uint32_t o = open; o; o &= o - 1) list[at++] = (uint16_t)(orow << 6 | (colq * 16 + __ffs(o) - 1));
         // A warp holds 32 rows (one a lane) of 16 columns.  Where rows are
         // contiguous in memory it stores them column by column; else it turns
         // its piece in shared memory (its own part: the products are done) and
         // stores two rows of 16 columns at a time, instead of 32 rows of one.
+        // Outputs in doubt get a zero: their sums are added.
         if (mine && !abort) {
-          const bool some = __any_sync(0xffffffffu, open != 0);
           const int exr = scale_exp(rscale[orow]);
           const bool lanes = T.cxs == 1;
           double* r = C + (orow < nx ? roff[orow] : 0);
@@ -723,56 +689,46 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
               const int col = colq * 16 + cb + j;
-              const double x = to_f64(hi[j], lo[j], exr + scale_exp(rscale[TM + col]));
+              double x = to_f64(hi[j], lo[j], exr + scale_exp(rscale[TM + col]));
+              if (open >> (cb + j) & 1) x = 0.0;
               if (!lanes) st[lane * 17 + cb + j] = x;
-              else if (col < ny && orow < nx && !(open >> (cb + j) & 1)) put(T, pm, r + coff[col], x);
+              else if (col < ny && orow < nx) put(T, pm, r + coff[col], x);
             }
           }
           if (!lanes) {
-            if (some) skip[tid] = (uint16_t)open;
             __syncwarp();
             const int col = colq * 16 + (lane & 15);
             double* c = C + (col < ny ? coff[col] : 0);
 #pragma unroll 4
             for (int i = lane >> 4; i < 32; i += 2) {
               const int row = quarter * 32 + i;
-              if (row < nx && col < ny && !(some && (skip[warp * 32 + i] >> (lane & 15) & 1)))
-                put(T, pm, c + roff[row], st[i * 17 + (lane & 15)]);
+              if (row < nx && col < ny) put(T, pm, c + roff[row], st[i * 17 + (lane & 15)]);
             }
           }
         }
         if (!MULTI) fence_before();
       }
-      // The outputs listed, or all of a tile with a row that is not finite, as
-      // plain FP64 sums.  At TN = 64 some hundred a tile are common (operator sums,
-      // 12 % of the outputs at M1 = 1500): staged (30000 clocks for 1330 outputs of
-      // K = 48, 110000 read directly).  At TN = 32 they are few (56 of 4096 in 4 % of
-      // the tiles of the energies) and the call would cost the loops before it
-      // registers: eight lanes an output read it directly (12000 clocks for 56,
-      // 24000 staged).
-      const int nsum = plain ? nx * ny : (abort ? 0 : *nagain);
+      // The listed outputs, or all of a block with a row that is not finite, as plain
+      // sums: eight lanes an output, each every eighth K value.
       if (nsum > 0) {
-        __syncthreads();   // the list, and the turned pieces are read
-        if constexpr (TN == 64) {
-          sum_again<TN>(slots[cur], plain ? nullptr : list, nsum, smem, tab, coff, roff, kb, len, pm);
-        } else {
-          const double* X = T.x + (long long)slots[cur].b * T.xub;
-          const double* Y = T.y + (long long)slots[cur].b * T.yub;
-          for (int e0 = warp * 4; e0 < nsum; e0 += THREADS / 8) {
-            const int e = min(e0 + (lane >> 3), nsum - 1);
-            const int i = plain ? e / ny : list[e] >> 6, j = plain ? e - i * ny : list[e] & 63;
-            const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
-            const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
-            double s = 0.0;
+        __syncthreads();   // the list
+        const int sm = plain ? pm : sum_mode(T);
+        const double* X = T.x + (long long)slots[cur].b * T.xub;
+        const double* Y = T.y + (long long)slots[cur].b * T.yub;
+        for (int e0 = warp * 4; e0 < nsum; e0 += THREADS / 8) {
+          const int e = min(e0 + (lane >> 3), nsum - 1);
+          const int i = plain ? e / ny : list[e] >> 6, j = plain ? e - i * ny : list[e] & 63;
+          const double* px = X + row_off(x0 + i, T.nx, T.xrs, T.xbs);
+          const double* py = Y + row_off(y0 + j, T.ny, T.yrs, T.ybs);
+          double s = 0.0;
 #pragma unroll 4
-            for (int k = lane & 7; k < len; k += 8) {
-              const int col = T.kr ? tab[k] : kb + k;
-              s = fma(__ldg(px + (long long)col * T.xks), __ldg(py + (long long)col * T.yks), s);
-            }
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if ((lane & 7) == 0 && e0 + (lane >> 3) < nsum) put(T, pm, C + roff[i] + coff[j], s);
+          for (int k = lane & 7; k < len; k += 8) {
+            const int col = T.kr ? tab[k] : kb + k;
+            s = fma(__ldg(px + (long long)col * T.xks), __ldg(py + (long long)col * T.yks), s);
           }
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          if ((lane & 7) == 0 && e0 + (lane >> 3) < nsum) put(T, sm, C + roff[i] + coff[j], s);
         }
       }
       if (warp == 1 && next && !fetched && kb + KB >= k1) {
@@ -792,6 +748,156 @@ __global__ void __launch_bounds__(F64Cfg<TN>::THREADS, F64Cfg<TN>::CTAS)
   fence_after();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(8 * TN) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Outputs that the digit products leave in doubt, summed in FP64 and added: a record
+// is a tile and a bit per output and block.  A kernel of its own: inlined or called,
+// this code made the tensor-core kernel's loops spill (phase 2 of the M1 = 500 sigma
+// 3.0 -> 4.4 ms without one output in doubt), and several CTAs an SM hide one
+// another's loads.  Bound by the FP64 pipe (two multiply-adds a clock and SM) where
+// most of a tile is in doubt, and by its loads otherwise.  The rows that hold such
+// outputs are staged 32 values at a time; many are sparse (5 of 48 terms in the
+// operator sums at M1 = 1500), so their terms are found from bit masks of the
+// non-zero values.  Against sums in the tensor-core kernel that read their operands
+// directly: 28.6 -> 24.0 s for the window above, 6.0 -> 4.6 s for the energies.
+// ---------------------------------------------------------------------------
+template <int TN> struct AgainCfg {
+  static constexpr int THREADS = 256, LD = KS + 1, CTAS = TN == 64 ? 3 : 4, ENTRIES = TM * TN / 16;
+  static constexpr int SMEM =
+      (TM + TN) * (LD * 8 + 2 * 8) + TM * TN * 2 + 2 * (TM + TN) * 4 + KS * 4 + 64 + (int)sizeof(F64Slot);
+};
+template <int TN>
+__global__ void __launch_bounds__(AgainCfg<TN>::THREADS, AgainCfg<TN>::CTAS)
+    gemm_f64_again_kernel(const F64Task* __restrict__ tasks, int ntasks, F64Doubt w, int* next_count) {
+  using A = AgainCfg<TN>;
+  constexpr int THREADS = A::THREADS, LD = A::LD, U = 4;
+  extern __shared__ uint8_t smem_raw[];
+  double* xs = (double*)smem_raw;                       // [row][k]
+  double* ys = xs + TM * LD;
+  long long* xo = (long long*)(ys + TN * LD);           // operand and output offsets of the rows
+  long long* yo = xo + TM;
+  long long* roff = yo + TN;
+  long long* coff = roff + TM;
+  F64Slot* slot = (F64Slot*)(coff + TN);
+  uint32_t* masks = (uint32_t*)(slot + 1);              // two sets, of this step's values and the next one's
+  uint32_t* need = masks + 2 * (TM + TN);               // rows of X, then of Y, that hold outputs of the list
+  int* kcol = (int*)(need + 8);
+  int* count = kcol + KS;
+  uint16_t* list = (uint16_t*)(count + 2);              // row << 6 | column
+  const int tid = threadIdx.x;
+  if (blockIdx.x == 0 && tid == 0) *next_count = 0;     // of the launch after this one
+  const int nrec = min(*w.count, w.cap);
+  for (int r = blockIdx.x; r < nrec; r += gridDim.x) {
+    __syncthreads();
+    if (tid < 32) fetch_slot(slot, tasks, ntasks, w.rec[r], 0);
+    if (tid < 2 * (TM + TN)) masks[tid] = 0;
+    if (TM + TN > THREADS / 2 && tid + THREADS < 2 * (TM + TN)) masks[tid + THREADS] = 0;
+    __syncthreads();
+    const F64Task& T = slot->t;
+    const int x0 = slot->ix * TM, y0 = slot->iy * TN;
+    const int nx = min(TM, T.mx - x0), ny = min(TN, T.my - y0);
+    const int k0 = slot->ks * T.kchunk, k1 = min(T.k, k0 + T.kchunk);
+    if (tid < nx) {
+      xo[tid] = row_off(x0 + tid, T.nx, T.xrs, T.xbs);
+      roff[tid] = row_off(x0 + tid, T.nx, T.cxs, T.cxb);
+    }
+    if (tid >= THREADS - ny) {
+      const int c = tid - (THREADS - ny);
+      yo[c] = row_off(y0 + c, T.ny, T.yrs, T.ybs);
+      coff[c] = row_off(y0 + c, T.ny, T.cys, T.cyb);
+    }
+    const double* X = T.x + (long long)slot->b * T.xub;
+    const double* Y = T.y + (long long)slot->b * T.yub;
+    double* C = T.c + (long long)slot->b * T.cub + (long long)slot->ks * T.sK;
+    const bool xk = T.xks == 1, yk = T.yks == 1;
+    const int mode = sum_mode(T);
+    uint32_t set = 0;
+    for (int blk = 0; blk < w.blocks; ++blk) {
+      const int ka = k0 + blk * KB, kz = min(k1, ka + KB);
+      __syncthreads();
+      if (tid < 8) need[tid] = 0;
+      if (tid == 8) *count = 0;
+      __syncthreads();
+      for (int e = tid; e < A::ENTRIES; e += THREADS) {
+        uint32_t bits = w.mask[((long long)r * w.blocks + blk) * A::ENTRIES + e];
+        const int row = e / (TN / 16), c0 = e % (TN / 16) * 16;
+        if (!bits) continue;
+        atomicOr(&need[row >> 5], 1u << (row & 31));
+        atomicOr(&need[4 + (c0 >> 5)], bits << (c0 & 31));
+        int at = atomicAdd(count, __popc(bits));
+        for (; bits; bits &= bits - 1) list[at++] = (uint16_t)(row << 6 | (c0 + __ffs(bits) - 1));
+      }
+      __syncthreads();
+      const int n = *count;
+      for (int base = 0; base < n; base += U * THREADS) {
+        int at[U];
+        double acc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = base + u * THREADS + tid;
+          at[u] = e < n ? list[e] : -1;
+          acc[u] = 0.0;
+        }
+        for (int kk = ka; kk < kz; kk += KS, set ^= 1u) {
+          const int nk = min(KS, kz - kk);
+          uint32_t* mx = masks + set * (TM + TN);
+          uint32_t* my = mx + TM;
+          if (tid < nk) kcol[tid] = k_col(T, kk + tid);
+          __syncthreads();
+          // rows in need of it; values of other rows are not read
+          auto stage = [&](auto cols, const double* P, const long long* off, const uint32_t* nd, int nr, bool alongk,
+                           long long ks, double* dst, uint32_t* mk) {
+            constexpr int R = decltype(cols)::value, N = R * KS / THREADS;
+#pragma unroll 1
+            for (int i0 = 0; i0 < N; i0 += 8 < N ? 8 : N) {
+              constexpr int B = 8 < N ? 8 : N;
+              double v[B];
+#pragma unroll
+              for (int i = 0; i < B; ++i) {
+                const int e = tid + (i0 + i) * THREADS, rr = alongk ? e / KS : e % R, q = alongk ? e % KS : e / R;
+                const bool on = rr < nr && q < nk && (nd[rr >> 5] >> (rr & 31) & 1u);
+                v[i] = on ? __ldg(P + off[rr] + (long long)kcol[q] * ks) : 0.0;
+              }
+#pragma unroll
+              for (int i = 0; i < B; ++i) {
+                const int e = tid + (i0 + i) * THREADS, rr = alongk ? e / KS : e % R, q = alongk ? e % KS : e / R;
+                dst[rr * LD + q] = v[i];
+                if (v[i] != 0.0) atomicOr(&mk[rr], 1u << q);
+              }
+            }
+          };
+          stage(std::integral_constant<int, TM>(), X, xo, need, nx, xk, T.xks, xs, mx);
+          stage(std::integral_constant<int, TN>(), Y, yo, need + 4, ny, yk, T.yks, ys, my);
+          __syncthreads();
+          if (tid < TM + TN) masks[(set ^ 1u) * (TM + TN) + tid] = 0;
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            if (at[u] < 0) continue;
+            const int i = at[u] >> 6, j = at[u] & 63;
+            const double* px = xs + i * LD;
+            const double* py = ys + j * LD;
+            double a = acc[u];
+            const uint32_t m0 = mx[i] & my[j];
+            if (__popc(m0) > nk / 2) {
+#pragma unroll 4
+              for (int q = 0; q < nk; ++q) a = fma(px[q], py[q], a);
+            } else {
+              for (uint32_t m = m0; m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                a = fma(px[q], py[q], a);
+              }
+            }
+            acc[u] = a;
+          }
+          __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (at[u] >= 0) put(T, mode, C + roff[at[u] >> 6] + coff[at[u] & 63], acc[u]);
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1093,6 +1199,7 @@ void plan_f64(const GemmTask* g, int n, F64Plan& p) {
     F64Task t = make_task(g[i], o[i].d, pipe ? o[i].pipe : o[i].tc[w]);
     t.tile0 = p.tiles[list];
     p.tiles[list] += (long long)t.batch * t.ksplit * t.tx * t.ty;
+    if (list == F64_LONG) p.blocks = std::max(p.blocks, (int)cdiv(std::min(t.k, t.kchunk), KB));
     p.t[list].push_back(t);
   }
   for (int l = 0; l < F64_LISTS; ++l) p.n[l] = (int)p.t[l].size();
@@ -1114,8 +1221,8 @@ void upload_f64(const F64Plan& p, void* d, cudaStream_t s) {
 }
 
 template <int TN, bool MULTI>
-static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, int sms, int* err, cudaStream_t s,
-                          unsigned long long wait_ns) {
+static int launch_f64_tc(const F64Task* d, int n, long long tiles, int device, int sms, int* err, cudaStream_t s,
+                         unsigned long long wait_ns, F64Scratch* scratch, int nblocks = 1) {
   using F = F64Cfg<TN>;
   static std::atomic<bool> attr[MAX_DEV];
   MPSLCC_REQUIRE(device >= 0 && device < MAX_DEV, ST_ARG, "device ordinal out of range");
@@ -1123,14 +1230,53 @@ static void launch_f64_tc(const F64Task* d, int n, long long tiles, int device, 
     cuda_check(cudaFuncSetAttribute(gemm_f64_tc_kernel<TN, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     f64_smem<F, MULTI>()),
                "smem attr");
+    cuda_check(cudaFuncSetAttribute(gemm_f64_again_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    AgainCfg<TN>::SMEM),
+               "smem attr");
     attr[device].store(true, std::memory_order_release);
   }
-  const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, sms) * F::CTAS);
-  gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F, MULTI>(), s>>>(d, n, tiles, err, wait_ns);
+  // Tiles in pairs of launches that the records have room for.  Two counts take
+  // turns: the second kernel of one pair clears the next one's.
+  const int blocks = MULTI ? nblocks : 1;
+  const size_t bytes = f64_record_bytes(TN, blocks);
+  const bool room = blocks <= F64_MAX_BLOCKS && scratch && scratch->bytes >= F64_SCRATCH_HEAD + bytes;
+  F64Doubt w = {nullptr, nullptr, nullptr, 0, blocks};
+  long long step = tiles;
+  if (room) {
+    const long long most = f64_launch_tiles(TN, blocks);
+    w.cap = (int)std::min((long long)((scratch->bytes - F64_SCRATCH_HEAD) / bytes), most);
+    w.rec = (long long*)((char*)scratch->p + F64_SCRATCH_HEAD);
+    w.mask = (uint16_t*)(w.rec + w.cap);
+    if (w.cap == most) step = most;
+  }
+  int launches = 0;
+  for (long long t0 = 0; t0 < tiles; t0 += step) {
+    const long long t1 = std::min(tiles, t0 + step);
+    int* counts = room ? (int*)scratch->p : nullptr;
+    if (room) w.count = counts + (scratch->turn++ & 1);
+    const int grid = (int)std::min<long long>(t1 - t0, (long long)std::max(1, sms) * F::CTAS);
+    gemm_f64_tc_kernel<TN, MULTI><<<grid, F::THREADS, f64_smem<F, MULTI>(), s>>>(d, n, t0, t1, err, wait_ns, w);
+    ++launches;
+    if (!room) continue;
+    const int g2 = (int)std::min<long long>(t1 - t0, (long long)std::max(1, sms) * AgainCfg<TN>::CTAS);
+    gemm_f64_again_kernel<TN>
+        <<<g2, AgainCfg<TN>::THREADS, AgainCfg<TN>::SMEM, s>>>(d, n, w, counts + (scratch->turn & 1));
+    ++launches;
+  }
+  return launches;
+}
+
+size_t f64_scratch_bytes(const F64Launch& l) {
+  const auto need = [](long long tiles, int tn, int blocks) {
+    if (blocks > F64_MAX_BLOCKS) return (size_t)0;
+    return (size_t)std::min(tiles, f64_launch_tiles(tn, blocks)) * f64_record_bytes(tn, blocks);
+  };
+  const size_t n = std::max(need(l.tiles[F64_SHORT], l.tn, 1), need(l.tiles[F64_LONG], 32, l.blocks));
+  return n ? F64_SCRATCH_HEAD + n : 0;
 }
 
 int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s,
-               unsigned long long wait_ns) {
+               unsigned long long wait_ns, F64Scratch* scratch) {
   int launches = 0;
   const F64Task* t = (const F64Task*)d;
   for (int i = 0; i < F64_LISTS; ++i) {
@@ -1138,13 +1284,17 @@ int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err,
     const long long tiles = l.tiles[i];
     MPSLCC_REQUIRE((tiles > 0) == (n > 0), ST_INTERNAL, "FP64 task list without its counts");
     if (n == 0) continue;
-    if (i == F64_PIPE)
+    if (i == F64_PIPE) {
       gemm_f64_pipe_kernel<<<(int)std::min<long long>(tiles, 152LL * 8), 256, 0, s>>>(t, n, tiles);
-    else if (i == F64_SHORT && l.tn == 32) launch_f64_tc<32, false>(t, n, tiles, device, sms, err, s, wait_ns);
-    else if (i == F64_SHORT) launch_f64_tc<64, false>(t, n, tiles, device, sms, err, s, wait_ns);
-    else launch_f64_tc<32, true>(t, n, tiles, device, sms, err, s, wait_ns);
+      ++launches;
+    } else if (i == F64_SHORT && l.tn == 32) {
+      launches += launch_f64_tc<32, false>(t, n, tiles, device, sms, err, s, wait_ns, scratch);
+    } else if (i == F64_SHORT) {
+      launches += launch_f64_tc<64, false>(t, n, tiles, device, sms, err, s, wait_ns, scratch);
+    } else {
+      launches += launch_f64_tc<32, true>(t, n, tiles, device, sms, err, s, wait_ns, scratch, l.blocks);
+    }
     t += n;
-    ++launches;
   }
   return launches;
 }

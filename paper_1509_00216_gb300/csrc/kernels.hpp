@@ -69,6 +69,7 @@ struct F64Launch {
   int n[F64_LISTS] = {0, 0, 0};
   long long tiles[F64_LISTS] = {0, 0, 0};
   int tn = 64;               // columns of a short sum's tile: 64 or 32 (long sums: 32)
+  int blocks = 1;            // scaling blocks of the longest sum
 };
 struct F64Plan : F64Launch {
   std::vector<F64Task> t[F64_LISTS];
@@ -78,11 +79,20 @@ bool f64_on_pipe(const GemmTask* g, int n);
 void plan_f64(const GemmTask* g, int n, F64Plan& p);
 size_t f64_plan_bytes(const F64Plan& p);
 void upload_f64(const F64Plan& p, void* d, cudaStream_t s);
+// Device memory that the tensor-core products of one stream share for the outputs
+// they leave in doubt: its first 256 bytes are zero before the first of them.
+// Without it (or beyond its room) such outputs are summed where they are found.
+struct F64Scratch {
+  void* p;
+  size_t bytes;
+  unsigned turn;   // launches so far
+};
+size_t f64_scratch_bytes(const F64Launch& l);
 // Runs the lists uploaded at d; returns the number of launches.  The
 // tensor-core kernel takes at most `sms` SMs and records a wait of more than
 // wait_ns in *err.
 int launch_f64(const F64Launch& l, const void* d, int device, int sms, int* err, cudaStream_t s,
-               unsigned long long wait_ns = 2000000000ull);
+               unsigned long long wait_ns = 2000000000ull, F64Scratch* scratch = nullptr);
 
 // Fill tile bookkeeping; returns total number of tiles.
 long long plan_copy_tiles(CopyTask* t, int n);
