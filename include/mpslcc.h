@@ -372,11 +372,12 @@ mpslcc_status mpslcc_debug_tc_gemm(mpslcc_ctx* ctx, int prec, int m, int n, int 
    - d_A (m x k), d_B (n x k), d_C (m x n): row-major FP64 DEVICE arrays owned
      by the caller; prec is TF32, BF16 or BF16X3; work runs on `stream` (NULL =
      legacy default stream) of `device`, which must be the current device.
-   - The call allocates nothing and needs no context: its operand copies, FP32
-     result, task descriptors and error flag live in one file-scope device
-     array of mpslcc_tc_gemm_noalloc_scratch_bytes() bytes (64 MiB), reserved
-     on every GPU that loads the library until the process exits.  Problems
-     whose scratch would exceed it return MPSLCC_E_ARG.
+   - The call allocates nothing and needs no context: its operand copies, task
+     descriptors and error flag live in one file-scope device array of
+     mpslcc_tc_gemm_noalloc_scratch_bytes() bytes (64 MiB), reserved on every
+     GPU that loads the library until the process exits.  Problems whose
+     scratch, with 4 bytes per element of C, would exceed it return
+     MPSLCC_E_ARG.
    - The first call on a device looks up the array's device address (set-up);
      make that first call before any stream capture.
    - Every call reuses the same array and overwrites what it needs (padding

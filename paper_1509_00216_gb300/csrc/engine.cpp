@@ -952,7 +952,7 @@ void build_fused_ahead(Ctx& c, Family& F, int l, bool right_side, FusedAhead& A)
   A.right = right_side;
 }
 
-static void finish_sigma_plan(Ctx& c, SigmaPlan& P);
+static void finish_sigma_plan(SigmaPlan& P);
 
 void make_sigma_plan(Ctx& c, Family& F, int l, SigmaPlan& P, FusedAhead* ahead) {
   ensure_envs(c, F, l);
@@ -977,7 +977,7 @@ void make_sigma_plan(Ctx& c, Family& F, int l, SigmaPlan& P, FusedAhead* ahead) 
     make_right_fused(c, F, l + 1, P.mid_b, P.mid_k, P.rf);
   }
   if (ahead) ahead->l = -1;
-  finish_sigma_plan(c, P);
+  finish_sigma_plan(P);
 }
 
 void make_sigma_plan1(Ctx& c, Family& F, int l, SigmaPlan& P) {
@@ -992,11 +992,11 @@ void make_sigma_plan1(Ctx& c, Family& F, int l, SigmaPlan& P) {
     make_left_fused(c, F, l, P.mid_b, P.mid_k, P.lf);
   }
   make_right_env(c, F, l, P.mid_b, P.mid_k, P.rf);
-  finish_sigma_plan(c, P);
+  finish_sigma_plan(P);
 }
 
 // Flops of a plan whose fused left operator and right operator are in place.
-static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
+static void finish_sigma_plan(SigmaPlan& P) {
   const LeftFused& lf = P.lf;
   const RightFused& rf = P.rf;
   P.f64_ready = false;
@@ -1035,7 +1035,6 @@ static void finish_sigma_plan(Ctx& c, SigmaPlan& P) {
       fl += dr * class_flops(mL, W.bond[lf.p + 1].class_start[sg.cls], sg.nw, lf.FLb, lf.kb[bi], lf.FLk, lf.kk[sg.kidx]);
   }
   P.flops = fl;
-  (void)c;
 }
 
 // Intermediate buffers and the task lists of both FP64 sigma phases, built

@@ -38,6 +38,7 @@ struct RunBuilder {   // the ranges one by one, in ascending order
   }
 };
 
+// The ranges in any order (the products add theirs in ascending order).
 inline std::vector<KRun> merge_runs(std::vector<std::pair<long, long>>& r, int KT) {
   std::sort(r.begin(), r.end());
   RunBuilder out(KT);

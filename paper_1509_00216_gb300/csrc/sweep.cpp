@@ -117,8 +117,9 @@ void jacobi_eigh(int n, std::vector<double>& A, std::vector<double>& w, std::vec
   for (int i = 0; i < n; ++i) w[i] = A[i * n + i];
 }
 
-// Its time is read when the next one begins or the statistics are asked for:
-// the dots that follow a product wait for it anyway.
+// The events around it are read when the next one begins or the statistics are
+// asked for.  (The product itself waits for its phases: it reads their times, and
+// whether they gave up.)
 void sigma_timed(Ctx& c, SigmaPlan& P, const double* x, double* y, int prec) {
   settle_sigma(c);
   cudaEventRecord(c.ev0, c.s());

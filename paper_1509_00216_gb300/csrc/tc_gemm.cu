@@ -1618,7 +1618,7 @@ constexpr int TC_CAPS[NSHAPE] = {256, 128, 64, 64};
 constexpr int TC_CFG[NSHAPE] = {0, 0, 0, 1};
 inline int list_of(int shape) { return shape < 3 ? shape : 2; }
 
-// K runs of a task: merge_runs (kruns.hpp).
+// K runs of a task: RunBuilder (kruns.hpp).
 // Appends a task's run table (pairs {kx, steps before}, a sentinel, then the
 // run of each K split's first step) to `tab`; returns its offset.
 long append_runs(std::vector<int>& tab, const std::vector<KRun>& runs, int kchunk, int ksplit) {
